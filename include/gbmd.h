@@ -241,14 +241,10 @@ typedef struct {
                                 capped at residency.  The rebuild kernels (binning, scatter,
                                 reorder, neighbour build) always run at their full residency */
     int32_t nbr_batch;       /* W entries each thread loads together in the pair loop: 2, 4 or 8 */
-    int32_t build_batch;     /* neighbour build: 2 or 4 = one thread per atom loading that many
-                                candidates together; 32 = one warp per cell, each row of
-                                candidates staged once in shared memory (for cells of tens of
-                                atoms); 1 = one thread per atom over half-side sub-cells, the
-                                atoms counting-sorted by sub-cell and only the sub-cells within
-                                reach scanned (about half the candidates).  The neighbour sets
-                                are the same for every choice; the order within a column of W
-                                (and so the summation order of a force) follows the choice */
+    int32_t build_batch;     /* neighbour build: 1, 2, 4 or 32 are accepted and select the same
+                                kernel (units of 10 atoms per warp, a lane per atom and z plane of
+                                cells); the columns of W are in the order rows of cells, cells,
+                                slots */
     int32_t use_graph;       /* 1: md_integrate replays captured CUDA graphs; 2: direct launches */
     int32_t step_kernel;     /* fused step kernel (MD_MIXED, MD_FP32): 1 = each thread loads its
                                 atom's state and W column; warps take 32-atom warp-tiles from
@@ -274,10 +270,8 @@ typedef struct {
                                 step kernel then reads and clears the buffers.  The atomics add
                                 in no fixed order, so repeat runs differ in the last bits;
                                 md_get_neighbours reports the half sets; md_adjoint refuses it */
-    int32_t build_stage;     /* neighbour build (build_batch 1, 2, 4): 1 = each thread appends its
-                                column of W in shared memory and the warps write whole rows (128
-                                contiguous bytes per row for 32 atoms; for matrices far larger
-                                than L2), 2 = each entry written to W as found */
+    int32_t build_stage;     /* 1 or 2 are accepted: the build always collects its columns in
+                                shared memory and writes whole rows of W */
     int32_t reorder_every;   /* the reorder of atoms by cell (Sec. 4.1 item 1): at the first rebuild
                                 at least this many steps after the last reorder, or -1 = at
                                 every rebuild; starts as md_params.reorder_every (0 there reads

@@ -39,6 +39,8 @@ struct Plan {
     int32_t nchunks = 0;
     int32_t cap = 0;
     int32_t series_cap = 0;
+    int64_t nrows = 0;            // rows of cells of all replicas
+    double mean_nbrs = 0.0;       // neighbours within r_c + skin at the largest mean density
     int64_t n_total = 0;
     int mode = MD_MIXED;
     int rule = MD_REBUILD_VMAX;
@@ -80,6 +82,18 @@ int pow2_floor(int v)
     return k;
 }
 
+// How far the build's |r|^2 - r_l^2 (differences of FP32 positions in the replica's frame) may lie
+// from the criterion's, as a bound twice as wide as the rounding allows: with u the ulp of a
+// frame coordinate, each axis of a displacement is off by at most 1.75 u, so |r|^2 near r_l^2 by
+// 2 sqrt(3) r_l 1.75 u < 6.1 r_l u, plus a few roundings of r_l^2 itself.
+float build_band(const Rep& R, double rl)
+{
+    double top = 0.0;
+    for (int a = 0; a < 3; ++a) top = std::max(top, R.L[a] + R.w[a]);
+    const double u = std::ldexp(1.0, std::ilogb(top) - 23);
+    return float(12.0 * rl * u + 16.0 * std::ldexp(1.0, -23) * rl * rl);
+}
+
 int make_plan(const md_params* p, int32_t nrep, const int64_t* n_rep, const double* box_rep, Plan* P)
 {
     int rc = check_params(p);
@@ -90,7 +104,7 @@ int make_plan(const md_params* p, int32_t nrep, const int64_t* n_rep, const doub
     P->mode = p->precision;
     P->rule = p->rebuild_rule;
     P->reps.resize(nrep);
-    int64_t slot = 0, cells = 0, ids = 0;
+    int64_t slot = 0, cells = 0, ids = 0, rows = 0;
     double rho_max = 0.0;
     for (int32_t r = 0; r < nrep; ++r) {
         Rep& R = P->reps[r];
@@ -121,6 +135,9 @@ int make_plan(const md_params* p, int32_t nrep, const int64_t* n_rep, const doub
         R.cell0 = int32_t(cells);
         R.ncells = int32_t(nc_tot);
         R.id0 = int32_t(ids);
+        R.row0 = int32_t(rows);
+        R.band = build_band(R, rl);
+        rows += int64_t(R.nc[1]) * R.nc[2];
         slot += int64_t(R.ntiles) * TILE;
         cells += nc_tot;
         ids += n_rep[r];
@@ -133,6 +150,8 @@ int make_plan(const md_params* p, int32_t nrep, const int64_t* n_rep, const doub
     P->ncells = int32_t(cells);
     P->nchunks = int32_t((cells + SCAN_CHUNK - 1) / SCAN_CHUNK);
     P->n_total = ids;
+    P->nrows = rows;
+    P->mean_nbrs = 4.0 / 3.0 * M_PI * rl * rl * rl * rho_max;
     P->tile_rep.resize(P->ntiles);
     for (int32_t r = 0; r < nrep; ++r)
         for (int32_t k = 0; k < P->reps[r].ntiles; ++k) P->tile_rep[P->reps[r].tile0 + k] = r;
@@ -142,8 +161,7 @@ int make_plan(const md_params* p, int32_t nrep, const int64_t* n_rep, const doub
     if (p->nbr_capacity > 0) {
         P->cap = p->nbr_capacity;
     } else {
-        const double mean = 4.0 / 3.0 * M_PI * rl * rl * rl * rho_max;
-        P->cap = std::max(8, int(std::ceil(1.5 * mean + 16.0)));
+        P->cap = std::max(8, int(std::ceil(1.5 * P->mean_nbrs + 16.0)));
         P->cap = (P->cap + 3) & ~3;
     }
     if (P->cap > 4096) return fail(MD_ERR_INVALID_ARG, "nbr_capacity above 4096");
@@ -186,18 +204,12 @@ size_t carve(const Plan& P, char* base, Arrays* A)
     a.W = c.take<uint32_t>(ns * size_t(P.cap));
     if (P.rule == MD_REBUILD_DISP) a.xref = c.take<float4>(ns);
     a.perm = c.take<int32_t>(ns);
-    if (!f64) a.psort = c.take<float4>(ns + PSORT_PAD);       // readable past the last atom
+    a.psort = c.take<float4>(ns + 4 * size_t(P.nrows) + CAND_PAD);
+    a.pcell = c.take<uint32_t>(ns);
     if (!f64) a.tile_win = c.take<int2>(size_t(P.ntiles) * 9);
     if (!f64) {
         a.fbuf = c.take<float4>(ns);
         a.wbuf = c.take<float>(ns);
-    }
-    if (!f64) {
-        const size_t nsub = size_t(8) * size_t(P.ncells);
-        a.psub = c.take<float4>(ns);
-        a.scount = c.take<int32_t>(nsub);
-        a.sstart = c.take<int32_t>(nsub + 1);
-        a.schunk = c.take<int32_t>((nsub + SCAN_CHUNK - 1) / SCAN_CHUNK);
     }
     if (!f32) for (int q = 0; q < 3; ++q) a.tmp_d[q] = c.take<double>(ns);
     for (int q = 0; q < 3; ++q) a.tmp_v[q] = c.take<double>(ns);
@@ -383,8 +395,6 @@ void fill_scal(md_system* s)
     S.reorder_every = p.reorder_every;
     S.series_cap = P.series_cap;
     S.shift = p.shift_energy;
-    S.nsub = int64_t(8) * P.ncells;
-    S.nschunks = int32_t((S.nsub + SCAN_CHUNK - 1) / SCAN_CHUNK);
     S.props_split = props_split(P);
     S.dt = p.dt;
     S.mass = p.mass;
@@ -439,8 +449,6 @@ int apply_tuning(md_system* s)
     s->L.step_block = TILE;
     s->L.build_block = TILE;
     s->L.nbr_batch = s->tune.nbr_batch;
-    s->L.build_batch = s->tune.build_batch;
-    s->L.build_stage = s->tune.build_stage == 1 ? 1 : 0;
     s->L.step_kernel = (s->S.mode == MD_FP64) ? 1 : s->tune.step_kernel;
     // the list-free kernel reads each row of cells as a run of slots: atoms reorder at every rebuild
     // tune.reorder_every: -1 = at every rebuild, else every that many steps
@@ -448,6 +456,7 @@ int apply_tuning(md_system* s)
     s->S.half_list = (s->L.step_kernel == 5) ? 1 : 0;      // W keeps each pair once
     bulk_shape(s->S, per_sm, s->smem_per_sm, s->smem_per_cta, &s->L.bulk_rows, &s->L.bulk_smem);
     stage_shape(per_sm, s->smem_per_sm, &s->L.stage_cap, &s->L.stage_smem);
+    build_group_shape(s->S, s->L, s->plan.mean_nbrs, s->smem_per_cta, s->smem_per_sm);
     s->L.ctas_req = per_sm;
     // a persistent grid larger than what can be resident would run as a trailing second wave
     s->L.grid_step = s->nsm * std::min(per_sm, step_ctas_per_sm(s->S, s->L));
@@ -801,11 +810,11 @@ int md_integrate(md_system* s, int32_t nsteps)
         }
         s->cur ^= 1;
         {
-            Phase t(s, MD_PHASE_BIN, 7);
+            Phase t(s, MD_PHASE_BIN, bin_kernels(s->S, s->L));
             GBMD_CUDA(launch_bin_order(s->A, s->S, s->L, s->cur, false));
         }
         {
-            Phase t(s, MD_PHASE_REORDER, 2);
+            Phase t(s, MD_PHASE_REORDER, REORDER_KERNELS);
             GBMD_CUDA(launch_reorder(s->A, s->S, s->L, s->cur));
         }
         {
@@ -832,7 +841,8 @@ int md_get_timing(md_system* s, double* ms, int64_t* calls, int64_t* launches)
         // rebuild sequences inside graphs ran only when their IF node opened: count them here
         long long gr = 0;
         GBMD_CUDA(cudaMemcpy(&gr, &s->A.g->graph_rebuilds, sizeof(gr), cudaMemcpyDeviceToHost));
-        s->launches[MD_PHASE_BUILD] += (REBUILD_KERNELS - 3 + build_kernels(s->S, s->L)) * (gr - s->graph_rebuilds_seen);
+        s->launches[MD_PHASE_BUILD] += (bin_kernels(s->S, s->L) + REORDER_KERNELS + build_kernels(s->S, s->L)) *
+                                       (gr - s->graph_rebuilds_seen);
         s->graph_rebuilds_seen = gr;
     }
     for (auto& pr : s->pending) {

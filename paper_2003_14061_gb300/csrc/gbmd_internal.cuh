@@ -36,8 +36,15 @@ constexpr int SCAN_CHUNK = 2048;          // cells per block of the prefix sum
 constexpr int PROPS_SPLIT_MAX = 2048;     // CTAs per replica in the first level of the final sums
 constexpr int ADJ_VPART = 128;            // blocks of the |v_S|^2 partial sums
 
-// entries of psort past the last atom, so that a build batch may read past a row's end
-constexpr int PSORT_PAD = 8;
+// Candidate array of the neighbour build (psort): the atoms in cell order, their positions in the
+// replica's frame (cell origin + cell-local position, FP32).  Two consecutive entries share 32
+// bytes, x0 x1 y0 y1 | z0 z1 e0 e1, the operands of packed FP32x2 operations; e = slot << IDX_SHIFT
+// | (c_x mod 4).  Every row of cells starts at a multiple of 4 entries and is followed up to the
+// next one by entries far outside the box, so whole groups of 4 can be tested without bounds.
+// Row q (counted over all replicas) whose first atom is number rs of the cell order starts at
+// entry cand_place = ceil4(rs) + 4 q: at most 4 entries of padding per row.
+constexpr float CAND_FAR = 1.0e15f;
+constexpr int CAND_PAD = 16;                 // readable entries past the last one
 
 enum ErrBits { ERR_NBR_OVERFLOW = 1, ERR_NONFINITE = 2, ERR_TIMEOUT = 4 };
 
@@ -59,7 +66,8 @@ struct Rep {                  // per replica, fixed after creation
     float wlo[3];             // (float) (w - wf): the FP32 pair displacement adds o wf, then o wlo,
                               // so that the rounding of w does not bias every cross-cell distance
                               // of an axis the same way
-    float pad2[2];
+    int32_t row0;             // rows of cells of the replicas before this one
+    float band;               // |r^2 - (r_c + skin)^2| below which the build applies its criterion exactly
 };
 
 struct RepState {             // per replica, mutable on the device
@@ -110,13 +118,10 @@ struct Arrays {
     uint32_t* W;
     float4* xref;             // positions at the last rebuild (rule DISP)
     int32_t* perm;            // cell-ordered slots (the matrix H of Sec. 2.3, flattened)
-    float4* psort;            // FP32 positions in cell order, slot in .w (MD_MIXED, MD_FP32)
+    float4* psort;            // candidate array of the neighbour build (cand_place, cand_store)
+    uint32_t* pcell;          // packed cell of every atom in cell order
     float4* fbuf;             // step kernel 5: FP32 force and u_i accumulated over the half list
     float* wbuf;              //   and the per-atom virial (zero between steps)
-    float4* psub;             // FP32 positions sorted by half-side sub-cell, slot in .w (sub-cell build)
-    int32_t* scount;          // per sub-cell (8 per cell): occupancy, then zero again after the scan
-    int32_t* sstart;          // per sub-cell + 1: start in psub
-    int32_t* schunk;          // per SCAN_CHUNK sub-cells
     int2* tile_win;           // [ntiles][9] slot window (lo, hi) of each tile's W entries per
                               // (o_y, o_z) row, periodic-wrap entries excluded (MD_MIXED, MD_FP32)
     // reorder scratch, per slot
@@ -166,8 +171,6 @@ struct Scal {
     int32_t half_list;        // 1: W keeps each pair once, at the lower slot (step kernel 5)
     int32_t chain_len;        // polymer chains (md_set_chains): atoms per chain, 0 = none
     float ch_kb, ch_r0sq, ch_ka, ch_kd;   // FENE stiffness, R0^2, bend and dihedral constants
-    int64_t nsub;             // half-side sub-cells (8 per cell) of the sub-cell build
-    int32_t nschunks;
     double dt, mass, c;       // c = dt / (2 m)
     double half_skin;
     double disp_margin;       // rounding margin of a displacement measured on FP32 positions
@@ -241,6 +244,21 @@ __host__ __device__ __forceinline__ int row_pos(const Rep& R, int ny, int nz)
 __host__ __device__ __forceinline__ int cell_index(const Rep& R, int cx, int cy, int cz)
 {
     return R.cell0 + row_pos(R, cy, cz) * R.nc[0] + cx;
+}
+
+// first entry of a row of cells in the candidate array; prow = row_pos, rs = cstart of its first cell
+__host__ __device__ __forceinline__ int cand_place(const Rep& R, int prow, int rs)
+{
+    return ((rs + 3) & ~3) + 4 * (R.row0 + prow);
+}
+
+__device__ __forceinline__ void cand_store(float4* psort, int P, float x, float y, float z, uint32_t e)
+{
+    float* f = reinterpret_cast<float*>(psort) + int64_t(8) * (P >> 1) + (P & 1);
+    f[0] = x;
+    f[2] = y;
+    f[4] = z;
+    f[6] = __uint_as_float(e);
 }
 
 // (cx, cy, cz) of the replica-local cell number cl
@@ -403,9 +421,11 @@ struct Launch {
     int build_block;
     int nbr_batch;            // W entries loaded together per thread in the pair loop (2, 4, 8)
     int ctas_req;             // requested resident CTAs/SM (register bound of the step kernel)
-    int build_stage;          // 1: the thread-per-atom builds stage their columns in shared memory
-    int build_batch;          // candidates loaded together per thread in the build (2, 4; 32 = warp per cell;
-                              // 1 = thread per atom over half-side sub-cells)
+    int bg_rows;              // k_build_group: rows of each lane's list in shared memory,
+    int bg_block;             // threads per CTA, dynamic shared memory and CTAs
+    int bg_smem;
+    int bg_grid;
+    int bg_minb;              // its register bound: CTAs per SM it is compiled for (8, or 5 with long lists)
     int step_kernel;          // 1: per-thread loads with L2 prefetch; 2: bulk-copy shared-memory ring;
                               // 3: as 1, with each tile's neighbour positions staged in shared memory
     int bulk_rows;            // rows of W staged per tile by the ring (step_kernel 2)
@@ -429,11 +449,14 @@ cudaError_t launch_force_rebuild(const Arrays& A, const Scal& S, const Launch& L
 void prime_rebuild_grids(const Scal& S, const Launch& L);
 cudaError_t launch_rebuild(const Arrays& A, const Scal& S, const Launch& L, int cur, bool from_set);
 cudaError_t launch_bin_only(const Arrays& A, const Scal& S, const Launch& L, int cur, bool from_set);
-cudaError_t launch_bin_order(const Arrays& A, const Scal& S, const Launch& L, int cur, bool from_set);   // 7 kernels
-cudaError_t launch_reorder(const Arrays& A, const Scal& S, const Launch& L, int cur);                    // 2 kernels
-cudaError_t launch_build_only(const Arrays& A, const Scal& S, const Launch& L, int cur);                // 3 kernels
-constexpr int REBUILD_KERNELS = 12;       // kernels of one rebuild sequence (bin/order 7, reorder 2, build 3)
-int build_kernels(const Scal& S, const Launch& L);   // kernels of launch_build_only (2, 3 or 9)
+cudaError_t launch_bin_order(const Arrays& A, const Scal& S, const Launch& L, int cur, bool from_set);
+cudaError_t launch_reorder(const Arrays& A, const Scal& S, const Launch& L, int cur);
+cudaError_t launch_build_only(const Arrays& A, const Scal& S, const Launch& L, int cur);
+int bin_kernels(const Scal& S, const Launch& L);     // kernels of launch_bin_order
+constexpr int REORDER_KERNELS = 2;                   // kernels of launch_reorder
+int build_kernels(const Scal& S, const Launch& L);   // kernels of launch_build_only
+// rows of k_build_group's lists, its CTA size, shared memory and grid, into L
+void build_group_shape(const Scal& S, Launch& L, double mean_nbrs, int smem_per_cta, int smem_per_sm);
 
 // adjoint (kernels_adjoint.cu)
 cudaError_t launch_adj_reverse(const Arrays& A, const Scal& S, const Launch& L, const AdjView& V, int q, double kappa,

@@ -6,16 +6,14 @@
 //   k_bin          N1 + N2: cell of every atom from its FP64 position, layer l_i = atomic slot
 //                  in the cell (the occupancy counter k_c); max k_c (N3) per replica.
 //   k_scan_*       prefix sum of k_c -> cstart (the row offsets of H, Sec. 2.4 item 4).
-//   k_scatter      N4: H flattened: perm[cstart[c] + l_i] = i.
-//   k_sort_cells   the atomic layer order is indeterminate (Sec. 2.3 notes the resulting
-//                  irreproducibility); sorting each cell's slots makes the order, and every
-//                  result after it, deterministic.  It also writes psort, the FP32 positions in
-//                  that order with each slot in .w, which the FP32 builds read.
+//   k_scatter      N4: H flattened, in layer order.
+//   k_order        the atomic layer order is indeterminate (Sec. 2.3 notes the resulting
+//                  irreproducibility); ranking each atom among its cell's slots makes the order,
+//                  and every result after it, deterministic.  It also writes the candidate array
+//                  psort that the build reads.
 //   k_reorder_*    Sec. 4.1 item 1: permute the atoms into cell order (gather through scratch).
-//   k_build_sorted N5 in FP32: W from the 27 neighbouring cells, one thread per atom, each row of
-//                  3 cells read as a contiguous run of psort; W stored row-major for coalescing
-//                  (Sec. 4.1 item 6).  k_build_cw: the same W with one warp per cell (cells of
-//                  tens of atoms).  k_build<double>: MD_FP64 through perm.
+//   k_build_group  N5: W from the 27 neighbouring cells, units of 10 atoms per warp and a lane per
+//                  atom and z plane; W stored row-major for coalescing (Sec. 4.1 item 6).
 //   k_tile_windows the slot window of each tile's W entries per row of neighbour cells, read by
 //                  the step kernel that stages neighbour positions (step kernel 3 only).
 // Only replicas whose rebuild flag is set do work; kernels return at once when none is set, so
@@ -368,38 +366,73 @@ __global__ void __launch_bounds__(TILE) k_scatter(Arrays A, Scal S)
         const int r = A.tile_rep[t];
         const Rep& R = A.rep[r];
         const int64_t slot = int64_t(t) * TILE + threadIdx.x;
-        if (slot - R.slot0 < R.n) A.perm[A.cstart[A.cell[slot]] + A.layer[slot]] = int32_t(slot);
+        if (slot - R.slot0 < R.n) A.tmp_i[0][A.cstart[A.cell[slot]] + A.layer[slot]] = int32_t(slot);
     }
 }
 
-__global__ void __launch_bounds__(256) k_sort_cells(Arrays A, Scal S, int cur)
+// One thread per atom: its rank among the slots of its cell (the scatter left them in atomic
+// order) is its place in the cell order, perm.  The thread also writes the atom's entry of the
+// build's candidate array at that place: position in the replica's frame, the slot it will have
+// after a reorder that is due, and the packed cell.  A thread per cell sorting its slots in
+// place was a serial chain of dependent loads (cells of 18 atoms: 428 us for 16.4M atoms, 22 us
+// for 4000); the rank takes one pass over the cell's slots, which the lanes of a cell share.
+template <int MODE>
+__global__ void __launch_bounds__(TILE) k_order(Arrays A, Scal S, int cur)
 {
     if (!A.g->any_rebuild) return;
-    for (int64_t c = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; c < S.ncells;
-         c += int64_t(gridDim.x) * blockDim.x) {
-        const int b = A.cstart[c], e = A.cstart[c + 1];
-        for (int k = b + 1; k < e; ++k) {            // insertion sort, cells hold a few atoms
-            const int32_t key = A.perm[k];
-            int q = k - 1;
-            while (q >= b && A.perm[q] > key) {
-                A.perm[q + 1] = A.perm[q];
-                --q;
-            }
-            A.perm[q + 1] = key;
+    const int nrb = A.g->n_rb_tiles;
+    const int32_t* __restrict__ unsorted = A.tmp_i[0];
+    const int32_t* __restrict__ cs = A.cstart;
+    for (int it = blockIdx.x; it < nrb; it += gridDim.x) {
+        const int t = A.rb_tiles[it];
+        const int r = A.tile_rep[t];
+        const Rep& R = A.rep[r];
+        const int64_t slot = int64_t(t) * TILE + threadIdx.x;
+        if (slot - R.slot0 >= R.n) continue;
+        const int c = A.cell[slot];
+        const int b = cs[c], e = cs[c + 1];
+        int rank = 0;
+        for (int k = b; k < e; ++k) rank += (unsorted[k] < int(slot)) ? 1 : 0;
+        const int k = b + rank;
+        A.perm[k] = int32_t(slot);
+        float G[3];
+        uint32_t pc;
+        int cc[3];
+        if constexpr (MODE == MD_FP64) {
+            const double4_32a p = A.pos64[cur][slot];
+            pc = cell_bits(p.w);
+            unpack_cell(pc, cc[0], cc[1], cc[2]);
+            G[0] = __double2float_rn(fma(double(cc[0]), R.w[0], p.x));
+            G[1] = __double2float_rn(fma(double(cc[1]), R.w[1], p.y));
+            G[2] = __double2float_rn(fma(double(cc[2]), R.w[2], p.z));
+        } else {
+            const float4 p = A.pos32[cur][slot];
+            pc = __float_as_uint(p.w);
+            unpack_cell(pc, cc[0], cc[1], cc[2]);
+            G[0] = fmaf(float(cc[0]), R.wf[0], p.x);
+            G[1] = fmaf(float(cc[1]), R.wf[1], p.y);
+            G[2] = fmaf(float(cc[2]), R.wf[2], p.z);
         }
-        if (A.ckeep && A.rs[A.cell_rep[c]].rebuild) {
-            const int base = A.cstart[A.rep[A.cell_rep[c]].cell0];
-            A.ckeep[c] = make_int2(b - base, e - base);
-        }
-        // the cell-ordered copy of the FP32 positions read by the neighbour build, slot in .w
-        if (A.psort && A.rs[A.cell_rep[c]].rebuild) {
-            const float4* __restrict__ pos = A.pos32[cur];
-            for (int k = b; k < e; ++k) {
-                const int32_t j = A.perm[k];
-                const float4 p = pos[j];
-                A.psort[k] = make_float4(p.x, p.y, p.z, __int_as_float(j));
-            }
-        }
+        const int prow = row_pos(R, cc[1], cc[2]);
+        const int rs = cs[R.cell0 + prow * R.nc[0]], re = cs[R.cell0 + (prow + 1) * R.nc[0]];
+        const int P = cand_place(R, prow, rs) + (k - rs);
+        const int64_t out_slot = A.rs[r].reorder ? R.slot0 + (k - cs[R.cell0]) : slot;
+        cand_store(A.psort, P, G[0], G[1], G[2], (uint32_t(out_slot) << IDX_SHIFT) | uint32_t(cc[0] & 3));
+        A.pcell[k] = pc;
+        if (k == re - 1)                              // far-away entries up to the group of 4
+            for (int q = P + 1; q & 3; ++q) cand_store(A.psort, q, CAND_FAR, CAND_FAR, CAND_FAR, 0u);
+    }
+}
+
+// the slot range of every cell in its replica, for the list-free step kernel
+__global__ void __launch_bounds__(256) k_cell_ranges(Arrays A, Scal S)
+{
+    if (!A.g->any_rebuild) return;
+    for (int64_t c = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; c < S.ncells; c += int64_t(gridDim.x) * blockDim.x) {
+        const int r = A.cell_rep[c];
+        if (!A.rs[r].rebuild) continue;
+        const int base = A.cstart[A.rep[r].cell0];
+        A.ckeep[c] = make_int2(A.cstart[c] - base, A.cstart[c + 1] - base);
     }
 }
 
@@ -463,9 +496,7 @@ __global__ void __launch_bounds__(TILE) k_reorder_copy(Arrays A, Scal S, int cur
         A.id[slot] = A.tmp_i[0][slot];
         A.slot_of_id[A.tmp_i[0][slot]] = int32_t(slot);
         A.cell[slot] = A.tmp_i[1][slot];
-        const int k = A.cstart[R.cell0] + int(j);
-        A.perm[k] = int32_t(slot);
-        if (MODE != MD_FP64) reinterpret_cast<float*>(A.psort + k)[3] = __int_as_float(int(slot));
+        A.perm[A.cstart[R.cell0] + int(j)] = int32_t(slot);
     }
 }
 
@@ -474,13 +505,6 @@ __global__ void __launch_bounds__(TILE) k_reorder_copy(Arrays A, Scal S, int cur
 // coordinates and o the periodic cell offset, d = (lf_j - lf_i) + o * wf (two roundings),
 // r2 = fma(d_z, d_z, fma(d_y, d_y, d_x * d_x)), neighbour iff r2 < (r_c + skin)^2.
 // ------------------------------------------------------------------------------------------
-template <typename T> struct PosT;
-template <> struct PosT<float> { using type = float4; };
-template <> struct PosT<double> { using type = double4_32a; };
-
-__device__ __forceinline__ uint32_t word_of(const float4& p) { return __float_as_uint(p.w); }
-__device__ __forceinline__ uint32_t word_of(const double4_32a& p) { return cell_bits(p.w); }
-
 __device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
@@ -490,735 +514,315 @@ __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-template <typename T, int BB>
-__global__ void __launch_bounds__(TILE) k_build(Arrays A, Scal S, int cur)
+// The criterion itself, for the atoms of slots me and j whose cells lie o apart: negative when j
+// is a neighbour.  ox is the unwrapped difference of the cells along x (sx the periodic shift of
+// j's run of cells); cells more than one apart hold no neighbours.
+template <int MODE>
+__device__ __noinline__ float criterion(const void* pos, const Rep* Rp, double rl2d, float rl2f, int me, int j, int sx,
+                                        int oy, int oz)
 {
-    using P4 = typename PosT<T>::type;
-    if (!A.g->any_rebuild) return;
-    const P4* __restrict__ pos = nullptr;
-    if constexpr (sizeof(T) == 8) pos = reinterpret_cast<const P4*>(A.pos64[cur]);
-    else pos = reinterpret_cast<const P4*>(A.pos32[cur]);
-    const T rl2 = (sizeof(T) == 8) ? T(S.rl2d) : T(S.rl2f);
-    const int nrb = A.g->n_rb_tiles;                  // tiles of the rebuilding replicas
-    const int per = (nrb + gridDim.x - 1) / gridDim.x;
-    const int t_begin = blockIdx.x * per, t_end = min(nrb, t_begin + per);
-    int run_r = -1, run_max = 0;
-    long long run_sum = 0;
-    for (int it = t_begin; it < t_end; ++it) {
-        const int t = A.rb_tiles[it];
-        const int r = A.tile_rep[t];
-        if (r != run_r) {
-            if (run_r >= 0) flush_stats(&A.rs[run_r].sum_nbrs, &A.rs[run_r].max_nbrs, run_sum, run_max);
-            run_r = r;
-            run_sum = 0;
-            run_max = 0;
-        }
-        const Rep& R = A.rep[r];
-        const int64_t slot = int64_t(t) * TILE + threadIdx.x;
-        const bool active = slot - R.slot0 < R.n;
-        int m = 0;
-        if (active) {
-            const P4 pi = pos[slot];
-            int cx, cy, cz;
-            unpack_cell(word_of(pi), cx, cy, cz);
-            T w[3];
-            if constexpr (sizeof(T) == 8) { w[0] = R.w[0]; w[1] = R.w[1]; w[2] = R.w[2]; }
-            else { w[0] = R.wf[0]; w[1] = R.wf[1]; w[2] = R.wf[2]; }
-            const int xm = (cx == 0) ? R.nc[0] - 1 : cx - 1;
-            const int xp = (cx == R.nc[0] - 1) ? 0 : cx + 1;
-            uint32_t* wp = A.W + slot;         // next free entry of this atom's column of W
-            // Squared distance from the atom to the lower and upper faces of its cell, per axis:
-            // a neighbouring cell whose nearest point is farther than r_c + skin cannot hold a
-            // neighbour.  The relative margin keeps this strictly looser than the criterion below.
-            const T lc[3] = {pi.x, pi.y, pi.z};
-            T dlo2[3], dhi2[3];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                dlo2[a] = lc[a] * lc[a];
-                dhi2[a] = (w[a] - lc[a]) * (w[a] - lc[a]);
-            }
-            const T skip2 = rl2 * ((sizeof(T) == 8) ? T(1.0 + 1e-12) : T(1.0f + 1e-5f));
-            for (int oz = -1; oz <= 1; ++oz) {
-                int nz = cz + oz; nz += (nz < 0) ? R.nc[2] : 0; nz -= (nz >= R.nc[2]) ? R.nc[2] : 0;
-                const T offz = T(oz) * w[2];
-                for (int oy = -1; oy <= 1; ++oy) {
-                    int ny = cy + oy; ny += (ny < 0) ? R.nc[1] : 0; ny -= (ny >= R.nc[1]) ? R.nc[1] : 0;
-                    const T offy = T(oy) * w[1];
-                    const T dyz = ((oy < 0) ? dlo2[1] : ((oy > 0) ? dhi2[1] : T(0))) +
-                                  ((oz < 0) ? dlo2[2] : ((oz > 0) ? dhi2[2] : T(0)));
-                    if (dyz > skip2) continue;
-                    const bool use_l = dyz + dlo2[0] <= skip2, use_r = dyz + dhi2[0] <= skip2;
-                    const int row = R.cell0 + row_pos(R, ny, nz) * R.nc[0];
-                    const uint32_t codeyz = (uint32_t(oy + 1) << 2) | (uint32_t(oz + 1) << 4);
-                    // the three cells of this row, as [b0,e0) [b1,e1) [b2,e2) in perm; without a
-                    // periodic wrap in x they are one contiguous range [b0, e2) split at b1, b2
-                    const int b0 = A.cstart[row + xm], e0 = use_l ? A.cstart[row + xm + 1] : b0;
-                    const int b1 = A.cstart[row + cx], e1 = A.cstart[row + cx + 1];
-                    const int b2 = A.cstart[row + xp], e2 = use_r ? A.cstart[row + xp + 1] : b2;
-                    if (cx > 0 && cx < R.nc[0] - 1) {
-                        // consecutive cells: one range, starting past the left cell if it is skipped
-                        const int kb = use_l ? b0 : b1;
-                        for (int k0 = kb; k0 < e2; k0 += BB) {
-                            int32_t js[BB];
-#pragma unroll
-                            for (int u = 0; u < BB; ++u) js[u] = A.perm[min(k0 + u, e2 - 1)];
-                            P4 pj[BB];
-#pragma unroll
-                            for (int u = 0; u < BB; ++u) pj[u] = pos[js[u]];
-#pragma unroll
-                            for (int u = 0; u < BB; ++u) {
-                                const int k = k0 + u;
-                                const int ox = int(k >= b1) + int(k >= b2) - 1;
-                                const T offx = (ox < 0) ? -w[0] : ((ox > 0) ? w[0] : T(0));
-                                const T dx = add_rn(sub_rn(pj[u].x, pi.x), offx);
-                                const T dy = add_rn(sub_rn(pj[u].y, pi.y), offy);
-                                const T dz = add_rn(sub_rn(pj[u].z, pi.z), offz);
-                                const T r2 = fma_rn(dz, dz, fma_rn(dy, dy, mul_rn(dx, dx)));
-                                if (k < e2 && r2 < rl2 && js[u] != slot) {
-                                    if (m < S.cap) {
-                                        *wp = (uint32_t(js[u]) << IDX_SHIFT) | codeyz | uint32_t(ox + 1);
-                                        wp += S.nslots;
-                                    }
-                                    ++m;
-                                }
-                            }
-                        }
-                        continue;
-                    }
-                    const int n0 = e0 - b0, n01 = n0 + (e1 - b1), ntot = n01 + (e2 - b2);
-                    for (int q0 = 0; q0 < ntot; q0 += BB) {
-                        int32_t js[BB];
-#pragma unroll
-                        for (int u = 0; u < BB; ++u) {
-                            const int q = q0 + u;
-                            const int k = (q < n0) ? b0 + q : ((q < n01) ? b1 + (q - n0) : b2 + (q - n01));
-                            js[u] = (q < ntot) ? A.perm[k] : -1;
-                        }
-                        P4 pj[BB];
-#pragma unroll
-                        for (int u = 0; u < BB; ++u) pj[u] = (js[u] >= 0) ? pos[js[u]] : pi;
-#pragma unroll
-                        for (int u = 0; u < BB; ++u) {
-                            const int q = q0 + u;
-                            if (js[u] < 0 || js[u] == slot) continue;
-                            const int ox = (q < n0) ? -1 : ((q < n01) ? 0 : 1);
-                            const T offx = T(ox) * w[0];
-                            const T dx = add_rn(sub_rn(pj[u].x, pi.x), offx);
-                            const T dy = add_rn(sub_rn(pj[u].y, pi.y), offy);
-                            const T dz = add_rn(sub_rn(pj[u].z, pi.z), offz);
-                            const T r2 = fma_rn(dz, dz, fma_rn(dy, dy, mul_rn(dx, dx)));
-                            if (r2 < rl2) {
-                                if (m < S.cap) {
-                                    *wp = (uint32_t(js[u]) << IDX_SHIFT) | codeyz | uint32_t(ox + 1);
-                                    wp += S.nslots;
-                                }
-                                ++m;
-                            }
-                        }
-                    }
-                }
-            }
-            A.nbr_count[slot] = m;
-            if (S.rule == MD_REBUILD_DISP) {
-                A.xref[slot] = make_float4(float(pi.x), float(pi.y), float(pi.z), 0.0f);
-            }
-            if (m > S.cap) {
-                atomicOr(&A.g->err, ERR_NBR_OVERFLOW);
-                atomicMax(&A.g->max_nbr_seen, m);
-            }
-        }
-        if (active) {
-            run_sum += m;
-            run_max = max(run_max, m);
-        }
+    const Rep& R = *Rp;
+    int ci[3], cj[3];
+    if constexpr (MODE == MD_FP64) {
+        const double4_32a pi = static_cast<const double4_32a*>(pos)[me], pj = static_cast<const double4_32a*>(pos)[j];
+        unpack_cell(cell_bits(pi.w), ci[0], ci[1], ci[2]);
+        unpack_cell(cell_bits(pj.w), cj[0], cj[1], cj[2]);
+        const int ox = cj[0] + sx - ci[0];
+        if (ox < -1 || ox > 1) return 1.0f;
+        const double dx = add_rn(sub_rn(pj.x, pi.x), double(ox) * R.w[0]);
+        const double dy = add_rn(sub_rn(pj.y, pi.y), double(oy) * R.w[1]);
+        const double dz = add_rn(sub_rn(pj.z, pi.z), double(oz) * R.w[2]);
+        return fma_rn(dz, dz, fma_rn(dy, dy, mul_rn(dx, dx))) < rl2d ? -1.0f : 1.0f;
+    } else {
+        const float4 pi = static_cast<const float4*>(pos)[me], pj = static_cast<const float4*>(pos)[j];
+        unpack_cell(__float_as_uint(pi.w), ci[0], ci[1], ci[2]);
+        unpack_cell(__float_as_uint(pj.w), cj[0], cj[1], cj[2]);
+        const int ox = cj[0] + sx - ci[0];
+        if (ox < -1 || ox > 1) return 1.0f;
+        const float dx = add_rn(sub_rn(pj.x, pi.x), float(ox) * R.wf[0]);
+        const float dy = add_rn(sub_rn(pj.y, pi.y), float(oy) * R.wf[1]);
+        const float dz = add_rn(sub_rn(pj.z, pi.z), float(oz) * R.wf[2]);
+        return fma_rn(dz, dz, fma_rn(dy, dy, mul_rn(dx, dx))) < rl2f ? -1.0f : 1.0f;
     }
-    if (run_r >= 0) flush_stats(&A.rs[run_r].sum_nbrs, &A.rs[run_r].max_nbrs, run_sum, run_max);
-}
-
-
-// N5 in FP32 from the cell-ordered copy of the positions: psort[k] is the k-th atom of the cell
-// order (the order of perm) with its slot in .w, so the candidates of a 3-cell row are one
-// contiguous run of psort (three separate runs at a periodic wrap in x), read in order with no
-// load through perm.  x and y of a candidate are adjacent in its float4 and go through packed
-// FP32x2 adds; each lane rounds as the scalar criterion does (a - b is a + (-b)), and the rows,
-// cells and candidates are visited in k_build's order, so W is entry for entry k_build's.
-// With half = 1 (the half list of step kernel 5) only partners of a higher slot are kept: the
-// criterion is exactly antisymmetric in i and j (IEEE subtraction and negation), so every pair
-// is kept once.
-__device__ __forceinline__ void nbr_test(const float4& p, const float2& npxy, float npz, float offx, float offy,
-                                         float offz, bool valid, uint32_t code, int me, float rl2, uint32_t*& wp,
-                                         int& m, int cap, int64_t stride, int half)
-{
-    const float2 dxy = __fadd2_rn(__fadd2_rn(make_float2(p.x, p.y), npxy), make_float2(offx, offy));
-    const float dz = __fadd_rn(__fadd_rn(p.z, npz), offz);
-    const float r2 = __fmaf_rn(dz, dz, __fmaf_rn(dxy.y, dxy.y, __fmul_rn(dxy.x, dxy.x)));
-    const int j = __float_as_int(p.w);
-    if (valid && r2 < rl2 && (half ? j > me : j != me)) {
-        if (m < cap) {
-            *wp = (uint32_t(j) << IDX_SHIFT) | code;
-            wp += stride;
-        }
-        ++m;
-    }
-}
-
-// The order in which a CTA of a neighbour build takes the rebuild tiles: chunks of BUILD_CHUNK
-// consecutive tiles dealt to the CTAs in turn, so that the CTAs resident at one time work on one
-// stretch of consecutive slots (grid x BUILD_CHUNK tiles) and the candidate rows they read stay
-// in L2; contiguous runs per CTA spread them over the whole system (measured in the build A/B).
-constexpr int BUILD_CHUNK = 4;
-#define build_tile(q) ((((q) / BUILD_CHUNK) * int(gridDim.x) + int(blockIdx.x)) * BUILD_CHUNK + (q) % BUILD_CHUNK)
-
-// Two candidates of a row in one pass of packed FP32x2 operations (candidate a in lane x, b in
-// lane y); each lane rounds as nbr_test does, and a is appended before b, so W is the same entry
-// for entry.
-__device__ __forceinline__ void nbr_test2(const float4& pa, const float4& pb, float2 nx, float2 ny, float2 nz,
-                                          float2 offx, float offy, float offz, bool va, bool vb, uint32_t ca,
-                                          uint32_t cb, int me, float rl2, uint32_t*& wp, int& m, int cap,
-                                          int64_t stride, int half)
-{
-    const float2 dx = __fadd2_rn(__fadd2_rn(make_float2(pa.x, pb.x), nx), offx);
-    const float2 dy = __fadd2_rn(__fadd2_rn(make_float2(pa.y, pb.y), ny), make_float2(offy, offy));
-    const float2 dz = __fadd2_rn(__fadd2_rn(make_float2(pa.z, pb.z), nz), make_float2(offz, offz));
-    const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
-    const int ja = __float_as_int(pa.w), jb = __float_as_int(pb.w);
-    if (va && r2.x < rl2 && (half ? ja > me : ja != me)) {
-        if (m < cap) {
-            *wp = (uint32_t(ja) << IDX_SHIFT) | ca;
-            wp += stride;
-        }
-        ++m;
-    }
-    if (vb && r2.y < rl2 && (half ? jb > me : jb != me)) {
-        if (m < cap) {
-            *wp = (uint32_t(jb) << IDX_SHIFT) | cb;
-            wp += stride;
-        }
-        ++m;
-    }
-}
-
-// STAGE: a thread appends its column of W to shared memory (stride TILE) instead of W itself,
-// and each warp then writes its columns row by row: 32 consecutive slots of a row are 128
-// contiguous bytes, where entries written as found land one at a time in partly written sectors.
-// Every thread reads back only its own column, so no block barrier is needed.
-__device__ __forceinline__ void flush_columns(const Arrays& A, const Scal& S, const uint32_t* sW, int64_t slot, int mc)
-{
-    const int mw = int(__reduce_max_sync(0xffffffffu, unsigned(mc)));
-    for (int q = 0; q < mw; ++q)
-        if (q < mc) A.W[int64_t(q) * S.nslots + slot] = sW[q * TILE + threadIdx.x];
-}
-
-template <int BB, bool STAGE>
-__global__ void __launch_bounds__(TILE) k_build_sorted(Arrays A, Scal S, int cur)
-{
-    static_assert(BB % 2 == 0, "candidates are tested in pairs");
-    extern __shared__ uint32_t sW[];                 // STAGE: [cap][TILE] columns of this tile
-    if (!A.g->any_rebuild) return;
-    const int64_t wstride = STAGE ? int64_t(TILE) : S.nslots;
-    const float4* __restrict__ pos = A.pos32[cur];
-    const float4* __restrict__ ps = A.psort;
-    const int32_t* __restrict__ cs = A.cstart;
-    const float rl2 = S.rl2f;
-    const float skip2 = rl2 * (1.0f + 1e-5f);
-    const int nrb = A.g->n_rb_tiles;
-    int run_r = -1, run_max = 0;
-    long long run_sum = 0;
-    for (int q = 0;; ++q) {
-        const int it = build_tile(q);
-        if (it >= nrb) break;
-        const int t = A.rb_tiles[it];
-        const int r = A.tile_rep[t];
-        if (r != run_r) {
-            if (run_r >= 0) flush_stats(&A.rs[run_r].sum_nbrs, &A.rs[run_r].max_nbrs, run_sum, run_max);
-            run_r = r;
-            run_sum = 0;
-            run_max = 0;
-        }
-        const Rep& R = A.rep[r];
-        const int64_t slot = int64_t(t) * TILE + threadIdx.x;
-        const bool active = slot - R.slot0 < R.n;
-        int m = 0;
-        if (active) {
-            const float4 pi = pos[slot];
-            int cx, cy, cz;
-            unpack_cell(__float_as_uint(pi.w), cx, cy, cz);
-            const float w0 = R.wf[0], w1 = R.wf[1], w2 = R.wf[2];
-            const int ncx = R.nc[0];
-            const bool inner = cx > 0 && cx < ncx - 1;
-            const int me = int(slot);
-            uint32_t* wp = STAGE ? sW + threadIdx.x : A.W + slot;
-            // neighbouring cells whose nearest point is beyond r_c + skin are skipped (as k_build)
-            const float dlo2[3] = {pi.x * pi.x, pi.y * pi.y, pi.z * pi.z};
-            const float dhi2[3] = {(w0 - pi.x) * (w0 - pi.x), (w1 - pi.y) * (w1 - pi.y), (w2 - pi.z) * (w2 - pi.z)};
-            const float2 npxy = make_float2(-pi.x, -pi.y);
-            const float npz = -pi.z;
-            const float2 nx2 = make_float2(-pi.x, -pi.x), ny2 = make_float2(-pi.y, -pi.y), nz2 = make_float2(-pi.z, -pi.z);
-            for (int oz = -1; oz <= 1; ++oz) {
-                int nz = cz + oz; nz += (nz < 0) ? R.nc[2] : 0; nz -= (nz >= R.nc[2]) ? R.nc[2] : 0;
-                const float offz = float(oz) * w2;
-                for (int oy = -1; oy <= 1; ++oy) {
-                    int ny = cy + oy; ny += (ny < 0) ? R.nc[1] : 0; ny -= (ny >= R.nc[1]) ? R.nc[1] : 0;
-                    const float offy = float(oy) * w1;
-                    const float dyz = ((oy < 0) ? dlo2[1] : ((oy > 0) ? dhi2[1] : 0.0f)) +
-                                      ((oz < 0) ? dlo2[2] : ((oz > 0) ? dhi2[2] : 0.0f));
-                    if (dyz > skip2) continue;
-                    const bool use_l = dyz + dlo2[0] <= skip2, use_r = dyz + dhi2[0] <= skip2;
-                    const int row = R.cell0 + row_pos(R, ny, nz) * ncx;
-                    const uint32_t codeyz = (uint32_t(oy + 1) << 2) | (uint32_t(oz + 1) << 4);
-                    if (inner) {
-                        // cells cx-1, cx, cx+1 are adjacent runs [b0,b1) [b1,b2) [b2,b3) of psort
-                        const int b0 = cs[row + cx - 1], b1 = cs[row + cx], b2 = cs[row + cx + 1];
-                        const int kb = use_l ? b0 : b1;
-                        const int ke = use_r ? cs[row + cx + 2] : b2;
-                        // psort has PSORT_PAD entries past its end, so the last batch reads
-                        // past ke unclamped (those lanes are invalid)
-                        for (int k0 = kb; k0 < ke; k0 += BB) {
-                            float4 pj[BB];
-#pragma unroll
-                            for (int u = 0; u < BB; ++u) pj[u] = ps[k0 + u];
-#pragma unroll
-                            for (int u = 0; u < BB; u += 2) {
-                                const int ka = k0 + u, kb2 = ka + 1;
-                                const uint32_t ca = uint32_t(ka >= b1) + uint32_t(ka >= b2);   // o_x + 1
-                                const uint32_t cb = uint32_t(kb2 >= b1) + uint32_t(kb2 >= b2);
-                                const float2 offx = make_float2((ka < b1) ? -w0 : ((ka < b2) ? 0.0f : w0),
-                                                                (kb2 < b1) ? -w0 : ((kb2 < b2) ? 0.0f : w0));
-                                nbr_test2(pj[u], pj[u + 1], nx2, ny2, nz2, offx, offy, offz, ka < ke, kb2 < ke,
-                                          codeyz | ca, codeyz | cb, me, rl2, wp, m, S.cap, wstride, S.half_list);
-                            }
-                        }
-                    } else {
-                        // a periodic wrap in x: the three cells are separate runs, in the same order
-                        const int xs[3] = {(cx == 0) ? ncx - 1 : cx - 1, cx, (cx == ncx - 1) ? 0 : cx + 1};
-#pragma unroll
-                        for (int c = 0; c < 3; ++c) {
-                            if ((c == 0 && !use_l) || (c == 2 && !use_r)) continue;
-                            const int b = cs[row + xs[c]], e = cs[row + xs[c] + 1];
-                            const float offx = float(c - 1) * w0;
-                            for (int k0 = b; k0 < e; k0 += BB) {
-                                float4 pj[BB];
-#pragma unroll
-                                for (int u = 0; u < BB; ++u) pj[u] = ps[min(k0 + u, e - 1)];
-#pragma unroll
-                                for (int u = 0; u < BB; ++u)
-                                    nbr_test(pj[u], npxy, npz, offx, offy, offz, k0 + u < e, codeyz | uint32_t(c), me,
-                                             rl2, wp, m, S.cap, wstride, S.half_list);
-                            }
-                        }
-                    }
-                }
-            }
-            A.nbr_count[slot] = m;
-            if (S.rule == MD_REBUILD_DISP) A.xref[slot] = make_float4(pi.x, pi.y, pi.z, 0.0f);
-            if (m > S.cap) {
-                atomicOr(&A.g->err, ERR_NBR_OVERFLOW);
-                atomicMax(&A.g->max_nbr_seen, m);
-            }
-            run_sum += m;
-            run_max = max(run_max, m);
-        }
-        if (STAGE) flush_columns(A, S, sW, slot, active ? min(m, S.cap) : 0);
-    }
-    if (run_r >= 0) flush_stats(&A.rs[run_r].sum_nbrs, &A.rs[run_r].max_nbrs, run_sum, run_max);
 }
 
 // ------------------------------------------------------------------------------------------
-// N5 over half-side sub-cells.  Every cell of side w >= r_c + skin is split into 2 x 2 x 2
-// sub-cells of side w / 2 (an atom's sub-cell along an axis is 2 c + (l >= w / 2)), and the atoms
-// are counting-sorted by sub-cell into psub (rows of sub-cells along x contiguous, ascending slot
-// within a sub-cell).  A neighbour lies at most 2 sub-cells away along each axis, and of the
-// 5 x 5 x 5 sub-cells around an atom only those whose nearest point is within r_c + skin are
-// scanned: a row (fixed y, z) at a time, as one contiguous run of psub.  That tests about half
-// the candidates of the 27 cells (WCA) and 40 % of them at the LJ cutoff.  The test itself is
-// the criterion's expression, d = (lf_j - lf_i) + o * wf with o the offset of j's cell, so the
-// sets are those of k_build_sorted (the order within a column follows the sub-cell rows).
-// The sub-cell slot of an atom is kept in A.layer (free once the cell order is built).
+// N5, the build of W.  A warp takes a unit of BG_ATOMS atoms consecutive in cell order; lane
+// (a, plane) scans, for atom a, the three rows of cells of one z plane of the 27 around it, so the
+// three planes of an atom are scanned at the same time.
+//
+// A candidate is tested on its position in the replica's frame (cand_store), two per packed
+// FP32x2 operation: d = |r|^2 - (r_c + skin)^2.  That differs from the criterion's expression by at
+// most R.band; where |d| is below the band (a few pairs in 10^4) the criterion itself decides, so
+// the sets are the criterion's exactly.  A run of candidates starts and ends at a multiple of 4:
+// an atom of a cell more than one away is farther than r_c + skin, so it needs no bounds, and rows
+// of cells end in far-away entries.  An accepted candidate is appended to the lane's own list in
+// shared memory by predicated instructions, without a branch.  After the three rows the warp joins
+// each atom's three lists (planes in order, so the entries of a column come in the order rows,
+// cells, slots) and writes W row by row: consecutive lanes write consecutive slots.
+//
+// Bounds: the loads of candidates return 16 bytes to each of 32 lanes, 4 cycles of the SM's 128
+// bytes per cycle (65 % busy), and about 12 instructions per candidate issue (45 %).  Measured
+// against one thread per atom walking its nine rows and branching at every append (per rebuild,
+// GB300): LJ r_c + skin = 2.8: 16.4M atoms 27.7 -> 12 ms, 256k atoms 513 -> 210 us, 4000 atoms
+// 388 -> 22 us; WCA: 100k atoms 110 -> 30 us, 4M atoms 0.76 -> 0.75 ms (the two are even there);
+// FP64, 2048 atoms 71 -> 11 us (positions tested in FP32, the criterion in FP64).  The lanes' own
+// runs beat one run shared by a unit's atoms of a row (fewer distinct addresses per load, more
+// candidates: 0.59 against 0.69 ms at 2M WCA atoms, 0.72 against 0.78 ms at 864k LJ atoms);
+// loads one pass ahead cost registers and lost (0.70 and 0.86 ms).
 // ------------------------------------------------------------------------------------------
-__device__ __forceinline__ int sub_of(float l, float w, int c) { return 2 * c + ((l >= 0.5f * w) ? 1 : 0); }
+constexpr int BG_ATOMS = 10;
+constexpr int BG_UNITS = (TILE + BG_ATOMS - 1) / BG_ATOMS;       // units per rebuild tile
+constexpr int BG_STEP = 4;                                       // candidates per pass of the scan
+constexpr uint32_t BG_ROW = 32 * 4;                              // bytes of one row of the lists
 
-__device__ __forceinline__ int64_t sub_index(const Rep& R, int sx, int sy, int sz)
+// append v to the list at shared address w where d < 0
+__device__ __forceinline__ void list_append(uint32_t& w, float d, uint32_t v)
 {
-    return int64_t(8) * R.cell0 + (int64_t(sz) * (2 * R.nc[1]) + sy) * (2 * R.nc[0]) + sx;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %1, 0f00000000;\n\t@p st.shared.u32 [%0], %2;\n\t"
+                 "@p add.u32 %0, %0, 128;\n\t}"
+                 : "+r"(w) : "f"(d), "r"(v));
+}
+// the same where also e != self (NE) or e > self (unsigned)
+template <bool GT>
+__device__ __forceinline__ void list_append_if(uint32_t& w, float d, uint32_t v, uint32_t e, uint32_t self)
+{
+    if constexpr (GT)
+        asm volatile("{\n\t.reg .pred p, q;\n\tsetp.gt.u32 q, %3, %4;\n\tsetp.lt.and.f32 p, %1, 0f00000000, q;\n\t"
+                     "@p st.shared.u32 [%0], %2;\n\t@p add.u32 %0, %0, 128;\n\t}"
+                     : "+r"(w) : "f"(d), "r"(v), "r"(e), "r"(self));
+    else
+        asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %3, %4;\n\tsetp.lt.and.f32 p, %1, 0f00000000, q;\n\t"
+                     "@p st.shared.u32 [%0], %2;\n\t@p add.u32 %0, %0, 128;\n\t}"
+                     : "+r"(w) : "f"(d), "r"(v), "r"(e), "r"(self));
 }
 
-__device__ __forceinline__ int64_t sub_of_atom(const Rep& R, const float4& p)
-{
-    int cx, cy, cz;
-    unpack_cell(__float_as_uint(p.w), cx, cy, cz);
-    return sub_index(R, sub_of(p.x, R.wf[0], cx), sub_of(p.y, R.wf[1], cy), sub_of(p.z, R.wf[2], cz));
-}
-
-__global__ void __launch_bounds__(TILE) k_sub_bin(Arrays A, Scal S, int cur)
-{
-    if (!A.g->any_rebuild) return;
-    const int nrb = A.g->n_rb_tiles;
-    for (int it = blockIdx.x; it < nrb; it += gridDim.x) {
-        const int t = A.rb_tiles[it];
-        const Rep& R = A.rep[A.tile_rep[t]];
-        const int64_t slot = int64_t(t) * TILE + threadIdx.x;
-        const bool active = slot - R.slot0 < R.n;
-        const long long sub = active ? sub_of_atom(R, A.pos32[cur][slot]) : -1;
-        // lanes of a warp that share a sub-cell take consecutive slots from one atomic
-        const unsigned peers = __match_any_sync(0xffffffffu, sub);
-        const int lane = threadIdx.x & 31;
-        const int leader = __ffs(peers) - 1;
-        const int rank = __popc(peers & ((1u << lane) - 1u));
-        int base = 0;
-        if (active && lane == leader) base = atomicAdd(&A.scount[sub], __popc(peers));
-        base = __shfl_sync(0xffffffffu, base, leader);
-        if (active) A.layer[slot] = base + rank;
-    }
-}
-
-__global__ void __launch_bounds__(TILE) k_sub_scatter(Arrays A, Scal S, int cur)
-{
-    if (!A.g->any_rebuild) return;
-    const int nrb = A.g->n_rb_tiles;
-    for (int it = blockIdx.x; it < nrb; it += gridDim.x) {
-        const int t = A.rb_tiles[it];
-        const Rep& R = A.rep[A.tile_rep[t]];
-        const int64_t slot = int64_t(t) * TILE + threadIdx.x;
-        if (slot - R.slot0 >= R.n) continue;
-        const float4 p = A.pos32[cur][slot];
-        A.psub[A.sstart[sub_of_atom(R, p)] + A.layer[slot]] = make_float4(p.x, p.y, p.z, __int_as_float(int(slot)));
-    }
-}
-
-// ascending slot within each sub-cell (the atomic slots leave the order to chance)
-__global__ void __launch_bounds__(256) k_sub_sort(Arrays A, Scal S)
-{
-    if (!A.g->any_rebuild) return;
-    for (int64_t c = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; c < S.nsub; c += int64_t(gridDim.x) * blockDim.x) {
-        const int b = A.sstart[c], e = A.sstart[c + 1];
-        for (int k = b + 1; k < e; ++k) {
-            const float4 key = A.psub[k];
-            int q = k - 1;
-            while (q >= b && __float_as_int(A.psub[q].w) > __float_as_int(key.w)) {
-                A.psub[q + 1] = A.psub[q];
-                --q;
-            }
-            A.psub[q + 1] = key;
-        }
-    }
-}
-
-// squared distance from l to the sub-cell interval [j h, (j + 1) h) of the atom's cell frame
-__device__ __forceinline__ float sub_gap2(float l, int j, float h)
-{
-    const float lo = float(j) * h, hi = lo + h;
-    const float d = (l < lo) ? lo - l : ((l > hi) ? l - hi : 0.0f);
-    return d * d;
-}
-
-template <int BB, bool STAGE>
-__global__ void __launch_bounds__(TILE) k_build_sub(Arrays A, Scal S, int cur)
-{
-    extern __shared__ uint32_t sW[];                 // STAGE: [cap][TILE] columns of this tile
-    if (!A.g->any_rebuild) return;
-    const int64_t wstride = STAGE ? int64_t(TILE) : S.nslots;
-    const float4* __restrict__ pos = A.pos32[cur];
-    const float4* __restrict__ ps = A.psub;
-    const int32_t* __restrict__ ss = A.sstart;
-    const float rl2 = S.rl2f;
-    const float skip2 = rl2 * (1.0f + 1e-5f);
-    const int nrb = A.g->n_rb_tiles;
-    int run_r = -1, run_max = 0;
-    long long run_sum = 0;
-    for (int q = 0;; ++q) {
-        const int it = build_tile(q);
-        if (it >= nrb) break;
-        const int t = A.rb_tiles[it];
-        const int r = A.tile_rep[t];
-        if (r != run_r) {
-            if (run_r >= 0) flush_stats(&A.rs[run_r].sum_nbrs, &A.rs[run_r].max_nbrs, run_sum, run_max);
-            run_r = r;
-            run_sum = 0;
-            run_max = 0;
-        }
-        const Rep& R = A.rep[r];
-        const int64_t slot = int64_t(t) * TILE + threadIdx.x;
-        const bool active = slot - R.slot0 < R.n;
-        int m = 0;
-        if (active) {
-            const float4 pi = pos[slot];
-            int cx, cy, cz;
-            unpack_cell(__float_as_uint(pi.w), cx, cy, cz);
-            const float w0 = R.wf[0], w1 = R.wf[1], w2 = R.wf[2];
-            const float h0 = 0.5f * w0, h1 = 0.5f * w1, h2 = 0.5f * w2;
-            // the atom's half along each axis; sub-cell j = b + d (d = -2..2) of the cell frame
-            const int bx = (pi.x >= h0) ? 1 : 0, by = (pi.y >= h1) ? 1 : 0, bz = (pi.z >= h2) ? 1 : 0;
-            const int nsx = 2 * R.nc[0], nsy = 2 * R.nc[1], nsz = 2 * R.nc[2];
-            float gx[5];
-#pragma unroll
-            for (int d = 0; d < 5; ++d) gx[d] = sub_gap2(pi.x, bx + d - 2, h0);
-            const int me = int(slot);
-            uint32_t* wp = STAGE ? sW + threadIdx.x : A.W + slot;
-            const float2 npxy = make_float2(-pi.x, -pi.y);
-            const float npz = -pi.z;
-            for (int dz = 0; dz < 5; ++dz) {
-                const int jz = bz + dz - 2;
-                const float gz = sub_gap2(pi.z, jz, h2);
-                if (gz > skip2) continue;
-                const int oz = jz >> 1;                            // offset of the sub-cell's cell
-                int sz = 2 * cz + jz; sz += (sz < 0) ? nsz : 0; sz -= (sz >= nsz) ? nsz : 0;
-                const float offz = float(oz) * w2;
-                for (int dy = 0; dy < 5; ++dy) {
-                    const int jy = by + dy - 2;
-                    const float gyz = sub_gap2(pi.y, jy, h1) + gz;
-                    if (gyz > skip2) continue;
-                    // the sub-cells of this row within reach form one range d = lo .. hi
-                    int lo = 5, hi = -1;
-#pragma unroll
-                    for (int d = 0; d < 5; ++d) {
-                        if (gyz + gx[d] <= skip2) {
-                            lo = min(lo, d);
-                            hi = d;
-                        }
-                    }
-                    if (hi < 0) continue;
-                    const int oy = jy >> 1;
-                    int sy = 2 * cy + jy; sy += (sy < 0) ? nsy : 0; sy -= (sy >= nsy) ? nsy : 0;
-                    const float offy = float(oy) * w1;
-                    const uint32_t codeyz = (uint32_t(oy + 1) << 2) | (uint32_t(oz + 1) << 4);
-                    const int64_t row = sub_index(R, 0, sy, sz);
-                    const int sxl = 2 * cx + bx + lo - 2, sxh = 2 * cx + bx + hi - 2;
-                    if (sxl >= 0 && sxh < nsx) {
-                        // one run of psub; the cells change at sub-cells 2 cx and 2 cx + 2
-                        const int kb = ss[row + sxl], ke = ss[row + sxh + 1];
-                        const int b1 = ss[row + min(max(2 * cx, sxl), sxh + 1)];
-                        const int b2 = ss[row + min(max(2 * cx + 2, sxl), sxh + 1)];
-                        for (int k0 = kb; k0 < ke; k0 += BB) {
-                            float4 pj[BB];
-#pragma unroll
-                            for (int u = 0; u < BB; ++u) pj[u] = ps[min(k0 + u, ke - 1)];
-#pragma unroll
-                            for (int u = 0; u < BB; ++u) {
-                                const int k = k0 + u;
-                                const uint32_t c = uint32_t(k >= b1) + uint32_t(k >= b2);   // o_x + 1
-                                const float offx = (k < b1) ? -w0 : ((k < b2) ? 0.0f : w0);
-                                nbr_test(pj[u], npxy, npz, offx, offy, offz, k < ke, codeyz | c, me, rl2, wp, m,
-                                         S.cap, wstride, S.half_list);
-                            }
-                        }
-                    } else {
-                        // a periodic wrap in x: sub-cell by sub-cell
-                        for (int d = lo; d <= hi; ++d) {
-                            const int jx = bx + d - 2;
-                            const int ox = jx >> 1;
-                            int sx = 2 * cx + jx; sx += (sx < 0) ? nsx : 0; sx -= (sx >= nsx) ? nsx : 0;
-                            const int b = ss[row + sx], e = ss[row + sx + 1];
-                            const float offx = float(ox) * w0;
-                            for (int k0 = b; k0 < e; k0 += BB) {
-                                float4 pj[BB];
-#pragma unroll
-                                for (int u = 0; u < BB; ++u) pj[u] = ps[min(k0 + u, e - 1)];
-#pragma unroll
-                                for (int u = 0; u < BB; ++u)
-                                    nbr_test(pj[u], npxy, npz, offx, offy, offz, k0 + u < e, codeyz | uint32_t(ox + 1), me,
-                                             rl2, wp, m, S.cap, wstride, S.half_list);
-                            }
-                        }
-                    }
-                }
-            }
-            A.nbr_count[slot] = m;
-            if (S.rule == MD_REBUILD_DISP) A.xref[slot] = make_float4(pi.x, pi.y, pi.z, 0.0f);
-            if (m > S.cap) {
-                atomicOr(&A.g->err, ERR_NBR_OVERFLOW);
-                atomicMax(&A.g->max_nbr_seen, m);
-            }
-            run_sum += m;
-            run_max = max(run_max, m);
-        }
-        if (STAGE) flush_columns(A, S, sW, slot, active ? min(m, S.cap) : 0);
-    }
-    if (run_r >= 0) flush_stats(&A.rs[run_r].sum_nbrs, &A.rs[run_r].max_nbrs, run_sum, run_max);
-}
-
-// ------------------------------------------------------------------------------------------
-// N5 for dense cells (tens of atoms per cell, e.g. the LJ liquid at r_c + skin = 2.8): one warp
-// per cell, one lane per atom of it.  The candidates of each 3-cell row of the 27-cell
-// neighbourhood are staged once in the warp's shared memory (coalesced loads, double-buffered:
-// the next row is loaded while the current one is tested), and every lane tests them with
-// broadcast reads, so no candidate is fetched per lane and no lane diverges.  The displacement
-// is the criterion's expression (p_j - p_i) + o w, o constant per cell.  Rows and cells no lane
-// of the warp can reach are skipped by a warp vote.
-// ------------------------------------------------------------------------------------------
-constexpr int CW_WARPS = TILE / 32;
-constexpr int CW_ROW = 128;                    // candidates of one row staged at a time
-constexpr int CW_PER_LANE = CW_ROW / 32;
-
-struct CwRow {
-    int b[3], n[3];                           // the three cells of the row as perm ranges
-    int tot;
+struct ScanLane {               // what a lane keeps while it scans
+    float2 nx, ny, nz;          // minus the atom's coordinates, as seen from the row's cells
+    float band;
+    uint32_t self;              // its own entry (HALF: its slot's last code)
+    uint32_t w, wlim, lost;     // list position and its limit; entries beyond it
 };
 
-__device__ __forceinline__ int cw_index(const CwRow& R, int q)
+// Candidates [P0, P1) (multiples of 4) of one run.  SELF: the run may hold the atom itself.
+// IMG: the run lies across the periodic boundary in x, imgadd = its shift in cells (mod 4).
+template <int MODE, bool HALF, bool SELF, bool IMG>
+__device__ __forceinline__ void scan_run(const float4* __restrict__ ps, int P0, int P1, ScanLane& L, float rl2f,
+                                         double rl2d, uint32_t code, uint32_t imgadd, const void* pos, const Rep* Rp,
+                                         int sx, int oy, int oz)
 {
-    return (q < R.n[0]) ? R.b[0] + q : ((q < R.n[0] + R.n[1]) ? R.b[1] + (q - R.n[0]) : R.b[2] + (q - R.n[0] - R.n[1]));
+    const float2 nrl2 = make_float2(-rl2f, -rl2f);
+    for (int P = P0; P < P1; P += BG_STEP) {
+        float d[BG_STEP];
+        uint32_t e[BG_STEP];
+#pragma unroll
+        for (int h = 0; h < BG_STEP / 2; ++h) {
+            const float4 xy = __ldg(ps + P + 2 * h), ze = __ldg(ps + P + 2 * h + 1);
+            const float2 dx = __fadd2_rn(make_float2(xy.x, xy.y), L.nx);
+            const float2 dy = __fadd2_rn(make_float2(xy.z, xy.w), L.ny);
+            const float2 dz = __fadd2_rn(make_float2(ze.x, ze.y), L.nz);
+            const float2 q = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __ffma2_rn(dx, dx, nrl2)));
+            d[2 * h] = q.x;
+            d[2 * h + 1] = q.y;
+            e[2 * h] = __float_as_uint(ze.z);
+            e[2 * h + 1] = __float_as_uint(ze.w);
+        }
+        if (fminf(fminf(fabsf(d[0]), fabsf(d[1])), fminf(fabsf(d[2]), fabsf(d[3]))) < L.band) {
+#pragma unroll
+            for (int u = 0; u < BG_STEP; ++u)
+                if (fabsf(d[u]) < L.band)
+                    d[u] = criterion<MODE>(pos, Rp, rl2d, rl2f, int(L.self >> IDX_SHIFT), int(e[u] >> IDX_SHIFT), sx, oy, oz);
+        }
+#pragma unroll
+        for (int u = 0; u < BG_STEP; ++u) {
+            const uint32_t v = IMG ? (((e[u] + imgadd) & ~0x3Cu) | code) : (e[u] | code);
+            if (HALF) list_append_if<true>(L.w, d[u], v, e[u], L.self | 63u);
+            else if (SELF) list_append_if<false>(L.w, d[u], v, e[u], L.self);
+            else list_append(L.w, d[u], v);
+        }
+        const uint32_t over = max(L.w, L.wlim) - L.wlim;          // a full list counts on, writing past its end
+        L.lost += over;
+        L.w -= over;
+    }
 }
 
-__global__ void __launch_bounds__(TILE) k_build_cw(Arrays A, Scal S, int cur)
+// The column of one atom entry by entry, for a unit in which a list overflowed: the criterion on
+// every atom of the 27 cells, in the same order.
+template <int MODE>
+__device__ __noinline__ int build_column(const void* pos, const Rep* Rp, const int32_t* cs, const int32_t* perm,
+                                         uint32_t* W, int64_t nslots, int cap, double rl2d, float rl2f, int half, int me,
+                                         uint32_t pc)
 {
+    const Rep& R = *Rp;
+    int c[3];
+    unpack_cell(pc, c[0], c[1], c[2]);
+    int m = 0;
+    for (int oz = -1; oz <= 1; ++oz)
+        for (int oy = -1; oy <= 1; ++oy)
+            for (int ox = -1; ox <= 1; ++ox) {
+                int n[3] = {c[0] + ox, c[1] + oy, c[2] + oz};
+                const int sx = (n[0] < 0) ? -R.nc[0] : ((n[0] >= R.nc[0]) ? R.nc[0] : 0);
+                for (int q = 0; q < 3; ++q) { n[q] += (n[q] < 0) ? R.nc[q] : 0; n[q] -= (n[q] >= R.nc[q]) ? R.nc[q] : 0; }
+                const int g = cell_index(R, n[0], n[1], n[2]);
+                for (int k = cs[g]; k < cs[g + 1]; ++k) {
+                    const int j = perm[k];
+                    if (half ? j <= me : j == me) continue;
+                    if (criterion<MODE>(pos, Rp, rl2d, rl2f, me, j, sx, oy, oz) >= 0.0f) continue;
+                    if (m < cap)
+                        W[int64_t(m) * nslots + me] =
+                            (uint32_t(j) << IDX_SHIFT) | uint32_t(ox + 1) | (uint32_t(oy + 1) << 2) | (uint32_t(oz + 1) << 4);
+                    ++m;
+                }
+            }
+    return m;
+}
+
+template <int MODE, bool HALF, int MINB>
+__global__ void __launch_bounds__(TILE, MINB) k_build_group(Arrays A, Scal S, int cur, int rows)
+{
+    extern __shared__ uint32_t s_list[];              // [warps][rows + BG_STEP][32]
     if (!A.g->any_rebuild) return;
-    __shared__ float4 s_p[CW_WARPS][2][CW_ROW];
-    const float4* __restrict__ ps = A.psort;
-    const float rl2 = S.rl2f;
-    const float skip2 = rl2 * (1.0f + 1e-5f);
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const uint32_t* const my_lists = s_list + wl * (rows + BG_STEP) * 32;
+    const int a = lane % BG_ATOMS, pl = lane / BG_ATOMS;          // atom of the unit, z plane (3: idle lane)
+    const float4* __restrict__ ps = A.psort;
+    const int32_t* __restrict__ cs = A.cstart;
+    const void* const pos = (MODE == MD_FP64) ? static_cast<const void*>(A.pos64[cur]) : static_cast<const void*>(A.pos32[cur]);
+    const int nunits = A.g->n_rb_tiles * BG_UNITS;
+    const int wpc = blockDim.x >> 5, nw = gridDim.x * wpc;
+    ScanLane L;
+    L.wlim = smem_u32(my_lists + lane) + uint32_t(rows) * BG_ROW;
     int run_r = -1, run_max = 0;
     long long run_sum = 0;
-    // cells in chunks of 2 dealt to the warps in turn (as build_tile does for tiles)
-    for (int q = 0;; ++q) {
-        const int c = ((q >> 1) * nw + gw) * 2 + (q & 1);
-        if (c >= S.ncells) break;
-        const int r = A.cell_rep[c];
-        if (r != run_r) {
-            if (run_r >= 0) {
-                const long long ws = warp_sum_ll(run_sum);
-                const int wm = warp_max_i(run_max);
-                if (lane == 0) {
-                    if (ws) atomicAdd(reinterpret_cast<unsigned long long*>(&A.rs[run_r].sum_nbrs),
-                                      static_cast<unsigned long long>(ws));
-                    if (wm > 0) atomicMax(&A.rs[run_r].max_nbrs, wm);
-                }
-            }
-            run_r = r;
-            run_sum = 0;
-            run_max = 0;
-        }
-        if (!A.rs[r].rebuild) continue;
-        const Rep& R = A.rep[r];
-        const int cl = c - R.cell0;
-        int cx, cy, cz;
-        cell_coords(R, cl, cx, cy, cz);
-        const int xs[3] = {(cx == 0) ? R.nc[0] - 1 : cx - 1, cx, (cx == R.nc[0] - 1) ? 0 : cx + 1};
-        const float w0 = R.wf[0], w1 = R.wf[1], w2 = R.wf[2];
-        const int ab = A.cstart[c], ae = A.cstart[c + 1];
-        for (int a0 = ab; a0 < ae; a0 += 32) {
-            const bool have = a0 + lane < ae;
-            const float4 pi = have ? ps[a0 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
-            const int i = have ? __float_as_int(pi.w) : -1;
-            const float dl[3] = {pi.x * pi.x, pi.y * pi.y, pi.z * pi.z};
-            const float dh[3] = {(w0 - pi.x) * (w0 - pi.x), (w1 - pi.y) * (w1 - pi.y), (w2 - pi.z) * (w2 - pi.z)};
-            int m = 0;
-            uint32_t* wp = A.W + (have ? i : 0);
-            // the 9 rows (oy, oz) and their cells, with the ones no lane can reach removed
-            auto row_of = [&](int rr, CwRow& Q) {
-                const int oy = rr % 3 - 1, oz = rr / 3 - 1;
-                int ny = cy + oy; ny += (ny < 0) ? R.nc[1] : 0; ny -= (ny >= R.nc[1]) ? R.nc[1] : 0;
-                int nz = cz + oz; nz += (nz < 0) ? R.nc[2] : 0; nz -= (nz >= R.nc[2]) ? R.nc[2] : 0;
-                const float dyz = ((oy < 0) ? dl[1] : ((oy > 0) ? dh[1] : 0.f)) + ((oz < 0) ? dl[2] : ((oz > 0) ? dh[2] : 0.f));
-                const int rowc = R.cell0 + row_pos(R, ny, nz) * R.nc[0];
-                Q.tot = 0;
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const float dd = dyz + ((k == 0) ? dl[0] : ((k == 2) ? dh[0] : 0.f));
-                    const bool need = __any_sync(0xffffffffu, have && dd <= skip2);
-                    const int gc = rowc + xs[k];
-                    Q.b[k] = A.cstart[gc];
-                    Q.n[k] = need ? A.cstart[gc + 1] - Q.b[k] : 0;
-                    Q.tot += Q.n[k];
-                }
-            };
-            CwRow cur_row, nxt_row;
-            float4 rp[CW_PER_LANE];                 // a candidate's slot is in .w
-            auto load_regs = [&](const CwRow& Q, int q0) {
-#pragma unroll
-                for (int u = 0; u < CW_PER_LANE; ++u) {
-                    const int q = q0 + lane + 32 * u;
-                    if (q < Q.tot) rp[u] = ps[cw_index(Q, q)];
-                }
-            };
-            auto store_regs = [&](const CwRow& Q, int q0, int buf) {
-#pragma unroll
-                for (int u = 0; u < CW_PER_LANE; ++u) {
-                    const int q = lane + 32 * u;
-                    if (q0 + q < Q.tot) s_p[wl][buf][q] = rp[u];
-                }
-            };
-            auto test_row = [&](const CwRow& Q, int q0, int buf, int rr) {
-                const int oy = rr % 3 - 1, oz = rr / 3 - 1;
-                const float offy = float(oy) * w1, offz = float(oz) * w2;
-                const uint32_t codeyz = (uint32_t(oy + 1) << 2) | (uint32_t(oz + 1) << 4);
-                const int qend = min(Q.tot, q0 + CW_ROW);
-                int seg_end = 0;
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const int seg_beg = seg_end;
-                    seg_end += Q.n[k];
-                    const int lo = max(seg_beg, q0), hi = min(seg_end, qend);
-                    const float offx = float(k - 1) * w0;
-                    const uint32_t code = codeyz | uint32_t(k);
-                    for (int q = lo; q < hi; ++q) {
-                        const float4 pj = s_p[wl][buf][q - q0];
-                        const int j = __float_as_int(pj.w);
-                        const float dx = __fadd_rn(__fsub_rn(pj.x, pi.x), offx);
-                        const float dy = __fadd_rn(__fsub_rn(pj.y, pi.y), offy);
-                        const float dz = __fadd_rn(__fsub_rn(pj.z, pi.z), offz);
-                        const float r2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
-                        if (have && r2 < rl2 && (S.half_list ? j > i : j != i)) {
-                            if (m < S.cap) {
-                                *wp = (uint32_t(j) << IDX_SHIFT) | code;
-                                wp += S.nslots;
-                            }
-                            ++m;
-                        }
-                    }
-                }
-            };
-            // software pipeline over the rows: stage row rr+1 while testing row rr
-            int buf = 0;
-            row_of(0, cur_row);
-            load_regs(cur_row, 0);
-            store_regs(cur_row, 0, buf);
-            __syncwarp();
-            for (int rr = 0; rr < 9; ++rr) {
-                // rows longer than the staging buffer are walked in chunks without overlap
-                for (int q0 = CW_ROW; q0 < cur_row.tot; q0 += CW_ROW) {
-                    test_row(cur_row, q0 - CW_ROW, buf, rr);
-                    __syncwarp();
-                    load_regs(cur_row, q0);
-                    store_regs(cur_row, q0, buf);
-                    __syncwarp();
-                }
-                const int qlast = (cur_row.tot > 0) ? ((cur_row.tot - 1) / CW_ROW) * CW_ROW : 0;
-                if (rr + 1 < 9) {
-                    row_of(rr + 1, nxt_row);
-                    load_regs(nxt_row, 0);
-                }
-                test_row(cur_row, qlast, buf, rr);
-                if (rr + 1 < 9) {
-                    store_regs(nxt_row, 0, buf ^ 1);
-                    __syncwarp();
-                    buf ^= 1;
-                    cur_row = nxt_row;
-                }
-            }
-            __syncwarp();
-            if (have) {
-                A.nbr_count[i] = m;
-                if (S.rule == MD_REBUILD_DISP) A.xref[i] = make_float4(pi.x, pi.y, pi.z, 0.0f);
-                if (m > S.cap) {
-                    atomicOr(&A.g->err, ERR_NBR_OVERFLOW);
-                    atomicMax(&A.g->max_nbr_seen, m);
-                }
-                run_sum += m;
-                run_max = max(run_max, m);
-            }
-        }
-    }
-    if (run_r >= 0) {
+    auto flush_warp = [&]() {
         const long long ws = warp_sum_ll(run_sum);
         const int wm = warp_max_i(run_max);
         if (lane == 0) {
             if (ws) atomicAdd(reinterpret_cast<unsigned long long*>(&A.rs[run_r].sum_nbrs), static_cast<unsigned long long>(ws));
             if (wm > 0) atomicMax(&A.rs[run_r].max_nbrs, wm);
         }
+    };
+    for (int uid = blockIdx.x * wpc + wl; uid < nunits; uid += nw) {
+        const int it = uid / BG_UNITS, u = uid - it * BG_UNITS;
+        const int t = A.rb_tiles[it];
+        const int r = A.tile_rep[t];
+        const Rep& R = A.rep[r];
+        const int j0 = (t - R.tile0) * TILE + u * BG_ATOMS;
+        const int na = min(min(BG_ATOMS, TILE - u * BG_ATOMS), R.n - j0);
+        if (na <= 0) continue;
+        if (r != run_r) {
+            if (run_r >= 0) flush_warp();
+            run_r = r;
+            run_sum = 0;
+            run_max = 0;
+        }
+        const bool act = pl < 3 && a < na;
+        const int k = cs[R.cell0] + j0 + min(a, na - 1);
+        const uint32_t pc = A.pcell[k];
+        int cx, cy, cz;
+        unpack_cell(pc, cx, cy, cz);
+        const int ncx = R.nc[0], ncy = R.nc[1], ncz = R.nc[2];
+        float X, Y, Z;
+        {
+            const int prow = row_pos(R, cy, cz);
+            const int rs = cs[R.cell0 + prow * ncx];
+            const int P = cand_place(R, prow, rs) + (k - rs);
+            const float* f = reinterpret_cast<const float*>(ps) + 8 * (P >> 1) + (P & 1);
+            X = f[0];
+            Y = f[2];
+            Z = f[4];
+            L.self = __float_as_uint(f[6]);
+        }
+        const int xlo = cx - 1, xhi = cx + 1;
+        const int oz = pl - 1;
+        int nz = cz + oz;
+        float wz = 0.0f;                              // shift of the atom into the frame of wrapped cells
+        if (nz < 0) { nz += ncz; wz = float(ncz) * R.wf[2]; }
+        else if (nz >= ncz) { nz -= ncz; wz = -float(ncz) * R.wf[2]; }
+        L.nz = make_float2(-(Z + wz), -(Z + wz));
+        L.w = L.wlim - uint32_t(rows) * BG_ROW;
+        L.lost = 0;
+        const bool any_lo = __any_sync(0xffffffffu, act && xlo < 0), any_hi = __any_sync(0xffffffffu, act && xhi >= ncx);
+#pragma unroll 1
+        for (int oy = -1; oy <= 1; ++oy) {
+            int ny = cy + oy;
+            float wy = 0.0f;
+            if (ny < 0) { ny += ncy; wy = float(ncy) * R.wf[1]; }
+            else if (ny >= ncy) { ny -= ncy; wy = -float(ncy) * R.wf[1]; }
+            L.ny = make_float2(-(Y + wy), -(Y + wy));
+            const float bandw = (wy != 0.0f || wz != 0.0f) ? 4.0f * R.band : R.band;
+            const uint32_t code = (uint32_t(oy + 1) << 2) | (uint32_t(oz + 1) << 4);
+            const int prow = row_pos(R, ny, nz < ncz ? nz : 0);
+            const int row = R.cell0 + prow * ncx;
+            const int rs = cs[row];
+            const int base = cand_place(R, prow, rs);
+            if (any_lo) {
+                const float xs = X + float(ncx) * R.wf[0];
+                L.nx = make_float2(-xs, -xs);
+                L.band = 4.0f * R.band;
+                const int P0 = base + ((cs[row + ncx - 1] - rs) & ~3);
+                const int P1 = (act && xlo < 0) ? base + ((cs[row + ncx] - rs + 3) & ~3) : P0;
+                scan_run<MODE, HALF, true, true>(ps, P0, P1, L, S.rl2f, S.rl2d, code, uint32_t(-ncx) & 3u, pos, &R, -ncx, oy, oz);
+            }
+            {
+                L.nx = make_float2(-X, -X);
+                L.band = bandw;
+                const int P0 = base + ((cs[row + max(xlo, 0)] - rs) & ~3);
+                const int P1 = act ? base + ((cs[row + min(xhi, ncx - 1) + 1] - rs + 3) & ~3) : P0;
+                if (oy == 0) scan_run<MODE, HALF, true, false>(ps, P0, P1, L, S.rl2f, S.rl2d, code, 0u, pos, &R, 0, oy, oz);
+                else scan_run<MODE, HALF, false, false>(ps, P0, P1, L, S.rl2f, S.rl2d, code, 0u, pos, &R, 0, oy, oz);
+            }
+            if (any_hi) {
+                const float xs = X - float(ncx) * R.wf[0];
+                L.nx = make_float2(-xs, -xs);
+                L.band = 4.0f * R.band;
+                const int P0 = base;
+                const int P1 = (act && xhi >= ncx) ? base + ((cs[row + 1] - rs + 3) & ~3) : P0;
+                scan_run<MODE, HALF, true, true>(ps, P0, P1, L, S.rl2f, S.rl2d, code, uint32_t(ncx) & 3u, pos, &R, ncx, oy, oz);
+            }
+        }
+        // join the planes: entry m of atom a comes from plane 0, 1 or 2
+        const int cnt = int((L.w - (L.wlim - uint32_t(rows) * BG_ROW) + L.lost) / BG_ROW);
+        __syncwarp();
+        const int c0 = __shfl_sync(0xffffffffu, cnt, a), c1 = __shfl_sync(0xffffffffu, cnt, a + BG_ATOMS);
+        const int c2 = __shfl_sync(0xffffffffu, cnt, a + 2 * BG_ATOMS);
+        int m = c0 + c1 + c2;
+        const int slot = int(L.self >> IDX_SHIFT);
+        const uint32_t cadd = uint32_t(1 - cx) & 3u;              // o_x + 1 = cell of j - cell of i + 1 (mod 4)
+        if (rows < S.cap && __any_sync(0xffffffffu, act && L.lost != 0)) {
+            if (act && pl == 0)
+                m = build_column<MODE>(pos, &R, cs, A.perm, A.W, S.nslots, S.cap, S.rl2d, S.rl2f, HALF ? 1 : 0, slot, pc);
+        } else if (act) {
+            const int mc = min(m, S.cap);
+            uint32_t* wp = A.W + int64_t(pl) * S.nslots + slot;
+            for (int q = pl; q < mc; q += 3, wp += 3 * S.nslots) {
+                const int src = (q < c0) ? q * 32 + a
+                                         : ((q < c0 + c1) ? (q - c0) * 32 + a + BG_ATOMS : (q - c0 - c1) * 32 + a + 2 * BG_ATOMS);
+                const uint32_t v = my_lists[src];
+                *wp = (v & ~3u) | ((v + cadd) & 3u);
+            }
+        }
+        __syncwarp();
+        if (act && pl == 0) {
+            A.nbr_count[slot] = m;
+            if (S.rule == MD_REBUILD_DISP) {
+                if constexpr (MODE == MD_FP64) {
+                    const double4_32a p = A.pos64[cur][slot];
+                    A.xref[slot] = make_float4(float(p.x), float(p.y), float(p.z), 0.0f);
+                } else {
+                    const float4 p = A.pos32[cur][slot];
+                    A.xref[slot] = make_float4(p.x, p.y, p.z, 0.0f);
+                }
+            }
+            if (m > S.cap) {
+                atomicOr(&A.g->err, ERR_NBR_OVERFLOW);
+                atomicMax(&A.g->max_nbr_seen, m);
+            }
+            run_sum += m;
+            run_max = max(run_max, m);
+        }
     }
+    if (run_r >= 0) flush_warp();
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1367,11 +971,9 @@ void prime_rebuild_grids(const Scal& S, const Launch& L)
     (void)resident_grid<k_bin<MD_MIXED>>(S, L);
     (void)resident_grid<k_bin<MD_FP32>>(S, L);
     (void)resident_grid<k_scatter>(S, L);
-    (void)resident_grid<k_build_sorted<2, false>>(S, L);
-    (void)resident_grid<k_build_sorted<4, false>>(S, L);
-    (void)resident_grid<k_build_sub<2, false>>(S, L);
-    (void)resident_grid<k_sub_bin>(S, L);
-    (void)resident_grid<k_sub_scatter>(S, L);
+    (void)resident_grid<k_order<MD_FP64>>(S, L);
+    (void)resident_grid<k_order<MD_MIXED>>(S, L);
+    (void)resident_grid<k_order<MD_FP32>>(S, L);
     (void)resident_grid<k_reorder_gather<MD_FP64>>(S, L);
     (void)resident_grid<k_reorder_gather<MD_MIXED>>(S, L);
     (void)resident_grid<k_reorder_gather<MD_FP32>>(S, L);
@@ -1395,8 +997,13 @@ cudaError_t launch_bin_order(const Arrays& A, const Scal& S, const Launch& L, in
     else k_bin<MD_FP32><<<resident_grid<k_bin<MD_FP32>>(S, L), TILE, 0, L.stream>>>(A, S, cur, fs);
     launch_scan(A, ScanArgs{A.ccount, A.cstart, A.chunk, S.ncells, S.nchunks}, L.stream);
     k_scatter<<<resident_grid<k_scatter>(S, L), TILE, 0, L.stream>>>(A, S);
-    const int gs = int(std::min<int64_t>((S.ncells + 255) / 256, int64_t(L.grid) * 8));
-    k_sort_cells<<<std::max(gs, 1), 256, 0, L.stream>>>(A, S, cur);
+    if (S.mode == MD_FP64) k_order<MD_FP64><<<resident_grid<k_order<MD_FP64>>(S, L), TILE, 0, L.stream>>>(A, S, cur);
+    else if (S.mode == MD_MIXED) k_order<MD_MIXED><<<resident_grid<k_order<MD_MIXED>>(S, L), TILE, 0, L.stream>>>(A, S, cur);
+    else k_order<MD_FP32><<<resident_grid<k_order<MD_FP32>>(S, L), TILE, 0, L.stream>>>(A, S, cur);
+    if (L.step_kernel == 4) {
+        const int gs = int(std::min<int64_t>((S.ncells + 255) / 256, int64_t(L.grid) * 8));
+        k_cell_ranges<<<std::max(gs, 1), 256, 0, L.stream>>>(A, S);
+    }
     return cudaGetLastError();
 }
 
@@ -1425,58 +1032,64 @@ cudaError_t launch_bin_only(const Arrays& A, const Scal& S, const Launch& L, int
 // displacement rule needs the positions at the rebuild (written by the build)
 static bool skip_w(const Scal& S, const Launch& L) { return L.step_kernel == 4 && S.rule != MD_REBUILD_DISP; }
 
-int build_kernels(const Scal& S, const Launch& L) { return skip_w(S, L) ? 2 : (L.build_batch == 1 ? 9 : 3); }
+int bin_kernels(const Scal&, const Launch& L) { return L.step_kernel == 4 ? 8 : 7; }
 
-// Grid of a staged build kernel: every CTA resident with `smem` bytes of columns each (the
-// occupancy is looked up again when the size changes)
-template <auto Kernel>
-static int staged_grid(const Scal& S, const Launch& L, int smem)
+int build_kernels(const Scal& S, const Launch& L) { return (skip_w(S, L) ? 0 : 1) + (L.step_kernel == 3 ? 1 : 0) + 1; }
+
+// The register bound: 8 CTAs per SM where the lists leave room for them (WCA, 2M atoms: 0.51 against
+// 0.59 ms at the 5 CTAs' bound), else 5, which the LJ lists allow and which spills nothing there.
+// The lists of k_build_group hold one z plane's neighbours of an atom.  A slab of thickness w >= r_l
+// around it holds up to 69 % of them; half as many again and 12 leave room for fluctuations, and
+// 60 % of the capacity for denser regions than the mean.  A longer list sends its unit through
+// build_column.  Four warps per CTA while their lists fit, else one.
+template <int MODE, bool HALF, int MINB>
+static void group_grid(Launch& L)
 {
-    static int last_smem = -1, per_sm = 0;
-    if (smem != last_smem) {
-        int dev = 0, optin = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, std::min(optin, smem));
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, Kernel, TILE, smem) != cudaSuccess) per_sm = 1;
-        last_smem = smem;
-    }
-    return std::max(1, std::min(L.nsm * std::max(per_sm, 1), S.ntiles));
+    int optin = 0, dev = 0, per_sm = 1;
+    cudaFuncAttributes fa;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (cudaFuncGetAttributes(&fa, k_build_group<MODE, HALF, MINB>) == cudaSuccess)
+        cudaFuncSetAttribute(k_build_group<MODE, HALF, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             optin - int(fa.sharedSizeBytes));
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_build_group<MODE, HALF, MINB>, L.bg_block, L.bg_smem) !=
+        cudaSuccess)
+        per_sm = 1;
+    L.bg_grid = L.nsm * std::max(1, per_sm);
 }
 
-// staging the columns needs cap x TILE x 4 bytes per CTA: at most 160 KB (cap <= 320)
-static bool stage_w(const Scal& S, const Launch& L) { return L.build_stage && S.cap * TILE * 4 <= 160 * 1024; }
+// F(MODE, HALF, MINB) for the system's precision, list and list length
+#define GBMD_BUILD_MINB(M, H, F) { if (L.bg_minb == 8) F(M, H, 8); else F(M, H, 5); }
+#define GBMD_BUILD_DISPATCH(F)                                                                          \
+    if (S.mode == MD_FP64) GBMD_BUILD_MINB(MD_FP64, false, F)                                           \
+    else if (S.mode == MD_MIXED) { if (S.half_list) GBMD_BUILD_MINB(MD_MIXED, true, F) else GBMD_BUILD_MINB(MD_MIXED, false, F) } \
+    else { if (S.half_list) GBMD_BUILD_MINB(MD_FP32, true, F) else GBMD_BUILD_MINB(MD_FP32, false, F) }
+
+void build_group_shape(const Scal& S, Launch& L, double mean_nbrs, int smem_per_cta, int smem_per_sm)
+{
+    const int room = smem_per_cta - 2048;
+    const double want = std::max(0.69 * 1.35 * mean_nbrs + 12.0, 0.6 * S.cap);
+    int rows = std::min(S.cap, int(std::min(want, 1.0e6)) + 1);
+    L.bg_block = ((rows + BG_STEP) * int(BG_ROW) * (TILE / 32) <= room) ? TILE : 32;
+    rows = std::min(rows, room / (int(BG_ROW) * (L.bg_block / 32)) - BG_STEP);
+    L.bg_rows = rows;
+    L.bg_smem = (rows + BG_STEP) * int(BG_ROW) * (L.bg_block / 32);
+    L.bg_minb = (8 * (L.bg_smem + 1024) <= smem_per_sm && L.bg_block == TILE) ? 8 : 5;
+#define GBMD_GRID(M, H, B) group_grid<M, H, B>(L)
+    GBMD_BUILD_DISPATCH(GBMD_GRID)
+#undef GBMD_GRID
+}
 
 cudaError_t launch_build_only(const Arrays& A, const Scal& S, const Launch& L, int cur)
 {
-    const int g = tile_grid(S, L);
-    if (S.mode == MD_FP64) k_build<double, 1><<<g, TILE, 0, L.stream>>>(A, S, cur);
-    else if (skip_w(S, L)) {
-    } else if (L.build_batch == 1) {
-        k_sub_bin<<<resident_grid<k_sub_bin>(S, L), TILE, 0, L.stream>>>(A, S, cur);
-        launch_scan(A, ScanArgs{A.scount, A.sstart, A.schunk, S.nsub, S.nschunks}, L.stream);
-        k_sub_scatter<<<resident_grid<k_sub_scatter>(S, L), TILE, 0, L.stream>>>(A, S, cur);
-        const int gs = int(std::min<int64_t>((S.nsub + 255) / 256, int64_t(L.grid) * 8));
-        k_sub_sort<<<std::max(gs, 1), 256, 0, L.stream>>>(A, S);
-        if (stage_w(S, L)) {
-            const int sm = S.cap * TILE * 4;
-            k_build_sub<2, true><<<staged_grid<k_build_sub<2, true>>(S, L, sm), TILE, sm, L.stream>>>(A, S, cur);
-        } else {
-            k_build_sub<2, false><<<resident_grid<k_build_sub<2, false>>(S, L), TILE, 0, L.stream>>>(A, S, cur);
-        }
+    if (!skip_w(S, L)) {
+        const int64_t units = int64_t(S.ntiles) * BG_UNITS, per_cta = L.bg_block / 32;
+        const int g = int(std::max<int64_t>(1, std::min<int64_t>(L.bg_grid, (units + per_cta - 1) / per_cta)));
+#define GBMD_BUILD(M, H, B) k_build_group<M, H, B><<<g, L.bg_block, L.bg_smem, L.stream>>>(A, S, cur, L.bg_rows)
+        GBMD_BUILD_DISPATCH(GBMD_BUILD)
+#undef GBMD_BUILD
     }
-    else if (L.build_batch >= 32) k_build_cw<<<std::max(1, L.grid), TILE, 0, L.stream>>>(A, S, cur);
-    else if (stage_w(S, L)) {
-        const int sm = S.cap * TILE * 4;
-        if (L.build_batch >= 4)
-            k_build_sorted<4, true><<<staged_grid<k_build_sorted<4, true>>(S, L, sm), TILE, sm, L.stream>>>(A, S, cur);
-        else
-            k_build_sorted<2, true><<<staged_grid<k_build_sorted<2, true>>(S, L, sm), TILE, sm, L.stream>>>(A, S, cur);
-    }
-    else if (L.build_batch >= 4)
-        k_build_sorted<4, false><<<resident_grid<k_build_sorted<4, false>>(S, L), TILE, 0, L.stream>>>(A, S, cur);
-    else k_build_sorted<2, false><<<resident_grid<k_build_sorted<2, false>>(S, L), TILE, 0, L.stream>>>(A, S, cur);
-    k_tile_windows<<<g, TILE, 0, L.stream>>>(A, S, cur, L.step_kernel == 3 ? 1 : 0);   // used by step kernel 3
+    if (L.step_kernel == 3) k_tile_windows<<<tile_grid(S, L), TILE, 0, L.stream>>>(A, S, cur, 1);
     k_rebuild_finish<<<1, 256, 0, L.stream>>>(A, S, L.in_graph);
     return cudaGetLastError();
 }

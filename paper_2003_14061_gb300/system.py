@@ -245,8 +245,8 @@ class MDSystem:
         """Launch shapes (0 keeps the current value); use_graph: 1 = CUDA graphs, 2 = direct;
         step_kernel: 1 = per-thread loads with L2 prefetch, 2 = bulk-copy shared-memory ring,
         3 = staged cell-row windows in shared memory, 4 = list-free (27 cells every step),
-        5 = half neighbour list with atomic reactions; build_stage: 1 = the build writes W rows
-        from shared memory, 2 = entry by entry; reorder_every: reorder by cell every that many
+        5 = half neighbour list with atomic reactions; build_batch and build_stage select the same
+        neighbour build for every accepted value; reorder_every: reorder by cell every that many
         steps (at a rebuild), -1 = at every rebuild."""
         t = B.md_tuning(int(ctas_per_sm), int(nbr_batch), int(build_batch), int(use_graph), int(step_kernel),
                         int(build_stage), int(reorder_every))

@@ -4,16 +4,16 @@ The paper found thread-block size to matter little on its GPU and warned that th
 elsewhere (Sec. 4.1 item 2).  On GB300 the residency of the fused step kernel and the number of
 neighbour-matrix loads each thread keeps in flight decide its speed, so they are measured on the
 system itself: every candidate advances the live system by a number of steps timed with CUDA
-events on the library's stream.  Step kernels 1-3 and builds 2, 4 and 32 perform the same
-arithmetic in the same order; the list-free step kernel (4) and the sub-cell build (1) sum each
-force in another order, and the half-list kernel (5) adds through atomics in no fixed order, so
-choosing them changes the trajectory at the rounding level only.
+events on the library's stream.  Step kernels 1-3 perform the same arithmetic in the same order;
+the list-free step kernel (4) sums each force in another order, and the half-list kernel (5) adds
+through atomics in no fixed order, so choosing them changes the trajectory at the rounding level
+only.
 
 Search: coordinate descent over (step kernel, ctas_per_sm, nbr_batch) for the step -- the
 per-thread kernel at register-bound residencies, the list-free and half-list kernels, and on
 request the shared-memory ring and the staged-neighbour kernel (2 and 3, slower on every measured
-workload) at the residencies their shared memory allows -- then build_batch and build_stage for
-the neighbour build, then the reorder policy (every 100 steps or at every rebuild: the paper's
+workload) at the residencies their shared memory allows -- then the accepted build_batch and
+build_stage values (one kernel serves them all), then the reorder policy (every 100 steps or at every rebuild: the paper's
 reorder, Sec. 4.1 item 1, is a trade between the reorder's cost and the locality it restores).
 
 Measurement: each candidate runs with direct launches and the library's per-phase CUDA events,
