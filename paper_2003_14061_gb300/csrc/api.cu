@@ -265,6 +265,7 @@ struct md_system {
     int64_t host_step = 0;
     bool binned_fresh = false;
     md_tuning tune;
+    bool shape_set = false;       // md_set_tuning has named ctas_per_sm or nbr_batch
     void* ws = nullptr;
     size_t ws_bytes = 0;
     // per-phase timers (CUDA events on the system's stream) and kernel-launch counts
@@ -457,9 +458,21 @@ int apply_tuning(md_system* s)
     bulk_shape(s->S, per_sm, s->smem_per_sm, s->smem_per_cta, &s->L.bulk_rows, &s->L.bulk_smem);
     stage_shape(per_sm, s->smem_per_sm, &s->L.stage_cap, &s->L.stage_smem);
     build_group_shape(s->S, s->L, s->plan.mean_nbrs, s->smem_per_cta, s->smem_per_sm);
-    s->L.ctas_req = per_sm;
+    // Step-kernel shape.  One that md_set_tuning never named is chosen by size: 4 CTAs per SM with 8
+    // W entries together (120 registers) up to 1.5M atoms and at 30 neighbours or more, else 8 CTAs
+    // and 2 entries, whose warps hide the HBM latency that the larger fluids wait for.  Step kernel,
+    // 4/8 against 8/2: LJ 256k atoms 59 / 71 us, 1M 176 / 198, 6.9M 1127 / 1158; WCA 108k 25 / 31,
+    // 1M 72 / 74 (with props 85 / 91), 4M 244 / 206.
+    const bool chosen = s->shape_set || s->L.step_kernel != 1;
+    const bool wide = !chosen && (s->plan.mean_nbrs >= 30.0 || s->plan.nslots <= 1500000);
+    const int step_ctas = wide ? 4 : per_sm;
+    if (wide) s->L.nbr_batch = 8;
+    // up to 16 warp-tiles per SM every warp-tile gets a warp of its own, one per CTA, so that they
+    // spread over all SMs and none claims or steals tiles
+    s->L.step_single = !chosen && s->plan.ntiles * (TILE / 32) <= s->nsm * 16;
+    s->L.ctas_req = step_ctas;
     // a persistent grid larger than what can be resident would run as a trailing second wave
-    s->L.grid_step = s->nsm * std::min(per_sm, step_ctas_per_sm(s->S, s->L));
+    s->L.grid_step = s->nsm * std::min(step_ctas, step_ctas_per_sm(s->S, s->L));
     return MD_OK;
 }
 
@@ -1137,6 +1150,7 @@ int md_set_tuning(md_system* s, const md_tuning* t)
     if (t->build_stage < 0 || t->build_stage > 2) return fail(MD_ERR_INVALID_ARG, "build_stage must be 0, 1 or 2");
     if (t->reorder_every < -1) return fail(MD_ERR_INVALID_ARG, "reorder_every must be >= -1");
     const int old_kernel = s->L.step_kernel;
+    if (t->ctas_per_sm || t->nbr_batch) s->shape_set = true;
     if (t->ctas_per_sm) s->tune.ctas_per_sm = t->ctas_per_sm;
     if (t->nbr_batch) s->tune.nbr_batch = t->nbr_batch;
     if (t->build_batch) s->tune.build_batch = t->build_batch;

@@ -421,6 +421,7 @@ struct Launch {
     int build_block;
     int nbr_batch;            // W entries loaded together per thread in the pair loop (2, 4, 8)
     int ctas_req;             // requested resident CTAs/SM (register bound of the step kernel)
+    int step_single;          // step kernel 1: one warp per CTA and warp-tile, all of them resident at once
     int bg_rows;              // k_build_group: rows of each lane's list in shared memory,
     int bg_block;             // threads per CTA, dynamic shared memory and CTAs
     int bg_smem;

@@ -19,6 +19,7 @@
 // Only replicas whose rebuild flag is set do work; kernels return at once when none is set, so
 // the whole sequence can sit in every step of md_integrate.
 #include <algorithm>
+#include <atomic>
 
 #include "gbmd_internal.cuh"
 
@@ -1045,17 +1046,30 @@ int build_kernels(const Scal& S, const Launch& L) { return (skip_w(S, L) ? 0 : 1
 template <int MODE, bool HALF, int MINB>
 static void group_grid(Launch& L)
 {
-    int optin = 0, dev = 0, per_sm = 1;
-    cudaFuncAttributes fa;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (cudaFuncGetAttributes(&fa, k_build_group<MODE, HALF, MINB>) == cudaSuccess)
-        cudaFuncSetAttribute(k_build_group<MODE, HALF, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             optin - int(fa.sharedSizeBytes));
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_build_group<MODE, HALF, MINB>, L.bg_block, L.bg_smem) !=
-        cudaSuccess)
-        per_sm = 1;
-    L.bg_grid = L.nsm * std::max(1, per_sm);
+    // the opt-in limit once per kernel, the occupancy again when the shared memory changes
+    static const bool raised = [] {
+        int optin = 0, dev = 0;
+        cudaFuncAttributes fa;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        return cudaFuncGetAttributes(&fa, k_build_group<MODE, HALF, MINB>) == cudaSuccess &&
+               cudaFuncSetAttribute(k_build_group<MODE, HALF, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    optin - int(fa.sharedSizeBytes)) == cudaSuccess;
+    }();
+    (void)raised;
+    static std::atomic<uint64_t> known{0};            // (shared memory, block) << 32 | CTAs per SM
+    const uint64_t key = uint64_t(uint32_t(L.bg_smem) | (L.bg_block == TILE ? 0x80000000u : 0u)) << 32;
+    const uint64_t seen = known.load(std::memory_order_relaxed);
+    int per_sm = 1;
+    if ((seen & 0xffffffff00000000ull) == key && uint32_t(seen) != 0) {
+        per_sm = int(uint32_t(seen));
+    } else {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_build_group<MODE, HALF, MINB>, L.bg_block, L.bg_smem) !=
+                cudaSuccess || per_sm < 1)
+            per_sm = 1;
+        known.store(key | uint32_t(per_sm), std::memory_order_relaxed);
+    }
+    L.bg_grid = L.nsm * per_sm;
 }
 
 // F(MODE, HALF, MINB) for the system's precision, list and list length

@@ -1,24 +1,23 @@
 // kernels_step.cu -- per-step kernels: fused force + leapfrog, standalone forces, reductions,
 // and the id-ordered state exchange.
 //
-//   k_step     F1 (Sec. 2.3) fused with the leapfrog update (Sec. 4.3 item 1).  One thread per
+//   k_step_sm  F1 (Sec. 2.3) fused with the leapfrog update (Sec. 4.3 item 1).  One thread per
 //              atom walks its column of W (coalesced rows, Sec. 4.1 item 6), gathers neighbour
 //              positions from the other position buffer, accumulates f_i without Newton's third
-//              law (Sec. 2.3), then kicks and drifts its own FP64 state and writes its next
-//              cell-local position.  Per tile, the maximum speed (or displacement) is reduced;
-//              the CTA that completes a replica's last tile (the "last block" pattern of
-//              Sec. 2.3, an atomic counter after a memory fence) updates the refresh criterion
-//              and raises the rebuild flag.  With PROPS, the step also forms F2 (U, K, virial,
-//              momentum): MD_FP64 tiles write FP64 partial sums for k_props_reduce; the MD_MIXED
-//              and MD_FP32 kernels add their warp sums in fixed point and the warp that completes
-//              a replica writes its props (no further launch).
-//   k_step_sm  the same for MD_MIXED and MD_FP32 (step kernel 1): warps take 32-slot warp-tiles
-//              from the slot range of the SM they run on, so the warps of an SM gather from one
-//              neighbourhood held in its L1.  k_step runs MD_FP64 and step kernel 3.
-//   k_step<..., STG = true>  the same with each tile's neighbour positions staged in shared
-//              memory by cp.async.bulk first (step kernel 3).
+//              law (Sec. 2.3), then kicks and drifts its own state and writes its next
+//              cell-local position.  Warps take 32-slot warp-tiles from the slot range of the SM
+//              they run on, so that the warps of an SM gather from one neighbourhood held in its
+//              L1; a system of few warp-tiles gives each a warp of its own.  The maximum speed
+//              (or displacement) is kept per warp; the warp that completes a replica's last
+//              warp-tile (the "last block" pattern of Sec. 2.3, an atomic counter after a memory
+//              fence) updates the refresh criterion and raises the rebuild flag.  With PROPS, the
+//              step also forms F2 (U, K, virial, momentum): MD_FP64 warps write FP64 partial sums
+//              for k_props_reduce; the MD_MIXED and MD_FP32 kernels add their warp sums in fixed
+//              point and the warp that completes a replica writes its props (no further launch).
+//   k_step     the same for MD_MIXED and MD_FP32 on 128-slot tiles per CTA with each tile's
+//              neighbour positions staged in shared memory by cp.async.bulk (step kernel 3).
 //   k_step_bulk  the same arithmetic with the tile's state and W rows in a two-stage shared-memory
-//              ring filled by cp.async.bulk (step kernel 2).  The four forms share the pair loop
+//              ring filled by cp.async.bulk (step kernel 2).  The three forms share the pair loop
 //              and the kick-drift, so they give bit-identical trajectories.
 //   k_forces   F1 alone: f_i, u_i and the per-atom virial at the current positions.
 //   k_props_*  F2 outside the step (and for MD_FP64 steps): per-warp FP64 partials, then CTA
@@ -538,28 +537,37 @@ __device__ __forceinline__ void prefetch_l2(const void* p)
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
+// FP64 pairs, NB entries at a time: their W rows, positions and pair terms are independent of each
+// other, the sums are added entry by entry in the column's order
+template <int NB>
 __device__ __forceinline__ AccD force_f64(const Arrays& A, const Scal& S, const Rep& R,
                                           const double4_32a* __restrict__ pos, int64_t slot, double4_32a pi)
 {
     AccD a{0.0, 0.0, 0.0, 0.0, 0.0};
     const int mm = min(A.nbr_count[slot], S.cap);
     const uint32_t* __restrict__ Wc = A.W + slot;
-    for (int m = 0; m < mm; ++m) {
-        const uint32_t e = Wc[int64_t(m) * S.nslots];
-        const double4_32a pj = pos[e >> IDX_SHIFT];
-        const double dx = fma(double(int(e & 3u) - 1), R.w[0], pj.x - pi.x);
-        const double dy = fma(double(int((e >> 2) & 3u) - 1), R.w[1], pj.y - pi.y);
-        const double dz = fma(double(int((e >> 4) & 3u) - 1), R.w[2], pj.z - pi.z);
-        const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-        if (r2 < S.rc2d) {
+    for (int m0 = 0; m0 < mm; m0 += NB) {
+        uint32_t e[NB];
+        double4_32a pj[NB];
+#pragma unroll
+        for (int k = 0; k < NB; ++k) e[k] = (m0 + k < mm) ? Wc[int64_t(m0 + k) * S.nslots] : 0u;
+#pragma unroll
+        for (int k = 0; k < NB; ++k) pj[k] = pos[e[k] >> IDX_SHIFT];
+#pragma unroll
+        for (int k = 0; k < NB; ++k) {
+            const double dx = fma(double(int(e[k] & 3u) - 1), R.w[0], pj[k].x - pi.x);
+            const double dy = fma(double(int((e[k] >> 2) & 3u) - 1), R.w[1], pj[k].y - pi.y);
+            const double dz = fma(double(int((e[k] >> 4) & 3u) - 1), R.w[2], pj[k].z - pi.z);
+            const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+            const bool in = m0 + k < mm && r2 < S.rc2d;
             const double ri2 = 1.0 / r2;
             const double sr2 = S.sig2d * ri2;
             const double sr6 = sr2 * sr2 * sr2;
-            const double fs = S.eps48d * sr6 * (sr6 - 0.5) * ri2;
+            const double fs = in ? S.eps48d * sr6 * (sr6 - 0.5) * ri2 : 0.0;
             a.fx -= fs * dx;
             a.fy -= fs * dy;
             a.fz -= fs * dz;
-            a.u += S.eps4d * sr6 * (sr6 - 1.0) - S.ucd;
+            a.u += in ? S.eps4d * sr6 * (sr6 - 1.0) - S.ucd : 0.0;
             a.w += fs * r2;
         }
     }
@@ -743,17 +751,6 @@ __device__ __forceinline__ void props_warp_flush_sh(const Arrays& A, int r, long
     __threadfence();
 }
 
-// one warp-tile's props: FP64 lanes (MD_FP64) store the warp's partials for k_props_reduce, FP32
-// lanes add them to the warp's fixed-point sums
-__device__ __forceinline__ void props_take(const Arrays&, int, double (&p)[NPROP], PropsAcc&, double* dst)
-{
-    warp_partials_store(p, dst);
-}
-__device__ __forceinline__ void props_take(const Arrays& A, int r, float (&p)[NPROP], PropsAcc& pa, double*)
-{
-    props_warp_add(A, r, p, pa);
-}
-
 // Refresh criterion and step bookkeeping, run by one thread of the CTA that completed the last
 // tile of replica r in this launch.  With props (fixed-point path), first the props of the step.
 __device__ void finish_replica_step(const Arrays& A, const Scal& S, int r, cudaGraphConditionalHandle cond,
@@ -835,6 +832,7 @@ template <int MODE, bool PROPS, int NB, int MINB, bool STG>
 __global__ void __launch_bounds__(TILE, MINB) k_step(Arrays A, Scal S, int cur, cudaGraphConditionalHandle cond,
                                                  int use_cond, int stage_cap)
 {
+    static_assert(MODE != MD_FP64 && STG, "other steps run k_step_sm");
     __shared__ float sh_max[TILE / 32];
     extern __shared__ __align__(16) float4 s_nb[];       // STG: staged neighbour positions
     __shared__ int4 sh_win[16];          // STG: per (o_y+1) + 4 (o_z+1): first slot, length, s_nb offset
@@ -858,16 +856,16 @@ __global__ void __launch_bounds__(TILE, MINB) k_step(Arrays A, Scal S, int cur, 
     const int t_begin = blockIdx.x * per;
     const int t_end = min(S.ntiles, t_begin + per);
     int c_ahead = 0;
-    if (MODE != MD_FP64 && t_begin + 1 < t_end)
+    if (t_begin + 1 < t_end)
         c_ahead = __ldcs(A.nbr_count + int64_t(t_begin + 1) * TILE + threadIdx.x);
     // the refresh metric is kept per thread across this CTA's tiles of one replica and folded
     // into the replica's counters once per replica (one fence per CTA, not per tile)
     int run_r = -1, run_tiles = 0;
     float run_max = 0.0f;
     PropsAcc pa{0, 0.0f};
-    PropsAcc* const pfix = (PROPS && MODE != MD_FP64) ? &pa : nullptr;
+    PropsAcc* const pfix = PROPS ? &pa : nullptr;
     for (int t = t_begin; t < t_end; ++t) {
-        if (MODE != MD_FP64) {
+        {
             if (t + 1 < t_end) {
                 // one prefetch per 128-byte line, spread over the warp's lanes: the warp's 32
                 // slots span 4 lines of positions, 2 lines of each FP64 stream (1 of each FP32
@@ -943,49 +941,11 @@ __global__ void __launch_bounds__(TILE, MINB) k_step(Arrays A, Scal S, int cur, 
             }
         }
         float metric = 0.0f;                     // |v|^2 (VMAX) or |x - x_ref|^2 (DISP)
-        using PT = typename std::conditional<MODE == MD_FP64, double, float>::type;
-        PT part[NPROP];
+        float part[NPROP];
 #pragma unroll
-        for (int q = 0; q < NPROP; ++q) part[q] = PT(0);
+        for (int q = 0; q < NPROP; ++q) part[q] = 0.0f;
         if (active) {
-            if constexpr (MODE == MD_FP64) {
-                const double4_32a* pos = A.pos64[cur];
-                const double4_32a pi = pos[slot];
-                const AccD a = force_f64(A, S, R, pos, slot, pi);
-                const double f[3] = {a.fx, a.fy, a.fz};
-                double xl[3] = {pi.x, pi.y, pi.z};
-                const double kick = vhalf ? 2.0 * S.c : S.c;
-                double vn2 = 0.0;
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    double v = A.v[q][slot];
-                    if (PROPS) {
-                        const double vn = vhalf ? fma(S.c, f[q], v) : v;
-                        vn2 = fma(vn, vn, vn2);
-                        part[3 + q] = vn;
-                    }
-                    v = fma(kick, f[q], v);
-                    xl[q] = fma(S.dt, v, xl[q]);
-                    A.v[q][slot] = v;
-                    A.xl[q][slot] = xl[q];
-                }
-                A.pos64[nxt][slot] = make_double4_32a(xl[0], xl[1], xl[2], pi.w);
-                if (S.rule == MD_REBUILD_DISP) {
-                    const float4 xr = A.xref[slot];
-                    const float d0 = float(xl[0] - double(xr.x)), d1 = float(xl[1] - double(xr.y)),
-                                d2 = float(xl[2] - double(xr.z));
-                    metric = d0 * d0 + d1 * d1 + d2 * d2;
-                } else {
-                    const double d0 = xl[0] - pi.x, d1 = xl[1] - pi.y, d2 = xl[2] - pi.z;
-                    metric = float(d0 * d0 + d1 * d1 + d2 * d2);
-                }
-                if (PROPS) {
-                    part[0] = a.u;
-                    part[1] = vn2;
-                    part[2] = a.w;
-                    part[NPROP - 1] = vn2;
-                }
-            } else {
+            {
                 const float4* pos = A.pos32[cur];
                 const float4 pi = __ldg(pos + slot);
                 if (t == t_begin) {                      // first tile of this CTA: nothing prefetched yet
@@ -1054,14 +1014,14 @@ __global__ void __launch_bounds__(TILE, MINB) k_step(Arrays A, Scal S, int cur, 
         }
         run_max = fmaxf(run_max, metric);
         run_tiles += 1;
-        if (PROPS) props_take(A, run_r, part, pa, warp_slot(A, int64_t(t) * (TILE / 32) + (threadIdx.x >> 5)));
+        if (PROPS) props_warp_add(A, run_r, part, pa);
     }
     if (run_r >= 0) flush_replica(A, S, run_r, run_max, run_tiles, sh_max, cond, use_cond, pfix);
     if (STG && stg_timeout) atomicOr(&A.g->err, ERR_TIMEOUT);
 }
 
 // ------------------------------------------------------------------------------------------
-// fused force + leapfrog step on a per-SM schedule (MD_MIXED, MD_FP32)
+// fused force + leapfrog step on a per-SM schedule
 // ------------------------------------------------------------------------------------------
 // The slots are cut into SM_RANGES-bounded contiguous ranges, one per SM id, and each warp takes
 // 32-slot warp-tiles from the range of the SM it runs on (an atomic counter per range), in
@@ -1070,7 +1030,9 @@ __global__ void __launch_bounds__(TILE, MINB) k_step(Arrays A, Scal S, int cur, 
 // gathers share one compact region in the SM's L1 instead of one region per CTA.  A warp whose
 // range is exhausted takes warp-tiles from any range with some left, so every warp-tile is
 // computed exactly once whatever the placement of the CTAs.  The last warp to finish resets the
-// counters for the next step.  Per atom the arithmetic is k_step's, bit for bit, and so are the
+// counters for the next step.  A launch with a warp for every warp-tile needs none of this: at 4000
+// LJ atoms the claims and scans of 128 warps over 152 ranges took most of a step (71 us; 14 us with
+// a warp-tile per warp, one warp per CTA and 8 entries per batch).  Per atom the arithmetic is k_step's, bit for bit, and so are the
 // props: the fixed-point sums do not depend on which warp took which warp-tile.
 __device__ __forceinline__ int ld_relaxed_gpu(const int* p)
 {
@@ -1109,7 +1071,7 @@ template <int MODE, bool PROPS, int NB, int MINB, int SRC = 0>
 __global__ void __launch_bounds__(TILE, MINB) k_step_sm(Arrays A, Scal S, int cur, cudaGraphConditionalHandle cond,
                                                       int use_cond)
 {
-    static_assert(MODE != MD_FP64, "MD_FP64 steps run k_step");
+    static_assert(MODE != MD_FP64 || SRC == 0, "MD_FP64 steps read W");
     const int nxt = cur ^ 1;
     const int lane = threadIdx.x & 31;
     uint32_t smid, nsmid;
@@ -1118,6 +1080,10 @@ __global__ void __launch_bounds__(TILE, MINB) k_step_sm(Arrays A, Scal S, int cu
     const int nr = max(1, min(int(nsmid), SM_RANGES));
     const int home = int(smid) % nr;
     const int nwt = S.ntiles * (TILE / 32);
+    const int wpc = blockDim.x >> 5, nwarps = gridDim.x * wpc;
+    // as many warps as warp-tiles: each takes its own, with no claims
+    const bool single = nwt <= nwarps;
+    const int own = blockIdx.x * wpc + (threadIdx.x >> 5);
     const int per = (nwt + nr - 1) / nr;
     int* const claimc = A.sm_claim;
     const float4* __restrict__ pos = A.pos32[cur];
@@ -1158,16 +1124,17 @@ __global__ void __launch_bounds__(TILE, MINB) k_step_sm(Arrays A, Scal S, int cu
 
     // w0 is computed while w1, the next warp-tile, has its positions and state prefetched into
     // L2 and the claim of the one after it is in flight
-    int w0 = claim_now();
-    int w1 = (w0 >= 0) ? claim_now() : -1;
+    int w0 = single ? (own < nwt ? own : -1) : claim_now();
+    int w1 = (!single && w0 >= 0) ? claim_now() : -1;
     int c0 = (w0 >= 0 && SRC == 0) ? __ldcs(A.nbr_count + int64_t(w0) * 32 + lane) : 0;   // w0's counts
     int run_r = -1, run_cnt = 0;
     float run_max = 0.0f;
     __shared__ long long s_pacc[TILE / 32][8];
     __shared__ float s_pvm[TILE / 32];
-    long long* const pacc = PROPS ? s_pacc[threadIdx.x >> 5] : nullptr;
-    float* const pvm = PROPS ? &s_pvm[threadIdx.x >> 5] : nullptr;
-    if (PROPS) {
+    constexpr bool FIX = PROPS && MODE != MD_FP64;        // props in fixed point
+    long long* const pacc = FIX ? s_pacc[threadIdx.x >> 5] : nullptr;
+    float* const pvm = FIX ? &s_pvm[threadIdx.x >> 5] : nullptr;
+    if (FIX) {
         if (lane < 8) pacc[lane] = 0;
         if (lane == 0) *pvm = 0.0f;
         __syncwarp();
@@ -1178,21 +1145,24 @@ __global__ void __launch_bounds__(TILE, MINB) k_step_sm(Arrays A, Scal S, int cu
         if (pending && lane == 0) pend = atomicAdd(claimc + home, 1);
         int c1 = 0;
         if (w1 >= 0) {
-            // one prefetch per 128-byte line: 4 lines of positions, 2 of each FP64 stream (1 of
-            // each FP32 stream), 4 of positions at the last rebuild (rule DISP)
+            // one prefetch per 128-byte line: 4 lines of positions (8 in FP64), 2 of each FP64 stream
+            // (1 of each FP32 stream), 4 of positions at the last rebuild (rule DISP)
             const int64_t s1 = int64_t(w1) * 32;
-            constexpr int NSTATE = (MODE == MD_MIXED) ? 12 : 3;
+            constexpr int NPOS = (MODE == MD_FP64) ? 8 : 4;
+            constexpr int NSTATE = (MODE == MD_MIXED) ? 12 : ((MODE == MD_FP64) ? 6 : 3);
             const int nref = (S.rule == MD_REBUILD_DISP) ? 4 : 0;
-            if (lane < 4 + NSTATE + nref) {
+            if (lane < NPOS + NSTATE + nref) {
                 const void* p;
-                if (lane < 4) {
-                    p = A.pos32[cur] + s1 + 8 * lane;
-                } else if (lane < 4 + NSTATE) {
-                    const int q = lane - 4;
-                    if (MODE == MD_MIXED) p = ((q & 1) ? A.v[q >> 2] : A.xl[q >> 2]) + s1 + 16 * ((q >> 1) & 1);
+                if (lane < NPOS) {
+                    if (MODE == MD_FP64) p = A.pos64[cur] + s1 + 4 * lane;
+                    else p = A.pos32[cur] + s1 + 8 * lane;
+                } else if (lane < NPOS + NSTATE) {
+                    const int q = lane - NPOS;
+                    if (MODE == MD_FP64) p = A.v[q >> 1] + s1 + 16 * (q & 1);
+                    else if (MODE == MD_MIXED) p = ((q & 1) ? A.v[q >> 2] : A.xl[q >> 2]) + s1 + 16 * ((q >> 1) & 1);
                     else p = A.v32[q] + s1;
                 } else {
-                    p = A.xref + s1 + 8 * (lane - 4 - NSTATE);
+                    p = A.xref + s1 + 8 * (lane - NPOS - NSTATE);
                 }
                 prefetch_l2(p);
             }
@@ -1211,10 +1181,54 @@ __global__ void __launch_bounds__(TILE, MINB) k_step_sm(Arrays A, Scal S, int cu
         const bool active = slot - R.slot0 < R.n;
         const int vhalf = A.rs[r].vhalf;
         float metric = 0.0f;                     // |v|^2 (VMAX) or |x - x_ref|^2 (DISP)
-        float part[NPROP];
+        using PT = typename std::conditional<MODE == MD_FP64, double, float>::type;
+        PT part[NPROP];
 #pragma unroll
-        for (int q = 0; q < NPROP; ++q) part[q] = 0.0f;
-        if (active) {
+        for (int q = 0; q < NPROP; ++q) part[q] = PT(0);
+        if constexpr (MODE == MD_FP64) {
+            if (active) {
+                const double4_32a* pos64 = A.pos64[cur];
+                const double4_32a pi = pos64[slot];
+                double vs[3];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) vs[q] = A.v[q][slot];
+                const AccD a = force_f64<NB>(A, S, R, pos64, slot, pi);
+                const double f[3] = {a.fx, a.fy, a.fz};
+                double xl[3] = {pi.x, pi.y, pi.z};
+                const double kick = vhalf ? 2.0 * S.c : S.c;
+                double vn2 = 0.0;
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    double v = vs[q];
+                    if (PROPS) {
+                        const double vn = vhalf ? fma(S.c, f[q], v) : v;
+                        vn2 = fma(vn, vn, vn2);
+                        part[3 + q] = vn;
+                    }
+                    v = fma(kick, f[q], v);
+                    xl[q] = fma(S.dt, v, xl[q]);
+                    A.v[q][slot] = v;
+                    A.xl[q][slot] = xl[q];
+                }
+                A.pos64[nxt][slot] = make_double4_32a(xl[0], xl[1], xl[2], pi.w);
+                if (S.rule == MD_REBUILD_DISP) {
+                    const float4 xr = A.xref[slot];
+                    const float d0 = float(xl[0] - double(xr.x)), d1 = float(xl[1] - double(xr.y)),
+                                d2 = float(xl[2] - double(xr.z));
+                    metric = d0 * d0 + d1 * d1 + d2 * d2;
+                } else {
+                    const double d0 = xl[0] - pi.x, d1 = xl[1] - pi.y, d2 = xl[2] - pi.z;
+                    metric = float(d0 * d0 + d1 * d1 + d2 * d2);
+                }
+                if (PROPS) {
+                    part[0] = a.u;
+                    part[1] = vn2;
+                    part[2] = a.w;
+                    part[NPROP - 1] = vn2;
+                }
+                if (!(metric <= 3.0e38f)) metric = __uint_as_float(0x7f800000u);
+            }
+        } else if (active) {
             const float4 pi = __ldg(pos + slot);
             AccF a;
             if (SRC == 1) {
@@ -1259,7 +1273,8 @@ __global__ void __launch_bounds__(TILE, MINB) k_step_sm(Arrays A, Scal S, int cu
         }
         run_max = fmaxf(run_max, metric);
         run_cnt += 1;
-        if (PROPS) props_warp_add_sh(A, r, part, pacc, pvm);
+        if constexpr (FIX) props_warp_add_sh(A, r, part, pacc, pvm);
+        else if constexpr (PROPS) warp_partials_store(part, warp_slot(A, w0));
         int w2 = -1;
         if (w1 >= 0) {
             // the rows of W below the next warp-tile's largest count into L2
@@ -1279,10 +1294,9 @@ __global__ void __launch_bounds__(TILE, MINB) k_step_sm(Arrays A, Scal S, int cu
     }
     if (run_r >= 0) flush_replica_warp(A, S, run_r, run_max, run_cnt, cond, use_cond, pacc, pvm);
     // the last warp of the launch resets the counters; the next launch is ordered after this one
-    if (lane == 0) {
+    if (!single && lane == 0) {
         __threadfence();
-        const int total = int(gridDim.x) * (TILE / 32);
-        if (atomicAdd(claimc + SM_RANGES, 1) == total - 1) {
+        if (atomicAdd(claimc + SM_RANGES, 1) == nwarps - 1) {
             for (int q = 0; q < nr; ++q) claimc[q] = 0;
             claimc[SM_RANGES] = 0;
             __threadfence();
@@ -1463,7 +1477,7 @@ __global__ void __launch_bounds__(TILE) k_forces(Arrays A, Scal S, int cur)
         if (slot - R.slot0 >= R.n) continue;
         if (MODE == MD_FP64) {
             const double4_32a pi = A.pos64[cur][slot];
-            const AccD a = force_f64(A, S, R, A.pos64[cur], slot, pi);
+            const AccD a = force_f64<4>(A, S, R, A.pos64[cur], slot, pi);
             A.f[slot] = make_double4_32a(a.fx, a.fy, a.fz, a.u);
             A.wvir[slot] = a.w;
         } else {
@@ -1706,7 +1720,7 @@ template <int M, int NB, int MINB, bool STG = false>
 static int occ_of(int dyn_smem = 0)
 {
     int a = 0, b = 0;
-    if constexpr (M != MD_FP64 && !STG) {
+    if constexpr (!STG) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_step_sm<M, false, NB, MINB>, TILE, dyn_smem);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_step_sm<M, true, NB, MINB>, TILE, dyn_smem);
     } else {
@@ -1813,7 +1827,7 @@ static int occ_src_mb(int mb)
 int step_ctas_per_sm(const Scal& S, const Launch& L)
 {
     int occ = 1;
-    if (S.mode == MD_FP64) return occ_of<MD_FP64, 2, 4>();
+    if (S.mode == MD_FP64) return occ_of<MD_FP64, 4, 4>();
     if (L.step_kernel == 4 || L.step_kernel == 5) {
         const int mb = minb_of(L.ctas_req);
         if (L.step_kernel == 4) return S.mode == MD_MIXED ? occ_src_mb<MD_MIXED, 1>(mb) : occ_src_mb<MD_FP32, 1>(mb);
@@ -1895,13 +1909,11 @@ cudaError_t launch_step(const Arrays& A, const Scal& S, const Launch& L, int cur
     } else {
 #define GBMD_STEP(M, NB, MB)                                                                           \
     {                                                                                                  \
-        if (props) k_step_sm<M, true, NB, MB><<<g, TILE, 0, L.stream>>>(A, S, cur, L.cond, L.use_cond);         \
-        else k_step_sm<M, false, NB, MB><<<g, TILE, 0, L.stream>>>(A, S, cur, L.cond, L.use_cond);               \
+        if (props) k_step_sm<M, true, NB, MB><<<gs, bs, 0, L.stream>>>(A, S, cur, L.cond, L.use_cond);         \
+        else k_step_sm<M, false, NB, MB><<<gs, bs, 0, L.stream>>>(A, S, cur, L.cond, L.use_cond);               \
     }
-        if (S.mode == MD_FP64) {
-            if (props) k_step<MD_FP64, true, 2, 4, false><<<g, TILE, 0, L.stream>>>(A, S, cur, L.cond, L.use_cond, 0);
-            else k_step<MD_FP64, false, 2, 4, false><<<g, TILE, 0, L.stream>>>(A, S, cur, L.cond, L.use_cond, 0);
-        }
+        const int gs = L.step_single ? S.ntiles * (TILE / 32) : g, bs = L.step_single ? 32 : TILE;
+        if (S.mode == MD_FP64) GBMD_STEP(MD_FP64, 4, 4)
         else if (S.mode == MD_MIXED) GBMD_DISPATCH_NB_MINB(MD_MIXED, GBMD_STEP)
         else GBMD_DISPATCH_NB_MINB(MD_FP32, GBMD_STEP)
 #undef GBMD_STEP
