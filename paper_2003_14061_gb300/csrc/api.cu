@@ -204,8 +204,11 @@ size_t carve(const Plan& P, char* base, Arrays* A)
     a.W = c.take<uint32_t>(ns * size_t(P.cap));
     if (P.rule == MD_REBUILD_DISP) a.xref = c.take<float4>(ns);
     a.perm = c.take<int32_t>(ns);
-    a.psort = c.take<float4>(ns + 4 * size_t(P.nrows) + CAND_PAD);
+    const size_t ncand = ns + 4 * size_t(P.nrows) + CAND_PAD;
+    a.psort = c.take<float4>(3 * (ncand / 4 + 1));
+    a.pent = c.take<uint32_t>(ncand);
     a.pcell = c.take<uint32_t>(ns);
+    a.crun = c.take<int2>(size_t(P.ncells));
     if (!f64) a.tile_win = c.take<int2>(size_t(P.ntiles) * 9);
     if (!f64) {
         a.fbuf = c.take<float4>(ns);
@@ -457,7 +460,7 @@ int apply_tuning(md_system* s)
     s->S.half_list = (s->L.step_kernel == 5) ? 1 : 0;      // W keeps each pair once
     bulk_shape(s->S, per_sm, s->smem_per_sm, s->smem_per_cta, &s->L.bulk_rows, &s->L.bulk_smem);
     stage_shape(per_sm, s->smem_per_sm, &s->L.stage_cap, &s->L.stage_smem);
-    build_group_shape(s->S, s->L, s->plan.mean_nbrs, s->smem_per_cta, s->smem_per_sm);
+    build_group_shape(s->S, s->L, s->plan.mean_nbrs, s->smem_per_cta);
     // Step-kernel shape.  One that md_set_tuning never named is chosen by size: 4 CTAs per SM with 8
     // W entries together (120 registers) up to 1.5M atoms and at 30 neighbours or more, else 8 CTAs
     // and 2 entries, whose warps hide the HBM latency that the larger fluids wait for.  Step kernel,

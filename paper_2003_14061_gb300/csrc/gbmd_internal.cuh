@@ -37,10 +37,10 @@ constexpr int PROPS_SPLIT_MAX = 2048;     // CTAs per replica in the first level
 constexpr int ADJ_VPART = 128;            // blocks of the |v_S|^2 partial sums
 
 // Candidate array of the neighbour build (psort): the atoms in cell order, their positions in the
-// replica's frame (cell origin + cell-local position, FP32).  Two consecutive entries share 32
-// bytes, x0 x1 y0 y1 | z0 z1 e0 e1, the operands of packed FP32x2 operations; e = slot << IDX_SHIFT
-// | (c_x mod 4).  Every row of cells starts at a multiple of 4 entries and is followed up to the
-// next one by entries far outside the box, so whole groups of 4 can be tested without bounds.
+// replica's frame (cell origin + cell-local position, FP32).  Four consecutive entries share 48
+// bytes, x0..x3 y0..y3 z0..z3, the operands of packed FP32x2 operations; pent holds slot << IDX_SHIFT
+// | (c_x mod 4) of each.  Every row of cells starts at a multiple of 4 entries and is followed up to
+// the next one by entries far outside the box, so whole groups of 4 can be tested without bounds.
 // Row q (counted over all replicas) whose first atom is number rs of the cell order starts at
 // entry cand_place = ceil4(rs) + 4 q: at most 4 entries of padding per row.
 constexpr float CAND_FAR = 1.0e15f;
@@ -119,7 +119,11 @@ struct Arrays {
     float4* xref;             // positions at the last rebuild (rule DISP)
     int32_t* perm;            // cell-ordered slots (the matrix H of Sec. 2.3, flattened)
     float4* psort;            // candidate array of the neighbour build (cand_place, cand_store)
+    uint32_t* pent;           //   and slot << IDX_SHIFT | (c_x mod 4) of its entries
     uint32_t* pcell;          // packed cell of every atom in cell order
+    int2* crun;               // per cell: the candidates of its row of cells from the cell before to the
+                              // cell after it (not across the boundary), [first, end) in groups of
+                              // 4 entries of the array, counted from its replica's first group
     float4* fbuf;             // step kernel 5: FP32 force and u_i accumulated over the half list
     float* wbuf;              //   and the per-atom virial (zero between steps)
     int2* tile_win;           // [ntiles][9] slot window (lo, hi) of each tile's W entries per
@@ -133,7 +137,7 @@ struct Arrays {
     // per cell
     int32_t* ccount;
     int32_t* cstart;
-    int2* ckeep;              // per cell: [start, end) in its replica's cell order at that replica's
+    int2* ckeep;              // (list-free kernel) per cell: [start, end) in its replica's cell order at that replica's
                               // last rebuild (the list-free step kernel reads it every step; cstart
                               // is recomputed for all cells when any replica rebuilds)
     int32_t* chunk;           // per SCAN_CHUNK cells
@@ -252,13 +256,13 @@ __host__ __device__ __forceinline__ int cand_place(const Rep& R, int prow, int r
     return ((rs + 3) & ~3) + 4 * (R.row0 + prow);
 }
 
-__device__ __forceinline__ void cand_store(float4* psort, int P, float x, float y, float z, uint32_t e)
+__device__ __forceinline__ void cand_store(float4* psort, uint32_t* pent, int P, float x, float y, float z, uint32_t e)
 {
-    float* f = reinterpret_cast<float*>(psort) + int64_t(8) * (P >> 1) + (P & 1);
+    float* f = reinterpret_cast<float*>(psort) + int64_t(12) * (P >> 2) + (P & 3);
     f[0] = x;
-    f[2] = y;
-    f[4] = z;
-    f[6] = __uint_as_float(e);
+    f[4] = y;
+    f[8] = z;
+    pent[P] = e;
 }
 
 // (cx, cy, cz) of the replica-local cell number cl
@@ -423,10 +427,9 @@ struct Launch {
     int ctas_req;             // requested resident CTAs/SM (register bound of the step kernel)
     int step_single;          // step kernel 1: one warp per CTA and warp-tile, all of them resident at once
     int bg_rows;              // k_build_group: rows of each lane's list in shared memory,
-    int bg_block;             // threads per CTA, dynamic shared memory and CTAs
+    int bg_block;             // threads per CTA (one CTA per SM), dynamic shared memory,
     int bg_smem;
-    int bg_grid;
-    int bg_minb;              // its register bound: CTAs per SM it is compiled for (8, or 5 with long lists)
+    int bg_warps;             // and the warps per CTA it is compiled for (32, or 20 with long lists)
     int step_kernel;          // 1: per-thread loads with L2 prefetch; 2: bulk-copy shared-memory ring;
                               // 3: as 1, with each tile's neighbour positions staged in shared memory
     int bulk_rows;            // rows of W staged per tile by the ring (step_kernel 2)
@@ -457,7 +460,7 @@ int bin_kernels(const Scal& S, const Launch& L);     // kernels of launch_bin_or
 constexpr int REORDER_KERNELS = 2;                   // kernels of launch_reorder
 int build_kernels(const Scal& S, const Launch& L);   // kernels of launch_build_only
 // rows of k_build_group's lists, its CTA size, shared memory and grid, into L
-void build_group_shape(const Scal& S, Launch& L, double mean_nbrs, int smem_per_cta, int smem_per_sm);
+void build_group_shape(const Scal& S, Launch& L, double mean_nbrs, int smem_per_cta);
 
 // adjoint (kernels_adjoint.cu)
 cudaError_t launch_adj_reverse(const Arrays& A, const Scal& S, const Launch& L, const AdjView& V, int q, double kappa,

@@ -19,7 +19,6 @@
 // Only replicas whose rebuild flag is set do work; kernels return at once when none is set, so
 // the whole sequence can sit in every step of md_integrate.
 #include <algorithm>
-#include <atomic>
 
 #include "gbmd_internal.cuh"
 
@@ -358,16 +357,31 @@ static void launch_scan(const Arrays& A, const ScanArgs& C, cudaStream_t st)
 // ------------------------------------------------------------------------------------------
 // N4 and the deterministic order within cells
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(TILE) k_scatter(Arrays A, Scal S)
+__global__ void __launch_bounds__(TILE) k_scatter(Arrays A, Scal S, int keep)
 {
     if (!A.g->any_rebuild) return;
     const int nrb = A.g->n_rb_tiles;
+    const int32_t* __restrict__ cs = A.cstart;
     for (int it = blockIdx.x; it < nrb; it += gridDim.x) {
         const int t = A.rb_tiles[it];
         const int r = A.tile_rep[t];
         const Rep& R = A.rep[r];
         const int64_t slot = int64_t(t) * TILE + threadIdx.x;
-        if (slot - R.slot0 < R.n) A.tmp_i[0][A.cstart[A.cell[slot]] + A.layer[slot]] = int32_t(slot);
+        if (slot - R.slot0 < R.n) A.tmp_i[0][cs[A.cell[slot]] + A.layer[slot]] = int32_t(slot);
+        // this tile's share of the replica's cells: their runs of candidates (keep: also their slot
+        // ranges, for the list-free step kernel)
+        const int tt = t - R.tile0, ncx = R.nc[0];
+        const int c_end = int(int64_t(R.ncells) * (tt + 1) / R.ntiles);
+        const int k0 = cs[R.cell0], P0 = cand_place(R, 0, k0);
+        for (int c = int(int64_t(R.ncells) * tt / R.ntiles) + int(threadIdx.x); c < c_end; c += TILE) {
+            const int prow = c / ncx, cx = c - prow * ncx;
+            const int32_t* row = cs + R.cell0 + prow * ncx;
+            const int rs = row[0];
+            const int base = cand_place(R, prow, rs) - P0;
+            A.crun[R.cell0 + c] = make_int2((base + ((row[max(cx - 1, 0)] - rs) & ~3)) >> 2,
+                                            (base + ((row[min(cx + 1, ncx - 1) + 1] - rs + 3) & ~3)) >> 2);
+            if (keep) A.ckeep[R.cell0 + c] = make_int2(row[cx] - k0, row[cx + 1] - k0);
+        }
     }
 }
 
@@ -418,22 +432,10 @@ __global__ void __launch_bounds__(TILE) k_order(Arrays A, Scal S, int cur)
         const int rs = cs[R.cell0 + prow * R.nc[0]], re = cs[R.cell0 + (prow + 1) * R.nc[0]];
         const int P = cand_place(R, prow, rs) + (k - rs);
         const int64_t out_slot = A.rs[r].reorder ? R.slot0 + (k - cs[R.cell0]) : slot;
-        cand_store(A.psort, P, G[0], G[1], G[2], (uint32_t(out_slot) << IDX_SHIFT) | uint32_t(cc[0] & 3));
+        cand_store(A.psort, A.pent, P, G[0], G[1], G[2], (uint32_t(out_slot) << IDX_SHIFT) | uint32_t(cc[0] & 3));
         A.pcell[k] = pc;
         if (k == re - 1)                              // far-away entries up to the group of 4
-            for (int q = P + 1; q & 3; ++q) cand_store(A.psort, q, CAND_FAR, CAND_FAR, CAND_FAR, 0u);
-    }
-}
-
-// the slot range of every cell in its replica, for the list-free step kernel
-__global__ void __launch_bounds__(256) k_cell_ranges(Arrays A, Scal S)
-{
-    if (!A.g->any_rebuild) return;
-    for (int64_t c = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; c < S.ncells; c += int64_t(gridDim.x) * blockDim.x) {
-        const int r = A.cell_rep[c];
-        if (!A.rs[r].rebuild) continue;
-        const int base = A.cstart[A.rep[r].cell0];
-        A.ckeep[c] = make_int2(A.cstart[c] - base, A.cstart[c + 1] - base);
+            for (int q = P + 1; q & 3; ++q) cand_store(A.psort, A.pent, q, CAND_FAR, CAND_FAR, CAND_FAR, 0u);
     }
 }
 
@@ -562,27 +564,28 @@ __device__ __noinline__ float criterion(const void* pos, const Rep* Rp, double r
 // each atom's three lists (planes in order, so the entries of a column come in the order rows,
 // cells, slots) and writes W row by row: consecutive lanes write consecutive slots.
 //
-// Bounds: the loads of candidates return 16 bytes to each of 32 lanes, 4 cycles of the SM's 128
-// bytes per cycle (65 % busy), and about 12 instructions per candidate issue (45 %).  Measured
-// against one thread per atom walking its nine rows and branching at every append (per rebuild,
-// GB300): LJ r_c + skin = 2.8: 16.4M atoms 27.7 -> 12 ms, 256k atoms 513 -> 210 us, 4000 atoms
-// 388 -> 22 us; WCA: 100k atoms 110 -> 30 us, 4M atoms 0.76 -> 0.75 ms (the two are even there);
-// FP64, 2048 atoms 71 -> 11 us (positions tested in FP32, the criterion in FP64).  The lanes' own
-// runs beat one run shared by a unit's atoms of a row (fewer distinct addresses per load, more
-// candidates: 0.59 against 0.69 ms at 2M WCA atoms, 0.72 against 0.78 ms at 864k LJ atoms);
-// loads one pass ahead cost registers and lost (0.70 and 0.86 ms).
+// Bounds: the loads of candidates (12 bytes to each of 32 lanes, SM load pipe 63-72 % busy) and
+// issue (44-60 %); what waits is their latency, so as many warps as fit matter: with 16-bit list
+// entries 31 of them at the LJ cutoff (0.67 ms per binning and build of 864k atoms; 20 with 32-bit
+// ones 0.77, 16 0.90), 32 at WCA.  Measured against one thread per atom walking its nine rows and
+// branching at every append (per rebuild): LJ r_c + skin = 2.8: 16.4M atoms 27.7 -> 11.5 ms, 256k
+// atoms 513 -> 200 us, 4000 atoms 388 -> 31 us; WCA: 100k atoms 110 -> 30 us, 4M atoms 0.76 ->
+// 0.75 ms; FP64, 2048 atoms 71 -> 9 us (positions tested in FP32, the criterion in FP64).  One run
+// shared by a unit's atoms of a row (fewer distinct addresses per load, more candidates) lost:
+// 0.69 against 0.59 ms at 2M WCA atoms; so did loads one pass ahead (registers) and passes of 8.
 // ------------------------------------------------------------------------------------------
 constexpr int BG_ATOMS = 10;
 constexpr int BG_UNITS = (TILE + BG_ATOMS - 1) / BG_ATOMS;       // units per rebuild tile
 constexpr int BG_STEP = 4;                                       // candidates per pass of the scan
-constexpr uint32_t BG_ROW = 32 * 4;                              // bytes of one row of the lists
+constexpr int BG_TABLE = 12 * 32 * 4;                            // bytes of a warp's table of run starts
+constexpr uint32_t BG_ROW = 32 * 2;                              // bytes of one row of the lists
 
 // append v to the list at shared address w where d < 0
 __device__ __forceinline__ void list_append(uint32_t& w, float d, uint32_t v)
 {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %1, 0f00000000;\n\t@p st.shared.u32 [%0], %2;\n\t"
-                 "@p add.u32 %0, %0, 128;\n\t}"
-                 : "+r"(w) : "f"(d), "r"(v));
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %1, 0f00000000;\n\t@p st.shared.u16 [%0], %2;\n\t"
+                 "@p add.u32 %0, %0, 64;\n\t}"
+                 : "+r"(w) : "f"(d), "h"(uint16_t(v)));
 }
 // the same where also e != self (NE) or e > self (unsigned)
 template <bool GT>
@@ -590,60 +593,64 @@ __device__ __forceinline__ void list_append_if(uint32_t& w, float d, uint32_t v,
 {
     if constexpr (GT)
         asm volatile("{\n\t.reg .pred p, q;\n\tsetp.gt.u32 q, %3, %4;\n\tsetp.lt.and.f32 p, %1, 0f00000000, q;\n\t"
-                     "@p st.shared.u32 [%0], %2;\n\t@p add.u32 %0, %0, 128;\n\t}"
-                     : "+r"(w) : "f"(d), "r"(v), "r"(e), "r"(self));
+                     "@p st.shared.u16 [%0], %2;\n\t@p add.u32 %0, %0, 64;\n\t}"
+                     : "+r"(w) : "f"(d), "h"(uint16_t(v)), "r"(e), "r"(self));
     else
         asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %3, %4;\n\tsetp.lt.and.f32 p, %1, 0f00000000, q;\n\t"
-                     "@p st.shared.u32 [%0], %2;\n\t@p add.u32 %0, %0, 128;\n\t}"
-                     : "+r"(w) : "f"(d), "r"(v), "r"(e), "r"(self));
+                     "@p st.shared.u16 [%0], %2;\n\t@p add.u32 %0, %0, 64;\n\t}"
+                     : "+r"(w) : "f"(d), "h"(uint16_t(v)), "r"(e), "r"(self));
 }
+
+// List entries, 16 bits: the candidate's number within its run, the row's o_y + 1 and the periodic
+// shift of the run in x (1: from the left image, 2: from the right one).  The start of each run is
+// kept in a table per lane, so that the place, the slot and the code of W follow when the lists are
+// joined.  A unit with a run of more than BG_RUN candidates goes through build_column.
+constexpr int BG_RUN = 4096, BG_OY = 12, BG_IMG = 14;
 
 struct ScanLane {               // what a lane keeps while it scans
     float2 nx, ny, nz;          // minus the atom's coordinates, as seen from the row's cells
     float band;
-    uint32_t self;              // its own entry (HALF: its slot's last code)
-    uint32_t w, wlim, lost;     // list position and its limit; entries beyond it
+    uint32_t self;              // its own W word (slot << IDX_SHIFT | c_x mod 4)
+    uint32_t w, wlim, lost;     // list position and its limit; bytes of entries beyond it
+    bool far;                   // a run was too long for the entries
 };
 
-// Candidates [P0, P1) (multiples of 4) of one run.  SELF: the run may hold the atom itself.
-// IMG: the run lies across the periodic boundary in x, imgadd = its shift in cells (mod 4).
-template <int MODE, bool HALF, bool SELF, bool IMG>
-__device__ __forceinline__ void scan_run(const float4* __restrict__ ps, int P0, int P1, ScanLane& L, float rl2f,
-                                         double rl2d, uint32_t code, uint32_t imgadd, const void* pos, const Rep* Rp,
-                                         int sx, int oy, int oz)
+// Candidate groups [g0, g1) of one run.  SELF: the run may hold the atom itself, whose list entry
+// would be `mine`.
+template <int MODE, bool HALF, bool SELF>
+__device__ __forceinline__ void scan_run(const float4* __restrict__ ps, const uint32_t* __restrict__ pent, int g0, int g1,
+                                         ScanLane& L, int* runs, float rl2f, double rl2d, uint32_t tag, uint32_t mine,
+                                         const void* pos, const Rep* Rp, int sx, int oy, int oz)
 {
     const float2 nrl2 = make_float2(-rl2f, -rl2f);
-    for (int P = P0; P < P1; P += BG_STEP) {
-        float d[BG_STEP];
-        uint32_t e[BG_STEP];
-#pragma unroll
-        for (int h = 0; h < BG_STEP / 2; ++h) {
-            const float4 xy = __ldg(ps + P + 2 * h), ze = __ldg(ps + P + 2 * h + 1);
-            const float2 dx = __fadd2_rn(make_float2(xy.x, xy.y), L.nx);
-            const float2 dy = __fadd2_rn(make_float2(xy.z, xy.w), L.ny);
-            const float2 dz = __fadd2_rn(make_float2(ze.x, ze.y), L.nz);
-            const float2 q = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __ffma2_rn(dx, dx, nrl2)));
-            d[2 * h] = q.x;
-            d[2 * h + 1] = q.y;
-            e[2 * h] = __float_as_uint(ze.z);
-            e[2 * h + 1] = __float_as_uint(ze.w);
-        }
+    runs[32 * (tag >> BG_OY)] = BG_STEP * g0;
+    L.far |= g1 - g0 > BG_RUN / BG_STEP;
+    for (int g = g0; g < g1; ++g) {
+        const float4 x = __ldg(ps + 3 * g), y = __ldg(ps + 3 * g + 1), z = __ldg(ps + 3 * g + 2);
+        const float2 dx0 = __fadd2_rn(make_float2(x.x, x.y), L.nx), dx1 = __fadd2_rn(make_float2(x.z, x.w), L.nx);
+        const float2 dy0 = __fadd2_rn(make_float2(y.x, y.y), L.ny), dy1 = __fadd2_rn(make_float2(y.z, y.w), L.ny);
+        const float2 dz0 = __fadd2_rn(make_float2(z.x, z.y), L.nz), dz1 = __fadd2_rn(make_float2(z.z, z.w), L.nz);
+        const float2 q0 = __ffma2_rn(dz0, dz0, __ffma2_rn(dy0, dy0, __ffma2_rn(dx0, dx0, nrl2)));
+        const float2 q1 = __ffma2_rn(dz1, dz1, __ffma2_rn(dy1, dy1, __ffma2_rn(dx1, dx1, nrl2)));
+        float d[BG_STEP] = {q0.x, q0.y, q1.x, q1.y};
         if (fminf(fminf(fabsf(d[0]), fabsf(d[1])), fminf(fabsf(d[2]), fabsf(d[3]))) < L.band) {
 #pragma unroll
             for (int u = 0; u < BG_STEP; ++u)
                 if (fabsf(d[u]) < L.band)
-                    d[u] = criterion<MODE>(pos, Rp, rl2d, rl2f, int(L.self >> IDX_SHIFT), int(e[u] >> IDX_SHIFT), sx, oy, oz);
+                    d[u] = criterion<MODE>(pos, Rp, rl2d, rl2f, int(L.self >> IDX_SHIFT),
+                                           int(pent[BG_STEP * g + u] >> IDX_SHIFT), sx, oy, oz);
         }
+        const uint32_t v = uint32_t(BG_STEP * (g - g0)) | tag;
 #pragma unroll
         for (int u = 0; u < BG_STEP; ++u) {
-            const uint32_t v = IMG ? (((e[u] + imgadd) & ~0x3Cu) | code) : (e[u] | code);
-            if (HALF) list_append_if<true>(L.w, d[u], v, e[u], L.self | 63u);
-            else if (SELF) list_append_if<false>(L.w, d[u], v, e[u], L.self);
-            else list_append(L.w, d[u], v);
+            if (HALF) list_append_if<true>(L.w, d[u], v | uint32_t(u), pent[BG_STEP * g + u], L.self | 63u);
+            else if (SELF) list_append_if<false>(L.w, d[u], v | uint32_t(u), uint32_t(BG_STEP * g + u), mine);
+            else list_append(L.w, d[u], v | uint32_t(u));
         }
-        const uint32_t over = max(L.w, L.wlim) - L.wlim;          // a full list counts on, writing past its end
-        L.lost += over;
-        L.w -= over;
+        if (L.w > L.wlim) {                           // a full list counts on, writing past its end
+            L.lost += L.w - L.wlim;
+            L.w = L.wlim;
+        }
     }
 }
 
@@ -678,21 +685,27 @@ __device__ __noinline__ int build_column(const void* pos, const Rep* Rp, const i
     return m;
 }
 
-template <int MODE, bool HALF, int MINB>
-__global__ void __launch_bounds__(TILE, MINB) k_build_group(Arrays A, Scal S, int cur, int rows)
+template <int MODE, bool HALF, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, 1) k_build_group(Arrays A, Scal S, int cur, int rows)
 {
     extern __shared__ uint32_t s_list[];              // [warps][rows + BG_STEP][32]
     if (!A.g->any_rebuild) return;
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-    const uint32_t* const my_lists = s_list + wl * (rows + BG_STEP) * 32;
+    // per warp: the table of run starts [BG_RUNS + 3][32], then the lists [rows + BG_STEP][32]
+    unsigned char* const mem = reinterpret_cast<unsigned char*>(s_list) + wl * (BG_TABLE + (rows + BG_STEP) * int(BG_ROW));
+    int* const my_runs = reinterpret_cast<int*>(mem);
+    const uint16_t* const my_lists = reinterpret_cast<const uint16_t*>(mem + BG_TABLE);
     const int a = lane % BG_ATOMS, pl = lane / BG_ATOMS;          // atom of the unit, z plane (3: idle lane)
-    const float4* __restrict__ ps = A.psort;
     const int32_t* __restrict__ cs = A.cstart;
     const void* const pos = (MODE == MD_FP64) ? static_cast<const void*>(A.pos64[cur]) : static_cast<const void*>(A.pos32[cur]);
     const int nunits = A.g->n_rb_tiles * BG_UNITS;
-    const int wpc = blockDim.x >> 5, nw = gridDim.x * wpc;
+    // every CTA takes a contiguous run of units, its warps side by side: neighbouring units read the
+    // same rows of candidates
+    const int wpc = blockDim.x >> 5;
+    const int per = (nunits + int(gridDim.x) - 1) / int(gridDim.x), u_begin = int(blockIdx.x) * per;
+    const int u_end = min(nunits, u_begin + per);
     ScanLane L;
-    L.wlim = smem_u32(my_lists + lane) + uint32_t(rows) * BG_ROW;
+    L.wlim = smem_u32(my_lists) + 2 * lane + uint32_t(rows) * BG_ROW;
     int run_r = -1, run_max = 0;
     long long run_sum = 0;
     auto flush_warp = [&]() {
@@ -703,7 +716,7 @@ __global__ void __launch_bounds__(TILE, MINB) k_build_group(Arrays A, Scal S, in
             if (wm > 0) atomicMax(&A.rs[run_r].max_nbrs, wm);
         }
     };
-    for (int uid = blockIdx.x * wpc + wl; uid < nunits; uid += nw) {
+    for (int uid = u_begin + wl; uid < u_end; uid += wpc) {
         const int it = uid / BG_UNITS, u = uid - it * BG_UNITS;
         const int t = A.rb_tiles[it];
         const int r = A.tile_rep[t];
@@ -718,23 +731,27 @@ __global__ void __launch_bounds__(TILE, MINB) k_build_group(Arrays A, Scal S, in
             run_max = 0;
         }
         const bool act = pl < 3 && a < na;
-        const int k = cs[R.cell0] + j0 + min(a, na - 1);
+        const int k0 = cs[R.cell0];
+        const int k = k0 + j0 + min(a, na - 1);
         const uint32_t pc = A.pcell[k];
         int cx, cy, cz;
         unpack_cell(pc, cx, cy, cz);
         const int ncx = R.nc[0], ncy = R.nc[1], ncz = R.nc[2];
+        const int P0 = cand_place(R, 0, k0);          // the replica's part of the candidate array
+        const float4* __restrict__ ps = A.psort + int64_t(3) * (P0 >> 2);
+        const uint32_t* __restrict__ pent = A.pent + P0;
         float X, Y, Z;
+        uint32_t mine;                                // the atom's own place
         {
             const int prow = row_pos(R, cy, cz);
             const int rs = cs[R.cell0 + prow * ncx];
-            const int P = cand_place(R, prow, rs) + (k - rs);
-            const float* f = reinterpret_cast<const float*>(ps) + 8 * (P >> 1) + (P & 1);
+            mine = uint32_t(cand_place(R, prow, rs) - P0 + (k - rs));
+            const float* f = reinterpret_cast<const float*>(ps) + 12 * (mine >> 2) + (mine & 3u);
             X = f[0];
-            Y = f[2];
-            Z = f[4];
-            L.self = __float_as_uint(f[6]);
+            Y = f[4];
+            Z = f[8];
+            L.self = pent[mine];
         }
-        const int xlo = cx - 1, xhi = cx + 1;
         const int oz = pl - 1;
         int nz = cz + oz;
         float wz = 0.0f;                              // shift of the atom into the frame of wrapped cells
@@ -743,7 +760,10 @@ __global__ void __launch_bounds__(TILE, MINB) k_build_group(Arrays A, Scal S, in
         L.nz = make_float2(-(Z + wz), -(Z + wz));
         L.w = L.wlim - uint32_t(rows) * BG_ROW;
         L.lost = 0;
-        const bool any_lo = __any_sync(0xffffffffu, act && xlo < 0), any_hi = __any_sync(0xffffffffu, act && xhi >= ncx);
+        L.far = false;
+        const bool lo = act && cx == 0, hi = act && cx == ncx - 1;
+        const bool any_lo = __any_sync(0xffffffffu, lo), any_hi = __any_sync(0xffffffffu, hi);
+        const float band = R.band;
 #pragma unroll 1
         for (int oy = -1; oy <= 1; ++oy) {
             int ny = cy + oy;
@@ -751,35 +771,35 @@ __global__ void __launch_bounds__(TILE, MINB) k_build_group(Arrays A, Scal S, in
             if (ny < 0) { ny += ncy; wy = float(ncy) * R.wf[1]; }
             else if (ny >= ncy) { ny -= ncy; wy = -float(ncy) * R.wf[1]; }
             L.ny = make_float2(-(Y + wy), -(Y + wy));
-            const float bandw = (wy != 0.0f || wz != 0.0f) ? 4.0f * R.band : R.band;
-            const uint32_t code = (uint32_t(oy + 1) << 2) | (uint32_t(oz + 1) << 4);
+            const uint32_t tag = uint32_t(oy + 1) << BG_OY;
             const int prow = row_pos(R, ny, nz < ncz ? nz : 0);
             const int row = R.cell0 + prow * ncx;
-            const int rs = cs[row];
-            const int base = cand_place(R, prow, rs);
-            if (any_lo) {
+            if (any_lo) {                             // the row's last cell, seen across the boundary
                 const float xs = X + float(ncx) * R.wf[0];
                 L.nx = make_float2(-xs, -xs);
-                L.band = 4.0f * R.band;
-                const int P0 = base + ((cs[row + ncx - 1] - rs) & ~3);
-                const int P1 = (act && xlo < 0) ? base + ((cs[row + ncx] - rs + 3) & ~3) : P0;
-                scan_run<MODE, HALF, true, true>(ps, P0, P1, L, S.rl2f, S.rl2d, code, uint32_t(-ncx) & 3u, pos, &R, -ncx, oy, oz);
+                L.band = 4.0f * band;
+                const int rs = cs[row], base = cand_place(R, prow, rs) - P0;
+                const int g0 = (base + ((cs[row + ncx - 1] - rs) & ~3)) >> 2;
+                const int g1 = lo ? (base + ((cs[row + ncx] - rs + 3) & ~3)) >> 2 : g0;
+                scan_run<MODE, HALF, false>(ps, pent, g0, g1, L, my_runs + lane, S.rl2f, S.rl2d, tag | (1u << BG_IMG), 0u, pos, &R, -ncx, oy, oz);
             }
             {
                 L.nx = make_float2(-X, -X);
-                L.band = bandw;
-                const int P0 = base + ((cs[row + max(xlo, 0)] - rs) & ~3);
-                const int P1 = act ? base + ((cs[row + min(xhi, ncx - 1) + 1] - rs + 3) & ~3) : P0;
-                if (oy == 0) scan_run<MODE, HALF, true, false>(ps, P0, P1, L, S.rl2f, S.rl2d, code, 0u, pos, &R, 0, oy, oz);
-                else scan_run<MODE, HALF, false, false>(ps, P0, P1, L, S.rl2f, S.rl2d, code, 0u, pos, &R, 0, oy, oz);
+                L.band = (wy != 0.0f || wz != 0.0f) ? 4.0f * band : band;
+                const int2 run = A.crun[row + cx];
+                const int g1 = act ? run.y : run.x;
+                if (oy == 0)
+                    scan_run<MODE, HALF, true>(ps, pent, run.x, g1, L, my_runs + lane, S.rl2f, S.rl2d, tag, mine, pos, &R, 0, oy, oz);
+                else
+                    scan_run<MODE, HALF, false>(ps, pent, run.x, g1, L, my_runs + lane, S.rl2f, S.rl2d, tag, 0u, pos, &R, 0, oy, oz);
             }
-            if (any_hi) {
+            if (any_hi) {                             // the row's first cell, seen across the boundary
                 const float xs = X - float(ncx) * R.wf[0];
                 L.nx = make_float2(-xs, -xs);
-                L.band = 4.0f * R.band;
-                const int P0 = base;
-                const int P1 = (act && xhi >= ncx) ? base + ((cs[row + 1] - rs + 3) & ~3) : P0;
-                scan_run<MODE, HALF, true, true>(ps, P0, P1, L, S.rl2f, S.rl2d, code, uint32_t(ncx) & 3u, pos, &R, ncx, oy, oz);
+                L.band = 4.0f * band;
+                const int rs = cs[row], g0 = (cand_place(R, prow, rs) - P0) >> 2;
+                const int g1 = hi ? g0 + ((cs[row + 1] - rs + 3) >> 2) : g0;
+                scan_run<MODE, HALF, false>(ps, pent, g0, g1, L, my_runs + lane, S.rl2f, S.rl2d, tag | (2u << BG_IMG), 0u, pos, &R, ncx, oy, oz);
             }
         }
         // join the planes: entry m of atom a comes from plane 0, 1 or 2
@@ -789,18 +809,31 @@ __global__ void __launch_bounds__(TILE, MINB) k_build_group(Arrays A, Scal S, in
         const int c2 = __shfl_sync(0xffffffffu, cnt, a + 2 * BG_ATOMS);
         int m = c0 + c1 + c2;
         const int slot = int(L.self >> IDX_SHIFT);
-        const uint32_t cadd = uint32_t(1 - cx) & 3u;              // o_x + 1 = cell of j - cell of i + 1 (mod 4)
-        if (rows < S.cap && __any_sync(0xffffffffu, act && L.lost != 0)) {
+        // o_x + 1 = cell of j, shifted by its run's image, - cell of i + 1 (mod 4)
+        const uint32_t cadd = uint32_t(1 - cx);
+        if (__any_sync(0xffffffffu, act && (L.far || (rows < S.cap && L.lost != 0)))) {
             if (act && pl == 0)
                 m = build_column<MODE>(pos, &R, cs, A.perm, A.W, S.nslots, S.cap, S.rl2d, S.rl2f, HALF ? 1 : 0, slot, pc);
         } else if (act) {
             const int mc = min(m, S.cap);
             uint32_t* wp = A.W + int64_t(pl) * S.nslots + slot;
-            for (int q = pl; q < mc; q += 3, wp += 3 * S.nslots) {
-                const int src = (q < c0) ? q * 32 + a
-                                         : ((q < c0 + c1) ? (q - c0) * 32 + a + BG_ATOMS : (q - c0 - c1) * 32 + a + 2 * BG_ATOMS);
-                const uint32_t v = my_lists[src];
-                *wp = (v & ~3u) | ((v + cadd) & 3u);
+            for (int q0 = pl; q0 < mc; q0 += 12, wp += 12 * S.nslots) {
+                uint32_t e[4], img[4], code[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int q = q0 + 3 * u;
+                    const int oz1 = (q < c0) ? 0 : ((q < c0 + c1) ? 1 : 2), from = a + BG_ATOMS * oz1;
+                    const int m0 = (oz1 == 0) ? 0 : ((oz1 == 1) ? c0 : c0 + c1);
+                    const uint32_t v = q < mc ? my_lists[(q - m0) * 32 + from] : 0u;
+                    e[u] = __ldg(pent + (q < mc ? my_runs[32 * (v >> BG_OY) + from] + int(v & (BG_RUN - 1)) : 0));
+                    img[u] = v >> BG_IMG;
+                    code[u] = (((v >> BG_OY) & 3u) << 2) | (uint32_t(oz1) << 4);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const uint32_t ox = (e[u] + cadd + (img[u] == 2u ? uint32_t(ncx) : 0u) - (img[u] == 1u ? uint32_t(ncx) : 0u)) & 3u;
+                    if (q0 + 3 * u < mc) wp[int64_t(3 * u) * S.nslots] = (e[u] & ~63u) | ox | code[u];
+                }
             }
         }
         __syncwarp();
@@ -997,14 +1030,10 @@ cudaError_t launch_bin_order(const Arrays& A, const Scal& S, const Launch& L, in
     else if (S.mode == MD_MIXED) k_bin<MD_MIXED><<<resident_grid<k_bin<MD_MIXED>>(S, L), TILE, 0, L.stream>>>(A, S, cur, fs);
     else k_bin<MD_FP32><<<resident_grid<k_bin<MD_FP32>>(S, L), TILE, 0, L.stream>>>(A, S, cur, fs);
     launch_scan(A, ScanArgs{A.ccount, A.cstart, A.chunk, S.ncells, S.nchunks}, L.stream);
-    k_scatter<<<resident_grid<k_scatter>(S, L), TILE, 0, L.stream>>>(A, S);
+    k_scatter<<<resident_grid<k_scatter>(S, L), TILE, 0, L.stream>>>(A, S, L.step_kernel == 4 ? 1 : 0);
     if (S.mode == MD_FP64) k_order<MD_FP64><<<resident_grid<k_order<MD_FP64>>(S, L), TILE, 0, L.stream>>>(A, S, cur);
     else if (S.mode == MD_MIXED) k_order<MD_MIXED><<<resident_grid<k_order<MD_MIXED>>(S, L), TILE, 0, L.stream>>>(A, S, cur);
     else k_order<MD_FP32><<<resident_grid<k_order<MD_FP32>>(S, L), TILE, 0, L.stream>>>(A, S, cur);
-    if (L.step_kernel == 4) {
-        const int gs = int(std::min<int64_t>((S.ncells + 255) / 256, int64_t(L.grid) * 8));
-        k_cell_ranges<<<std::max(gs, 1), 256, 0, L.stream>>>(A, S);
-    }
     return cudaGetLastError();
 }
 
@@ -1033,73 +1062,63 @@ cudaError_t launch_bin_only(const Arrays& A, const Scal& S, const Launch& L, int
 // displacement rule needs the positions at the rebuild (written by the build)
 static bool skip_w(const Scal& S, const Launch& L) { return L.step_kernel == 4 && S.rule != MD_REBUILD_DISP; }
 
-int bin_kernels(const Scal&, const Launch& L) { return L.step_kernel == 4 ? 8 : 7; }
+int bin_kernels(const Scal&, const Launch&) { return 7; }
 
 int build_kernels(const Scal& S, const Launch& L) { return (skip_w(S, L) ? 0 : 1) + (L.step_kernel == 3 ? 1 : 0) + 1; }
 
-// The register bound: 8 CTAs per SM where the lists leave room for them (WCA, 2M atoms: 0.51 against
-// 0.59 ms at the 5 CTAs' bound), else 5, which the LJ lists allow and which spills nothing there.
 // The lists of k_build_group hold one z plane's neighbours of an atom.  A slab of thickness w >= r_l
 // around it holds up to 69 % of them; half as many again and 12 leave room for fluctuations, and
 // 60 % of the capacity for denser regions than the mean.  A longer list sends its unit through
-// build_column.  Four warps per CTA while their lists fit, else one.
-template <int MODE, bool HALF, int MINB>
-static void group_grid(Launch& L)
+// build_column.  One CTA per SM with as many warps as their lists allow,
+// up to 32; with room for fewer than 24 the kernel compiled for 20, which has more registers.
+template <int MODE, bool HALF, int WARPS>
+static void group_limit()
 {
-    // the opt-in limit once per kernel, the occupancy again when the shared memory changes
+    // the opt-in limit, once per kernel
     static const bool raised = [] {
         int optin = 0, dev = 0;
         cudaFuncAttributes fa;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        return cudaFuncGetAttributes(&fa, k_build_group<MODE, HALF, MINB>) == cudaSuccess &&
-               cudaFuncSetAttribute(k_build_group<MODE, HALF, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        return cudaFuncGetAttributes(&fa, k_build_group<MODE, HALF, WARPS>) == cudaSuccess &&
+               cudaFuncSetAttribute(k_build_group<MODE, HALF, WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     optin - int(fa.sharedSizeBytes)) == cudaSuccess;
     }();
     (void)raised;
-    static std::atomic<uint64_t> known{0};            // (shared memory, block) << 32 | CTAs per SM
-    const uint64_t key = uint64_t(uint32_t(L.bg_smem) | (L.bg_block == TILE ? 0x80000000u : 0u)) << 32;
-    const uint64_t seen = known.load(std::memory_order_relaxed);
-    int per_sm = 1;
-    if ((seen & 0xffffffff00000000ull) == key && uint32_t(seen) != 0) {
-        per_sm = int(uint32_t(seen));
-    } else {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_build_group<MODE, HALF, MINB>, L.bg_block, L.bg_smem) !=
-                cudaSuccess || per_sm < 1)
-            per_sm = 1;
-        known.store(key | uint32_t(per_sm), std::memory_order_relaxed);
-    }
-    L.bg_grid = L.nsm * per_sm;
 }
 
-// F(MODE, HALF, MINB) for the system's precision, list and list length
-#define GBMD_BUILD_MINB(M, H, F) { if (L.bg_minb == 8) F(M, H, 8); else F(M, H, 5); }
+// F(MODE, HALF, WARPS) for the system's precision, list and list length
+#define GBMD_BUILD_WARPS(M, H, F) { if (L.bg_warps == 32) F(M, H, 32); else F(M, H, 20); }
 #define GBMD_BUILD_DISPATCH(F)                                                                          \
-    if (S.mode == MD_FP64) GBMD_BUILD_MINB(MD_FP64, false, F)                                           \
-    else if (S.mode == MD_MIXED) { if (S.half_list) GBMD_BUILD_MINB(MD_MIXED, true, F) else GBMD_BUILD_MINB(MD_MIXED, false, F) } \
-    else { if (S.half_list) GBMD_BUILD_MINB(MD_FP32, true, F) else GBMD_BUILD_MINB(MD_FP32, false, F) }
+    if (S.mode == MD_FP64) GBMD_BUILD_WARPS(MD_FP64, false, F)                                           \
+    else if (S.mode == MD_MIXED) { if (S.half_list) GBMD_BUILD_WARPS(MD_MIXED, true, F) else GBMD_BUILD_WARPS(MD_MIXED, false, F) } \
+    else { if (S.half_list) GBMD_BUILD_WARPS(MD_FP32, true, F) else GBMD_BUILD_WARPS(MD_FP32, false, F) }
 
-void build_group_shape(const Scal& S, Launch& L, double mean_nbrs, int smem_per_cta, int smem_per_sm)
+void build_group_shape(const Scal& S, Launch& L, double mean_nbrs, int smem_per_cta)
 {
     const int room = smem_per_cta - 2048;
     const double want = std::max(0.69 * 1.35 * mean_nbrs + 12.0, 0.6 * S.cap);
     int rows = std::min(S.cap, int(std::min(want, 1.0e6)) + 1);
-    L.bg_block = ((rows + BG_STEP) * int(BG_ROW) * (TILE / 32) <= room) ? TILE : 32;
-    rows = std::min(rows, room / (int(BG_ROW) * (L.bg_block / 32)) - BG_STEP);
+    rows = std::min(rows, (room - BG_TABLE) / int(BG_ROW) - BG_STEP);
+    const int fit = room / (BG_TABLE + (rows + BG_STEP) * int(BG_ROW));
+    L.bg_warps = fit >= 24 ? 32 : 20;
+    L.bg_block = 32 * std::min(L.bg_warps, fit);
     L.bg_rows = rows;
-    L.bg_smem = (rows + BG_STEP) * int(BG_ROW) * (L.bg_block / 32);
-    L.bg_minb = (8 * (L.bg_smem + 1024) <= smem_per_sm && L.bg_block == TILE) ? 8 : 5;
-#define GBMD_GRID(M, H, B) group_grid<M, H, B>(L)
-    GBMD_BUILD_DISPATCH(GBMD_GRID)
-#undef GBMD_GRID
+    L.bg_smem = (BG_TABLE + (rows + BG_STEP) * int(BG_ROW)) * (L.bg_block / 32);
+#define GBMD_LIMIT(M, H, B) group_limit<M, H, B>()
+    GBMD_BUILD_DISPATCH(GBMD_LIMIT)
+#undef GBMD_LIMIT
 }
 
 cudaError_t launch_build_only(const Arrays& A, const Scal& S, const Launch& L, int cur)
 {
     if (!skip_w(S, L)) {
-        const int64_t units = int64_t(S.ntiles) * BG_UNITS, per_cta = L.bg_block / 32;
-        const int g = int(std::max<int64_t>(1, std::min<int64_t>(L.bg_grid, (units + per_cta - 1) / per_cta)));
-#define GBMD_BUILD(M, H, B) k_build_group<M, H, B><<<g, L.bg_block, L.bg_smem, L.stream>>>(A, S, cur, L.bg_rows)
+        // no more warps per CTA than units per SM (a CTA of 32 warps and 200 KB starts later)
+        const int64_t units = int64_t(S.ntiles) * BG_UNITS;
+        const int g = int(std::max<int64_t>(1, std::min<int64_t>(L.nsm, units)));
+        const int warps = int(std::min<int64_t>(L.bg_block / 32, (units + g - 1) / g));
+        const int block = 32 * warps, smem = L.bg_smem / (L.bg_block / 32) * warps;
+#define GBMD_BUILD(M, H, B) k_build_group<M, H, B><<<g, block, smem, L.stream>>>(A, S, cur, L.bg_rows)
         GBMD_BUILD_DISPATCH(GBMD_BUILD)
 #undef GBMD_BUILD
     }
