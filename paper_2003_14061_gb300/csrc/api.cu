@@ -226,7 +226,6 @@ size_t carve(const Plan& P, char* base, Arrays* A)
     a.tile_rep = c.take<int32_t>(size_t(P.ntiles));
     a.rb_tiles = c.take<int32_t>(size_t(P.ntiles));
     a.cell_rep = c.take<int32_t>(size_t(P.ncells));
-    a.rb_base = c.take<int32_t>(size_t(P.nrep));
     a.warp_part = c.take<double>(size_t(P.ntiles) * (TILE / 32) * NPROP);
     a.slice_part = c.take<double>(size_t(P.nrep) * props_split(P) * NPROP);
     a.rep = c.take<Rep>(size_t(P.nrep));

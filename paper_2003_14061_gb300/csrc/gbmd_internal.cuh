@@ -145,7 +145,6 @@ struct Arrays {
     int32_t* tile_rep;
     int32_t* rb_tiles;        // tiles of the replicas rebuilding in this step
     int32_t* cell_rep;        // replica of every (global) cell
-    int32_t* rb_base;         // per replica: its first entry in rb_tiles
     double* warp_part;        // NPROP per warp of every tile (32 slots): the props partials
     double* slice_part;       // NPROP per (replica, slice) of the final sums, props_split per replica
     // per replica
@@ -425,7 +424,7 @@ struct Launch {
     int build_block;
     int nbr_batch;            // W entries loaded together per thread in the pair loop (2, 4, 8)
     int ctas_req;             // requested resident CTAs/SM (register bound of the step kernel)
-    int step_single;          // step kernel 1: one warp per CTA and warp-tile, all of them resident at once
+    int step_single;          // step kernel 1: threads per CTA when every warp-tile has a warp of its own (0: claims)
     int bg_rows;              // k_build_group: rows of each lane's list in shared memory,
     int bg_block;             // threads per CTA (one CTA per SM), dynamic shared memory,
     int bg_smem;

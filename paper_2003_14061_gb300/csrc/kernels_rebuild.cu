@@ -53,10 +53,17 @@ __device__ void flush_stats(int64_t* sum_dst, int* max_dst, long long sum, int m
 // ------------------------------------------------------------------------------------------
 // The tiles of the replicas that rebuild in this step, listed contiguously so that the rebuild
 // kernels share them evenly among their CTAs (in a batch only some replicas rebuild per step).
+// Every CTA computes the replicas' positions in the list and fills those of its share of them, a
+// warp per replica: one CTA filling all of them in turn took 44 us of a step of 512 replicas.
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(1024) k_rebuild_list(Arrays A, Scal S)
 {
     if (!A.g->any_rebuild) return;
+    if (S.nrep == 1) {
+        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < S.ntiles; k += gridDim.x * blockDim.x) A.rb_tiles[k] = k;
+        if (blockIdx.x == 0 && threadIdx.x == 0) A.g->n_rb_tiles = S.ntiles;
+        return;
+    }
     __shared__ int sh[33];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int carry = 0;
@@ -83,17 +90,21 @@ __global__ void __launch_bounds__(1024) k_rebuild_list(Arrays A, Scal S)
             if (lane == 31) sh[32] = wi;
         }
         __syncthreads();
-        if (r < S.nrep) A.rb_base[r] = carry + sh[wid] + incl - v;
+        const int base = carry + sh[wid] + incl - v;
         carry += sh[32];
+        // this CTA's warps of replicas
+        const int w0 = (r0 >> 5) + wid;               // the replicas 32 w0 .. 32 w0 + 31
+        if (w0 % int(gridDim.x) == int(blockIdx.x)) {
+            for (unsigned todo = __ballot_sync(0xffffffffu, v > 0); todo; todo &= todo - 1) {
+                const int l = __ffs(todo) - 1;
+                const int nt = __shfl_sync(0xffffffffu, v, l), b = __shfl_sync(0xffffffffu, base, l);
+                const int t0 = A.rep[32 * w0 + l].tile0;
+                for (int k = lane; k < nt; k += 32) A.rb_tiles[b + k] = t0 + k;
+            }
+        }
         __syncthreads();
     }
-    if (threadIdx.x == 0) A.g->n_rb_tiles = carry;
-    // fill: replica by replica, all threads writing its consecutive tiles
-    for (int r = 0; r < S.nrep; ++r) {
-        if (!A.rs[r].rebuild) continue;
-        const int base = A.rb_base[r], t0 = A.rep[r].tile0, nt = A.rep[r].ntiles;
-        for (int k = threadIdx.x; k < nt; k += blockDim.x) A.rb_tiles[base + k] = t0 + k;
-    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) A.g->n_rb_tiles = carry;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -278,80 +289,96 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* sh_warp, int& to
     return r;
 }
 
-// The scan of n counters `count` into `start` (n + 1 entries), through per-chunk totals in
-// `chunk`; the counters are left at zero for the next binning.  Serves the cells and the half-side
-// sub-cells of the sub-cell neighbour build.
-struct ScanArgs {
-    int32_t* count;
-    int32_t* start;
-    int32_t* chunk;
-    int64_t n;
-    int32_t nchunks;
-};
+// The scan of the cells' occupancies into cstart (ncells + 1 entries), through per-chunk totals;
+// the counters are left at zero for the next binning.  Only the cells of rebuilding replicas have
+// atoms counted, and only their starts are read: a chunk of cells without any is passed over (in a
+// batch about a tenth of the replicas rebuilds in a step).
+__device__ __forceinline__ bool chunk_live(const Arrays& A, const Scal& S, int64_t c0)
+{
+    if (S.nrep == 1) return true;
+    const int r0 = A.cell_rep[c0], r1 = A.cell_rep[min(c0 + SCAN_CHUNK, int64_t(S.ncells)) - 1];
+    bool live = false;
+    for (int r = r0 + int(threadIdx.x); r <= r1; r += blockDim.x) live |= A.rs[r].rebuild != 0;
+    return __syncthreads_or(live) != 0;
+}
 
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_chunks(Arrays A, ScanArgs C)
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_chunks(Arrays A, Scal S)
 {
     if (!A.g->any_rebuild) return;
     __shared__ int sh[33];
-    const int64_t base = int64_t(blockIdx.x) * SCAN_CHUNK + threadIdx.x * SCAN_PER_THREAD;
-    int s = 0;
+    const int64_t c0 = int64_t(blockIdx.x) * SCAN_CHUNK;
+    int total = 0;
+    if (chunk_live(A, S, c0)) {
+        const int64_t base = c0 + threadIdx.x * SCAN_PER_THREAD;
+        int s = 0;
 #pragma unroll
-    for (int k = 0; k < SCAN_PER_THREAD; ++k) {
-        const int64_t c = base + k;
-        if (c < C.n) s += C.count[c];
+        for (int k = 0; k < SCAN_PER_THREAD; ++k) {
+            const int64_t c = base + k;
+            if (c < S.ncells) s += A.ccount[c];
+        }
+        block_exclusive_scan(s, sh, total);
     }
-    int total;
-    block_exclusive_scan(s, sh, total);
-    if (threadIdx.x == 0) C.chunk[blockIdx.x] = total;
+    if (threadIdx.x == 0) A.chunk[blockIdx.x] = total;
 }
 
-__global__ void __launch_bounds__(1024) k_scan_top(Arrays A, ScanArgs C)
+__global__ void __launch_bounds__(1024) k_scan_top(Arrays A, Scal S)
 {
     if (!A.g->any_rebuild) return;
     __shared__ int sh[33];
     int carry = 0;
-    for (int b0 = 0; b0 < C.nchunks; b0 += blockDim.x) {
+    for (int b0 = 0; b0 < S.nchunks; b0 += blockDim.x) {
         const int b = b0 + threadIdx.x;
-        const int v = (b < C.nchunks) ? C.chunk[b] : 0;
+        const int v = (b < S.nchunks) ? A.chunk[b] : 0;
         int total;
         const int ex = block_exclusive_scan(v, sh, total);
-        if (b < C.nchunks) C.chunk[b] = carry + ex;
+        if (b < S.nchunks) A.chunk[b] = carry + ex;
         carry += total;
     }
 }
 
-__global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(Arrays A, ScanArgs C)
+// SOLO: the only chunk, which needs neither the chunk totals nor the launch that adds them up
+template <bool SOLO>
+__global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(Arrays A, Scal S)
 {
     if (!A.g->any_rebuild) return;
     __shared__ int sh[33];
-    const int64_t base = int64_t(blockIdx.x) * SCAN_CHUNK + threadIdx.x * SCAN_PER_THREAD;
+    const int64_t c0 = int64_t(blockIdx.x) * SCAN_CHUNK;
+    if (!chunk_live(A, S, c0)) return;
+    const int64_t base = c0 + threadIdx.x * SCAN_PER_THREAD;
     int v[SCAN_PER_THREAD];
     int s = 0;
 #pragma unroll
     for (int k = 0; k < SCAN_PER_THREAD; ++k) {
         const int64_t c = base + k;
-        v[k] = (c < C.n) ? C.count[c] : 0;
+        v[k] = (c < S.ncells) ? A.ccount[c] : 0;
         s += v[k];
     }
     int total;
-    int run = C.chunk[blockIdx.x] + block_exclusive_scan(s, sh, total);
+    int run = block_exclusive_scan(s, sh, total) + (SOLO ? 0 : A.chunk[blockIdx.x]);
+    const int64_t end = min(c0 + SCAN_CHUNK, int64_t(S.ncells));
 #pragma unroll
     for (int k = 0; k < SCAN_PER_THREAD; ++k) {
         const int64_t c = base + k;
-        if (c < C.n) {
-            C.start[c] = run;
-            C.count[c] = 0;               // ready for the next binning
+        if (c < end) {
+            A.cstart[c] = run;
+            A.ccount[c] = 0;               // ready for the next binning
             run += v[k];
-            if (c == C.n - 1) C.start[C.n] = run;
+            if (c == end - 1) A.cstart[end] = run;      // also the start of the next chunk, if that is passed over
         }
     }
 }
 
-static void launch_scan(const Arrays& A, const ScanArgs& C, cudaStream_t st)
+static bool solo_scan(const Scal& S) { return S.nchunks == 1; }
+
+static void launch_scan(const Arrays& A, const Scal& S, cudaStream_t st)
 {
-    k_scan_chunks<<<C.nchunks, SCAN_THREADS, 0, st>>>(A, C);
-    k_scan_top<<<1, 1024, 0, st>>>(A, C);
-    k_scan_apply<<<C.nchunks, SCAN_THREADS, 0, st>>>(A, C);
+    if (solo_scan(S)) {
+        k_scan_apply<true><<<1, SCAN_THREADS, 0, st>>>(A, S);
+        return;
+    }
+    k_scan_chunks<<<S.nchunks, SCAN_THREADS, 0, st>>>(A, S);
+    k_scan_top<<<1, 1024, 0, st>>>(A, S);
+    k_scan_apply<false><<<S.nchunks, SCAN_THREADS, 0, st>>>(A, S);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1024,12 +1051,13 @@ cudaError_t launch_force_rebuild(const Arrays& A, const Scal& S, const Launch& L
 
 cudaError_t launch_bin_order(const Arrays& A, const Scal& S, const Launch& L, int cur, bool from_set)
 {
-    k_rebuild_list<<<1, 1024, 0, L.stream>>>(A, S);
+    const int gl = S.nrep == 1 ? (S.ntiles + 4095) / 4096 : (S.nrep + 31) / 32;
+    k_rebuild_list<<<std::max(1, std::min(gl, L.nsm)), S.nrep == 1 ? std::min(1024, (S.ntiles + 31) / 32 * 32) : 1024, 0, L.stream>>>(A, S);
     const int fs = from_set ? 1 : 0;
     if (S.mode == MD_FP64) k_bin<MD_FP64><<<resident_grid<k_bin<MD_FP64>>(S, L), TILE, 0, L.stream>>>(A, S, cur, fs);
     else if (S.mode == MD_MIXED) k_bin<MD_MIXED><<<resident_grid<k_bin<MD_MIXED>>(S, L), TILE, 0, L.stream>>>(A, S, cur, fs);
     else k_bin<MD_FP32><<<resident_grid<k_bin<MD_FP32>>(S, L), TILE, 0, L.stream>>>(A, S, cur, fs);
-    launch_scan(A, ScanArgs{A.ccount, A.cstart, A.chunk, S.ncells, S.nchunks}, L.stream);
+    launch_scan(A, S, L.stream);
     k_scatter<<<resident_grid<k_scatter>(S, L), TILE, 0, L.stream>>>(A, S, L.step_kernel == 4 ? 1 : 0);
     if (S.mode == MD_FP64) k_order<MD_FP64><<<resident_grid<k_order<MD_FP64>>(S, L), TILE, 0, L.stream>>>(A, S, cur);
     else if (S.mode == MD_MIXED) k_order<MD_MIXED><<<resident_grid<k_order<MD_MIXED>>(S, L), TILE, 0, L.stream>>>(A, S, cur);
@@ -1062,7 +1090,7 @@ cudaError_t launch_bin_only(const Arrays& A, const Scal& S, const Launch& L, int
 // displacement rule needs the positions at the rebuild (written by the build)
 static bool skip_w(const Scal& S, const Launch& L) { return L.step_kernel == 4 && S.rule != MD_REBUILD_DISP; }
 
-int bin_kernels(const Scal&, const Launch&) { return 7; }
+int bin_kernels(const Scal& S, const Launch&) { return solo_scan(S) ? 5 : 7; }
 
 int build_kernels(const Scal& S, const Launch& L) { return (skip_w(S, L) ? 0 : 1) + (L.step_kernel == 3 ? 1 : 0) + 1; }
 
