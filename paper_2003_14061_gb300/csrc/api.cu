@@ -461,17 +461,22 @@ int apply_tuning(md_system* s)
     stage_shape(per_sm, s->smem_per_sm, &s->L.stage_cap, &s->L.stage_smem);
     build_group_shape(s->S, s->L, s->plan.mean_nbrs, s->smem_per_cta);
     // Step-kernel shape.  One that md_set_tuning never named is chosen by size: 4 CTAs per SM with 8
-    // W entries together (120 registers) up to 1.5M atoms and at 30 neighbours or more, else 8 CTAs
+    // W entries together (120 registers) up to 600k atoms and at 30 neighbours or more, else 8 CTAs
     // and 2 entries, whose warps hide the HBM latency that the larger fluids wait for.  Step kernel,
     // 4/8 against 8/2: LJ 256k atoms 59 / 71 us, 1M 176 / 198, 6.9M 1127 / 1158; WCA 108k 25 / 31,
-    // 1M 72 / 74 (with props 85 / 91), 4M 244 / 206.
+    // 1M 72 / 74 (density 1.0: 70 / 67), 4M 244 / 206.
+    // Up to 40 warp-tiles per SM every warp-tile gets a warp of its own and none claims or steals
+    // tiles: up to 16 per SM one warp per CTA in the wide shape, which spreads them over all SMs
+    // (4000 LJ atoms 71 -> 11 us), else CTAs of 4 in the 8/2 shape, of which an SM holds 32 (100k WCA
+    // atoms 16 us against 22 with claims, 108k LJ 32 against 39, 187k WCA in 64 replicas 27 against
+    // 35; at 389k atoms, 80 per SM, the claims' locality wins, 36 against 41).
     const bool chosen = s->shape_set || s->L.step_kernel != 1;
-    const bool wide = !chosen && (s->plan.mean_nbrs >= 30.0 || s->plan.nslots <= 1500000);
+    const int per_sm_tiles = (s->plan.ntiles * (TILE / 32) + s->nsm - 1) / s->nsm;
+    s->L.step_single = (chosen || per_sm_tiles > 40) ? 0 : (per_sm_tiles <= 16 ? 32 : TILE);
+    const bool wide = !chosen && (s->L.step_single == 32 ||
+                                  (s->L.step_single == 0 && (s->plan.mean_nbrs >= 30.0 || s->plan.nslots <= 600000)));
     const int step_ctas = wide ? 4 : per_sm;
     if (wide) s->L.nbr_batch = 8;
-    // up to 16 warp-tiles per SM every warp-tile gets a warp of its own, one per CTA, so that they
-    // spread over all SMs and none claims or steals tiles
-    s->L.step_single = !chosen && s->plan.ntiles * (TILE / 32) <= s->nsm * 16;
     s->L.ctas_req = step_ctas;
     // a persistent grid larger than what can be resident would run as a trailing second wave
     s->L.grid_step = s->nsm * std::min(step_ctas, step_ctas_per_sm(s->S, s->L));

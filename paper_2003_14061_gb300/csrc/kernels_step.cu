@@ -1912,7 +1912,7 @@ cudaError_t launch_step(const Arrays& A, const Scal& S, const Launch& L, int cur
         if (props) k_step_sm<M, true, NB, MB><<<gs, bs, 0, L.stream>>>(A, S, cur, L.cond, L.use_cond);         \
         else k_step_sm<M, false, NB, MB><<<gs, bs, 0, L.stream>>>(A, S, cur, L.cond, L.use_cond);               \
     }
-        const int gs = L.step_single ? S.ntiles * (TILE / 32) : g, bs = L.step_single ? 32 : TILE;
+        const int bs = L.step_single ? L.step_single : TILE, gs = L.step_single ? S.ntiles * (TILE / bs) : g;
         if (S.mode == MD_FP64) GBMD_STEP(MD_FP64, 4, 4)
         else if (S.mode == MD_MIXED) GBMD_DISPATCH_NB_MINB(MD_MIXED, GBMD_STEP)
         else GBMD_DISPATCH_NB_MINB(MD_FP32, GBMD_STEP)
