@@ -1043,14 +1043,13 @@ int dyn_shape(const md_system* s, int32_t nlag, int32_t origin_every, int32_t* n
     return MD_OK;
 }
 
-size_t dyn_carve(int64_t n, int32_t nlag, char* base, DynView* V)
+size_t dyn_carve(int64_t n, int32_t nlag, int32_t norg, char* base, DynView* V)
 {
     Carver c{base};
     DynView d{};
     d.n = n;
-    d.xprev = c.take<double>(size_t(n) * 3);
-    d.v0 = c.take<double>(size_t(DYN_MAX_ORG) * n * 3);
-    d.dr = c.take<double>(size_t(DYN_MAX_ORG) * n * 3);
+    d.xprev = c.take<double4_32a>(size_t(n));
+    d.org = c.take<double4_32a>(size_t(norg) * n * 2);
     d.part = c.take<double>(size_t(DYN_BLOCKS) * 2 * DYN_MAX_ORG);
     d.vacf = c.take<double>(size_t(nlag));
     d.msd = c.take<double>(size_t(nlag));
@@ -1063,7 +1062,7 @@ size_t md_dyn_workspace_bytes(const md_system* s, int32_t nlag, int32_t origin_e
 {
     int32_t norg = 0;
     if (dyn_shape(s, nlag, origin_every, &norg) != MD_OK) return 0;
-    return dyn_carve(s->plan.n_total, nlag, nullptr, nullptr);
+    return dyn_carve(s->plan.n_total, nlag, norg, nullptr, nullptr);
 }
 
 int md_dyn_begin(md_system* s, void* d_work, size_t work_bytes, int32_t nlag, int32_t origin_every)
@@ -1071,11 +1070,11 @@ int md_dyn_begin(md_system* s, void* d_work, size_t work_bytes, int32_t nlag, in
     int32_t norg = 0;
     int rc = dyn_shape(s, nlag, origin_every, &norg);
     if (rc) return rc;
-    const size_t need = dyn_carve(s->plan.n_total, nlag, nullptr, nullptr);
+    const size_t need = dyn_carve(s->plan.n_total, nlag, norg, nullptr, nullptr);
     if (!d_work || (reinterpret_cast<uintptr_t>(d_work) & 255u) || work_bytes < need)
         return fail(MD_ERR_WORKSPACE, "measurement buffer missing, misaligned or smaller than " + std::to_string(need) +
                                           " bytes");
-    dyn_carve(s->plan.n_total, nlag, static_cast<char*>(d_work), &s->dyn);
+    dyn_carve(s->plan.n_total, nlag, norg, static_cast<char*>(d_work), &s->dyn);
     GBMD_CUDA(cudaMemsetAsync(s->dyn.vacf, 0, sizeof(double) * size_t(nlag), s->L.stream));
     GBMD_CUDA(cudaMemsetAsync(s->dyn.msd, 0, sizeof(double) * size_t(nlag), s->L.stream));
     s->dyn_on = true;

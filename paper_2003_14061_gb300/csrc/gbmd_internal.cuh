@@ -206,9 +206,8 @@ constexpr int DYN_MAX_ORG = 8;            // time origins followed at once
 constexpr int DYN_BLOCKS = 1024;          // CTAs of the sample kernel (partial sums per CTA)
 struct DynView {
     int64_t n;                // atoms (all replicas)
-    double* xprev;            // [n][3] wrapped positions of the previous sample
-    double* v0;               // [DYN_MAX_ORG][n][3] velocities at each origin
-    double* dr;               // [DYN_MAX_ORG][n][3] displacements since each origin
+    double4_32a* xprev;       // [n] wrapped positions of the previous sample
+    double4_32a* org;         // [origins][n][2] velocities at each origin, displacements since it
     double* part;             // [DYN_BLOCKS][2 DYN_MAX_ORG] per-CTA sums of one sample
     double* vacf;             // [nlag] sums over origins and atoms
     double* msd;              // [nlag]

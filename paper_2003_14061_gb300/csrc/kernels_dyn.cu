@@ -7,7 +7,12 @@
 //                 periodic positions), the integer-step velocity v_n = v + c f (the forces were
 //                 just evaluated), and for every time origin that is being followed the products
 //                 v_i(t0) . v_i(t) and |r_i(t) - r_i(t0)|^2, summed per CTA in FP64.
-//   k_dyn_finish  adds the CTAs' sums in CTA order into the per-lag accumulators (deterministic).
+//                 An atom's records are 32-byte vectors, one memory access each wherever its id lies
+//                 (as three doubles each was three scattered accesses).  Bound by the FP64 pipe, 1/64
+//                 of the FP32 rate: the boundary tests and the count of periods run outside it.
+//   k_dyn_finish  adds the CTAs' sums into the per-lag accumulators, a warp per quantity, in an
+//                 order fixed by the launch (deterministic).  One thread per quantity adding 1024
+//                 sums one after the other took 74 us.
 #include <algorithm>
 
 #include "gbmd_internal.cuh"
@@ -43,37 +48,47 @@ __global__ void __launch_bounds__(TILE) k_dyn_sample(Arrays A, Scal S, DynView D
         const int vhalf = A.rs[r].vhalf;
         const double4_32a f = vhalf ? A.f[slot] : make_double4_32a(0, 0, 0, 0);
         const double fq[3] = {f.x, f.y, f.z};
-        double vn[3], d[3];
+        double vn[3], x[3];
+        const float invL[3] = {1.0f / float(R.L[0]), 1.0f / float(R.L[1]), 1.0f / float(R.L[2])};
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             double xa = __dadd_rn(__dmul_rn(double(c[a]), R.w[a]), loc[a]);
-            if (xa < 0.0) xa += R.L[a];
-            if (xa >= R.L[a]) xa -= R.L[a];
+            // x < 0 and x >= L on the bit patterns (for x >= 0 they order as the values do)
+            if (__double_as_longlong(xa) < 0) xa += R.L[a];
+            if (__double_as_longlong(xa) >= __double_as_longlong(R.L[a])) xa -= R.L[a];
             double v = (S.mode == MD_FP32) ? double(A.v32[a][slot]) : A.v[a][slot];
             if (vhalf) {
                 if (S.mode == MD_FP32) v = double(fmaf(float(S.c), float(fq[a]), float(v)));
                 else v = fma(S.c, fq[a], v);
             }
             vn[a] = v;
-            // displacement since the previous sample: the minimum image of the wrapped difference
-            const double dd = xa - D.xprev[id * 3 + a];
-            d[a] = dd - R.L[a] * rint(dd / R.L[a]);
-            D.xprev[id * 3 + a] = xa;
+            x[a] = xa;
         }
+        // displacement since the previous sample: the minimum image of the wrapped difference (the
+        // number of periods, nearly always 0, from FP32)
+        const double4_32a xp = D.xprev[id];
+        double d[3] = {x[0] - xp.x, x[1] - xp.y, x[2] - xp.z};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const float k = rintf(float(d[a]) * invL[a]);
+            if (k != 0.0f) d[a] -= R.L[a] * double(k);
+        }
+        D.xprev[id] = make_double4_32a(x[0], x[1], x[2], 0.0);
 #pragma unroll
         for (int b = 0; b < DYN_MAX_ORG; ++b) {
             if (b >= P.norg) break;
-            double* v0 = D.v0 + (int64_t(b) * D.n + id) * 3;
-            double* dr = D.dr + (int64_t(b) * D.n + id) * 3;
+            double4_32a* o = D.org + (int64_t(b) * D.n + id) * 2;         // v(t0), displacement since t0
             if (b == P.start) {
-                v0[0] = vn[0]; v0[1] = vn[1]; v0[2] = vn[2];
-                dr[0] = 0.0; dr[1] = 0.0; dr[2] = 0.0;
+                o[0] = make_double4_32a(vn[0], vn[1], vn[2], 0.0);
+                o[1] = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+                if (P.lag[b] >= 0) acc[2 * b] += vn[0] * vn[0] + vn[1] * vn[1] + vn[2] * vn[2];
             } else if (P.lag[b] >= 0) {
-                dr[0] += d[0]; dr[1] += d[1]; dr[2] += d[2];
-            }
-            if (P.lag[b] >= 0) {
-                acc[2 * b] += vn[0] * v0[0] + vn[1] * v0[1] + vn[2] * v0[2];
-                acc[2 * b + 1] += dr[0] * dr[0] + dr[1] * dr[1] + dr[2] * dr[2];
+                const double4_32a v0 = o[0];
+                double4_32a r = o[1];
+                r.x += d[0]; r.y += d[1]; r.z += d[2];
+                o[1] = r;
+                acc[2 * b] += vn[0] * v0.x + vn[1] * v0.y + vn[2] * v0.z;
+                acc[2 * b + 1] += r.x * r.x + r.y * r.y + r.z * r.z;
             }
         }
     }
@@ -91,16 +106,18 @@ __global__ void __launch_bounds__(TILE) k_dyn_sample(Arrays A, Scal S, DynView D
     }
 }
 
-__global__ void k_dyn_finish(DynView D, DynStep P, int nblocks)
+// one warp per quantity, its lanes the CTAs' sums in turn, then a butterfly: the same order every time
+__global__ void __launch_bounds__(32 * 2 * DYN_MAX_ORG) k_dyn_finish(DynView D, DynStep P, int nblocks)
 {
-    const int q = threadIdx.x;                       // 2 b + (0: VACF, 1: MSD)
+    const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;        // 2 b + (0: VACF, 1: MSD)
     if (q >= 2 * P.norg) return;
     const int b = q >> 1;
     if (P.lag[b] < 0) return;
     double s = 0.0;
-    for (int k = 0; k < nblocks; ++k) s += D.part[int64_t(k) * 2 * DYN_MAX_ORG + q];
+    for (int k = lane; k < nblocks; k += 32) s += D.part[int64_t(k) * 2 * DYN_MAX_ORG + q];
+    s = warp_sum(s);
     double* dst = (q & 1) ? D.msd : D.vacf;
-    dst[P.lag[b]] += s;                              // one origin per lag per sample: no race
+    if (lane == 0) dst[P.lag[b]] += s;               // one origin per lag per sample: no race
 }
 
 cudaError_t launch_dyn_sample(const Arrays& A, const Scal& S, const Launch& L, const DynView& D, const DynStep& P,
@@ -108,7 +125,7 @@ cudaError_t launch_dyn_sample(const Arrays& A, const Scal& S, const Launch& L, c
 {
     const int g = std::max(1, std::min(std::min(L.grid, DYN_BLOCKS), S.ntiles));
     k_dyn_sample<<<g, TILE, 0, L.stream>>>(A, S, D, P, cur);
-    k_dyn_finish<<<1, 2 * DYN_MAX_ORG, 0, L.stream>>>(D, P, g);
+    k_dyn_finish<<<1, 32 * 2 * DYN_MAX_ORG, 0, L.stream>>>(D, P, g);
     return cudaGetLastError();
 }
 
