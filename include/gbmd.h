@@ -356,7 +356,7 @@ int md_destroy(md_system* s);
  * plug-ins running between someone else's kernels where the synchronisation of cudaMalloc/
  * cudaFree is not allowed, code with no workspace to hand -- this computes f_i and u_i as
  * md_compute_forces does (FP32 pair arithmetic on cell-local coordinates), over a plain cell
- * list of side >= rc (skin is ignored) kept in one file-scope device array of 1.75 MiB that
+ * list of side >= rc (skin is ignored) kept in one file-scope device array of 3.25 MiB that
  * every GPU loading the library holds until exit.  The atoms of each cell are visited in index
  * order, so repeated calls on the same input return the same bits.
  *   p      : eps, sigma, rc, shift_energy and box are used; the rest is ignored.
