@@ -217,6 +217,7 @@ size_t carve(const Plan& P, char* base, Arrays* A)
     if (!f32) for (int q = 0; q < 3; ++q) a.tmp_d[q] = c.take<double>(ns);
     for (int q = 0; q < 3; ++q) a.tmp_v[q] = c.take<double>(ns);
     for (int q = 0; q < 2; ++q) a.tmp_i[q] = c.take<int32_t>(ns);
+    a.tmp_id = c.take<int32_t>(ns);
     if (f64) a.tmp_p64 = c.take<double4_32a>(ns);
     else a.tmp_p32 = c.take<float4>(ns);
     a.ccount = c.take<int32_t>(size_t(P.ncells));
@@ -733,6 +734,7 @@ int md_create_batch(const md_params* p, int32_t nrep, const int64_t* n_rep, cons
         cudaMemcpyAsync(s->A.cell_rep, s->plan.cell_rep.data(), sizeof(int32_t) * s->plan.ncells,
                         cudaMemcpyHostToDevice, s->L.stream) != cudaSuccess)
         return bail(fail(MD_ERR_CUDA, "upload of the replica table"));
+    if (s->plan.nrep == 1 && launch_all_tiles(s->A, s->S, s->L) != cudaSuccess) return bail(fail(MD_ERR_CUDA, "tile list"));
     rc = load_state(s, x0, v0);
     if (rc) return bail(rc);
     rc = latch_error(s);

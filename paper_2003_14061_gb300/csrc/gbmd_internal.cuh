@@ -97,7 +97,7 @@ struct Global {               // device-wide words
     int32_t err;              // ErrBits, latched
     int32_t max_nbr_seen;     // largest m_i that overflowed
     int32_t n_rb_tiles;       // entries of rb_tiles for the rebuild in progress
-    int32_t pad;
+    int32_t build_done;       // CTAs of the build that have finished
     long long graph_rebuilds; // rebuild sequences that ran inside captured graphs
 };
 
@@ -131,7 +131,8 @@ struct Arrays {
     // reorder scratch, per slot
     double* tmp_d[3];
     double* tmp_v[3];
-    int32_t* tmp_i[2];
+    int32_t* tmp_i[2];        // slots by cell in layer order; cells
+    int32_t* tmp_id;
     float4* tmp_p32;
     double4_32a* tmp_p64;
     // per cell
@@ -447,6 +448,7 @@ int set_last_error(int code, const char* msg);
 cudaError_t launch_debug_error(const Arrays& A, const Launch& L, int bits, int nbr_seen);
 
 // rebuild path (kernels_rebuild.cu)
+cudaError_t launch_all_tiles(const Arrays& A, const Scal& S, const Launch& L);           // creation, one system
 cudaError_t launch_force_rebuild(const Arrays& A, const Scal& S, const Launch& L, int reorder);
 void prime_rebuild_grids(const Scal& S, const Launch& L);
 cudaError_t launch_rebuild(const Arrays& A, const Scal& S, const Launch& L, int cur, bool from_set);
@@ -455,7 +457,7 @@ cudaError_t launch_bin_order(const Arrays& A, const Scal& S, const Launch& L, in
 cudaError_t launch_reorder(const Arrays& A, const Scal& S, const Launch& L, int cur);
 cudaError_t launch_build_only(const Arrays& A, const Scal& S, const Launch& L, int cur);
 int bin_kernels(const Scal& S, const Launch& L);     // kernels of launch_bin_order
-constexpr int REORDER_KERNELS = 2;                   // kernels of launch_reorder
+constexpr int REORDER_KERNELS = 1;                   // kernels of launch_reorder
 int build_kernels(const Scal& S, const Launch& L);   // kernels of launch_build_only
 // rows of k_build_group's lists, its CTA size, shared memory and grid, into L
 void build_group_shape(const Scal& S, Launch& L, double mean_nbrs, int smem_per_cta);

@@ -11,7 +11,7 @@
 //                  irreproducibility); ranking each atom among its cell's slots makes the order,
 //                  and every result after it, deterministic.  It also writes the candidate array
 //                  psort that the build reads.
-//   k_reorder_*    Sec. 4.1 item 1: permute the atoms into cell order (gather through scratch).
+//   k_reorder_copy Sec. 4.1 item 1: the atoms into cell order, from the scratch that k_order filled.
 //   k_build_group  N5: W from the 27 neighbouring cells, units of 10 atoms per warp and a lane per
 //                  atom and z plane; W stored row-major for coalescing (Sec. 4.1 item 6).
 //   k_tile_windows the slot window of each tile's W entries per row of neighbour cells, read by
@@ -59,11 +59,6 @@ __device__ void flush_stats(int64_t* sum_dst, int* max_dst, long long sum, int m
 __global__ void __launch_bounds__(1024) k_rebuild_list(Arrays A, Scal S)
 {
     if (!A.g->any_rebuild) return;
-    if (S.nrep == 1) {
-        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < S.ntiles; k += gridDim.x * blockDim.x) A.rb_tiles[k] = k;
-        if (blockIdx.x == 0 && threadIdx.x == 0) A.g->n_rb_tiles = S.ntiles;
-        return;
-    }
     __shared__ int sh[33];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int carry = 0;
@@ -289,8 +284,9 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int* sh_warp, int& to
     return r;
 }
 
-// The scan of the cells' occupancies into cstart (ncells + 1 entries), through per-chunk totals;
-// the counters are left at zero for the next binning.  Only the cells of rebuilding replicas have
+// The scan of the cells' occupancies into cstart (ncells + 1 entries), through per-chunk totals; up
+// to SCAN_SOLO chunks in one launch whose CTAs each add up the counts before theirs (three launches
+// of a few us otherwise).  The scatter clears the counters for the next binning.  Only the cells of rebuilding replicas have
 // atoms counted, and only their starts are read: a chunk of cells without any is passed over (in a
 // batch about a tenth of the replicas rebuilds in a step).
 __device__ __forceinline__ bool chunk_live(const Arrays& A, const Scal& S, int64_t c0)
@@ -336,7 +332,6 @@ __global__ void __launch_bounds__(1024) k_scan_top(Arrays A, Scal S)
     }
 }
 
-// SOLO: the only chunk, which needs neither the chunk totals nor the launch that adds them up
 template <bool SOLO>
 __global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(Arrays A, Scal S)
 {
@@ -344,6 +339,19 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(Arrays A, Scal S)
     __shared__ int sh[33];
     const int64_t c0 = int64_t(blockIdx.x) * SCAN_CHUNK;
     if (!chunk_live(A, S, c0)) return;
+    int before = 0;
+    if (SOLO) {
+        // cells of replicas that do not rebuild count zero; c0 is a multiple of 4
+        const int4* __restrict__ cnt = reinterpret_cast<const int4*>(A.ccount);
+        int s = 0;
+        for (int q = threadIdx.x; q < int(c0 >> 2); q += SCAN_THREADS) {
+            const int4 v = __ldg(cnt + q);
+            s += (v.x + v.y) + (v.z + v.w);
+        }
+        block_exclusive_scan(s, sh, before);
+    } else {
+        before = A.chunk[blockIdx.x];
+    }
     const int64_t base = c0 + threadIdx.x * SCAN_PER_THREAD;
     int v[SCAN_PER_THREAD];
     int s = 0;
@@ -354,26 +362,26 @@ __global__ void __launch_bounds__(SCAN_THREADS) k_scan_apply(Arrays A, Scal S)
         s += v[k];
     }
     int total;
-    int run = block_exclusive_scan(s, sh, total) + (SOLO ? 0 : A.chunk[blockIdx.x]);
+    int run = before + block_exclusive_scan(s, sh, total);
     const int64_t end = min(c0 + SCAN_CHUNK, int64_t(S.ncells));
 #pragma unroll
     for (int k = 0; k < SCAN_PER_THREAD; ++k) {
         const int64_t c = base + k;
         if (c < end) {
             A.cstart[c] = run;
-            A.ccount[c] = 0;               // ready for the next binning
             run += v[k];
             if (c == end - 1) A.cstart[end] = run;      // also the start of the next chunk, if that is passed over
         }
     }
 }
 
-static bool solo_scan(const Scal& S) { return S.nchunks == 1; }
+constexpr int SCAN_SOLO = 32;
+static bool solo_scan(const Scal& S) { return S.nchunks <= SCAN_SOLO; }
 
 static void launch_scan(const Arrays& A, const Scal& S, cudaStream_t st)
 {
     if (solo_scan(S)) {
-        k_scan_apply<true><<<1, SCAN_THREADS, 0, st>>>(A, S);
+        k_scan_apply<true><<<S.nchunks, SCAN_THREADS, 0, st>>>(A, S);
         return;
     }
     k_scan_chunks<<<S.nchunks, SCAN_THREADS, 0, st>>>(A, S);
@@ -395,8 +403,8 @@ __global__ void __launch_bounds__(TILE) k_scatter(Arrays A, Scal S, int keep)
         const Rep& R = A.rep[r];
         const int64_t slot = int64_t(t) * TILE + threadIdx.x;
         if (slot - R.slot0 < R.n) A.tmp_i[0][cs[A.cell[slot]] + A.layer[slot]] = int32_t(slot);
-        // this tile's share of the replica's cells: their runs of candidates (keep: also their slot
-        // ranges, for the list-free step kernel)
+        // this tile's share of the replica's cells: their runs of candidates, their counters cleared
+        // (keep: also their slot ranges, for the list-free step kernel)
         const int tt = t - R.tile0, ncx = R.nc[0];
         const int c_end = int(int64_t(R.ncells) * (tt + 1) / R.ntiles);
         const int k0 = cs[R.cell0], P0 = cand_place(R, 0, k0);
@@ -407,6 +415,7 @@ __global__ void __launch_bounds__(TILE) k_scatter(Arrays A, Scal S, int keep)
             const int base = cand_place(R, prow, rs) - P0;
             A.crun[R.cell0 + c] = make_int2((base + ((row[max(cx - 1, 0)] - rs) & ~3)) >> 2,
                                             (base + ((row[min(cx + 1, ncx - 1) + 1] - rs + 3) & ~3)) >> 2);
+            A.ccount[R.cell0 + c] = 0;               // ready for the next binning
             if (keep) A.ckeep[R.cell0 + c] = make_int2(row[cx] - k0, row[cx + 1] - k0);
         }
     }
@@ -458,7 +467,23 @@ __global__ void __launch_bounds__(TILE) k_order(Arrays A, Scal S, int cur)
         const int prow = row_pos(R, cc[1], cc[2]);
         const int rs = cs[R.cell0 + prow * R.nc[0]], re = cs[R.cell0 + (prow + 1) * R.nc[0]];
         const int P = cand_place(R, prow, rs) + (k - rs);
-        const int64_t out_slot = A.rs[r].reorder ? R.slot0 + (k - cs[R.cell0]) : slot;
+        const bool reorder = A.rs[r].reorder != 0;
+        const int64_t out_slot = reorder ? R.slot0 + (k - cs[R.cell0]) : slot;
+        if (reorder) {                                // the atom's state to its new place in the scratch
+            if (MODE == MD_FP64) A.tmp_p64[out_slot] = A.pos64[cur][slot];
+            else A.tmp_p32[out_slot] = A.pos32[cur][slot];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                if (MODE == MD_FP32) {
+                    A.tmp_v[a][out_slot] = double(A.v32[a][slot]);
+                } else {
+                    A.tmp_d[a][out_slot] = A.xl[a][slot];
+                    A.tmp_v[a][out_slot] = A.v[a][slot];
+                }
+            }
+            A.tmp_i[1][out_slot] = c;
+            A.tmp_id[out_slot] = A.id[slot];
+        }
         cand_store(A.psort, A.pent, P, G[0], G[1], G[2], (uint32_t(out_slot) << IDX_SHIFT) | uint32_t(cc[0] & 3));
         A.pcell[k] = pc;
         if (k == re - 1)                              // far-away entries up to the group of 4
@@ -467,38 +492,9 @@ __global__ void __launch_bounds__(TILE) k_order(Arrays A, Scal S, int cur)
 }
 
 // ------------------------------------------------------------------------------------------
-// reorder (Sec. 4.1 item 1): new slot slot0 + j takes the j-th atom in cell order
+// reorder (Sec. 4.1 item 1): new slot slot0 + j takes the j-th atom in cell order, from the scratch
+// that k_order has filled
 // ------------------------------------------------------------------------------------------
-template <int MODE>
-__global__ void __launch_bounds__(TILE) k_reorder_gather(Arrays A, Scal S, int cur)
-{
-    if (!A.g->any_reorder) return;
-    const int nrb = A.g->n_rb_tiles;
-    for (int it = blockIdx.x; it < nrb; it += gridDim.x) {
-        const int t = A.rb_tiles[it];
-        const int r = A.tile_rep[t];
-        if (!A.rs[r].reorder) continue;
-        const Rep& R = A.rep[r];
-        const int64_t slot = int64_t(t) * TILE + threadIdx.x;
-        const int64_t j = slot - R.slot0;
-        if (j >= R.n) continue;
-        const int32_t src = A.perm[A.cstart[R.cell0] + j];
-        if (MODE == MD_FP32) {
-            A.tmp_p32[slot] = A.pos32[cur][src];
-            for (int a = 0; a < 3; ++a) A.tmp_v[a][slot] = double(A.v32[a][src]);
-        } else {
-            if (MODE == MD_FP64) A.tmp_p64[slot] = A.pos64[cur][src];
-            else A.tmp_p32[slot] = A.pos32[cur][src];
-            for (int a = 0; a < 3; ++a) {
-                A.tmp_d[a][slot] = A.xl[a][src];
-                A.tmp_v[a][slot] = A.v[a][src];
-            }
-        }
-        A.tmp_i[0][slot] = A.id[src];
-        A.tmp_i[1][slot] = A.cell[src];
-    }
-}
-
 template <int MODE>
 __global__ void __launch_bounds__(TILE) k_reorder_copy(Arrays A, Scal S, int cur)
 {
@@ -523,8 +519,9 @@ __global__ void __launch_bounds__(TILE) k_reorder_copy(Arrays A, Scal S, int cur
                 A.v[a][slot] = A.tmp_v[a][slot];
             }
         }
-        A.id[slot] = A.tmp_i[0][slot];
-        A.slot_of_id[A.tmp_i[0][slot]] = int32_t(slot);
+        const int32_t id = A.tmp_id[slot];
+        A.id[slot] = id;
+        A.slot_of_id[id] = int32_t(slot);
         A.cell[slot] = A.tmp_i[1][slot];
         A.perm[A.cstart[R.cell0] + int(j)] = int32_t(slot);
     }
@@ -712,8 +709,33 @@ __device__ __noinline__ int build_column(const void* pos, const Rep* Rp, const i
     return m;
 }
 
+// Bookkeeping after a rebuild, by one CTA.
+__device__ void rebuild_finish(const Arrays& A, const Scal& S, int in_graph)
+{
+    for (int r = threadIdx.x; r < S.nrep; r += blockDim.x) {
+        RepState& st = A.rs[r];
+        if (!st.rebuild) continue;
+        if (st.reorder) {
+            st.last_reorder = st.step;
+            st.reorders += 1;
+        }
+        st.reorder = 0;
+        st.rebuild = 0;
+        st.D = 0.0;
+        st.rebuilds += 1;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        A.g->any_rebuild = 0;
+        A.g->any_reorder = 0;
+        if (in_graph) A.g->graph_rebuilds += 1;
+    }
+}
+
+// finish: 1 when no kernel of the rebuild follows, so that the last CTA closes it (in_graph as
+// for k_rebuild_finish)
 template <int MODE, bool HALF, int WARPS>
-__global__ void __launch_bounds__(32 * WARPS, 1) k_build_group(Arrays A, Scal S, int cur, int rows)
+__global__ void __launch_bounds__(32 * WARPS, 1) k_build_group(Arrays A, Scal S, int cur, int rows, int finish, int in_graph)
 {
     extern __shared__ uint32_t s_list[];              // [warps][rows + BG_STEP][32]
     if (!A.g->any_rebuild) return;
@@ -884,6 +906,20 @@ __global__ void __launch_bounds__(32 * WARPS, 1) k_build_group(Arrays A, Scal S,
         }
     }
     if (run_r >= 0) flush_warp();
+    if (finish) {
+        // every CTA has read the rebuild flags by the time it counts itself in
+        __shared__ int last;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            last = atomicAdd(&A.g->build_done, 1) == int(gridDim.x) - 1;
+        }
+        __syncthreads();
+        if (!last) return;
+        if (threadIdx.x == 0) A.g->build_done = 0;
+        __threadfence();
+        rebuild_finish(A, S, in_graph);
+    }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -963,27 +999,18 @@ __global__ void __launch_bounds__(TILE) k_tile_windows(Arrays A, Scal S, int cur
 // ------------------------------------------------------------------------------------------
 // bookkeeping after a rebuild
 // ------------------------------------------------------------------------------------------
+// (k_build_group's last CTA; a launch of its own when there is no build)
 __global__ void k_rebuild_finish(Arrays A, Scal S, int in_graph)
 {
     if (!A.g->any_rebuild) return;
-    for (int r = threadIdx.x; r < S.nrep; r += blockDim.x) {
-        RepState& st = A.rs[r];
-        if (!st.rebuild) continue;
-        if (st.reorder) {
-            st.last_reorder = st.step;
-            st.reorders += 1;
-        }
-        st.reorder = 0;
-        st.rebuild = 0;
-        st.D = 0.0;
-        st.rebuilds += 1;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        A.g->any_rebuild = 0;
-        A.g->any_reorder = 0;
-        if (in_graph) A.g->graph_rebuilds += 1;
-    }
+    rebuild_finish(A, S, in_graph);
+}
+
+// The tile list of a single system: all its tiles, written once at creation.
+__global__ void k_all_tiles(Arrays A, Scal S)
+{
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < S.ntiles; t += gridDim.x * blockDim.x) A.rb_tiles[t] = t;
+    if (blockIdx.x == 0 && threadIdx.x == 0) A.g->n_rb_tiles = S.ntiles;
 }
 
 // Mark every replica for a rebuild (creation, md_set_state, md_bin_cells).
@@ -1035,12 +1062,15 @@ void prime_rebuild_grids(const Scal& S, const Launch& L)
     (void)resident_grid<k_order<MD_FP64>>(S, L);
     (void)resident_grid<k_order<MD_MIXED>>(S, L);
     (void)resident_grid<k_order<MD_FP32>>(S, L);
-    (void)resident_grid<k_reorder_gather<MD_FP64>>(S, L);
-    (void)resident_grid<k_reorder_gather<MD_MIXED>>(S, L);
-    (void)resident_grid<k_reorder_gather<MD_FP32>>(S, L);
     (void)resident_grid<k_reorder_copy<MD_FP64>>(S, L);
     (void)resident_grid<k_reorder_copy<MD_MIXED>>(S, L);
     (void)resident_grid<k_reorder_copy<MD_FP32>>(S, L);
+}
+
+cudaError_t launch_all_tiles(const Arrays& A, const Scal& S, const Launch& L)
+{
+    k_all_tiles<<<std::max(1, std::min(L.nsm, (S.ntiles + 255) / 256)), 256, 0, L.stream>>>(A, S);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_force_rebuild(const Arrays& A, const Scal& S, const Launch& L, int reorder)
@@ -1051,8 +1081,8 @@ cudaError_t launch_force_rebuild(const Arrays& A, const Scal& S, const Launch& L
 
 cudaError_t launch_bin_order(const Arrays& A, const Scal& S, const Launch& L, int cur, bool from_set)
 {
-    const int gl = S.nrep == 1 ? (S.ntiles + 4095) / 4096 : (S.nrep + 31) / 32;
-    k_rebuild_list<<<std::max(1, std::min(gl, L.nsm)), S.nrep == 1 ? std::min(1024, (S.ntiles + 31) / 32 * 32) : 1024, 0, L.stream>>>(A, S);
+    // a single system's list is all its tiles, written at creation
+    if (S.nrep > 1) k_rebuild_list<<<std::min((S.nrep + 31) / 32, L.nsm), 1024, 0, L.stream>>>(A, S);
     const int fs = from_set ? 1 : 0;
     if (S.mode == MD_FP64) k_bin<MD_FP64><<<resident_grid<k_bin<MD_FP64>>(S, L), TILE, 0, L.stream>>>(A, S, cur, fs);
     else if (S.mode == MD_MIXED) k_bin<MD_MIXED><<<resident_grid<k_bin<MD_MIXED>>(S, L), TILE, 0, L.stream>>>(A, S, cur, fs);
@@ -1067,14 +1097,10 @@ cudaError_t launch_bin_order(const Arrays& A, const Scal& S, const Launch& L, in
 
 cudaError_t launch_reorder(const Arrays& A, const Scal& S, const Launch& L, int cur)
 {
-#define GBMD_REORDER(M)                                                                               \
-    {                                                                                                 \
-        k_reorder_gather<M><<<resident_grid<k_reorder_gather<M>>(S, L), TILE, 0, L.stream>>>(A, S, cur); \
-        k_reorder_copy<M><<<resident_grid<k_reorder_copy<M>>(S, L), TILE, 0, L.stream>>>(A, S, cur);     \
-    }
-    if (S.mode == MD_FP64) GBMD_REORDER(MD_FP64)
-    else if (S.mode == MD_MIXED) GBMD_REORDER(MD_MIXED)
-    else GBMD_REORDER(MD_FP32)
+#define GBMD_REORDER(M) k_reorder_copy<M><<<resident_grid<k_reorder_copy<M>>(S, L), TILE, 0, L.stream>>>(A, S, cur)
+    if (S.mode == MD_FP64) GBMD_REORDER(MD_FP64);
+    else if (S.mode == MD_MIXED) GBMD_REORDER(MD_MIXED);
+    else GBMD_REORDER(MD_FP32);
 #undef GBMD_REORDER
     return cudaGetLastError();
 }
@@ -1090,9 +1116,12 @@ cudaError_t launch_bin_only(const Arrays& A, const Scal& S, const Launch& L, int
 // displacement rule needs the positions at the rebuild (written by the build)
 static bool skip_w(const Scal& S, const Launch& L) { return L.step_kernel == 4 && S.rule != MD_REBUILD_DISP; }
 
-int bin_kernels(const Scal& S, const Launch&) { return solo_scan(S) ? 5 : 7; }
+int bin_kernels(const Scal& S, const Launch&) { return (S.nrep > 1 ? 1 : 0) + (solo_scan(S) ? 4 : 6); }
 
-int build_kernels(const Scal& S, const Launch& L) { return (skip_w(S, L) ? 0 : 1) + (L.step_kernel == 3 ? 1 : 0) + 1; }
+int build_kernels(const Scal& S, const Launch& L)
+{
+    return skip_w(S, L) ? (L.step_kernel == 3 ? 2 : 1) : (L.step_kernel == 3 ? 3 : 1);
+}
 
 // The lists of k_build_group hold one z plane's neighbours of an atom.  A slab of thickness w >= r_l
 // around it holds up to 69 % of them; half as many again and 12 leave room for fluctuations, and
@@ -1140,18 +1169,19 @@ void build_group_shape(const Scal& S, Launch& L, double mean_nbrs, int smem_per_
 
 cudaError_t launch_build_only(const Arrays& A, const Scal& S, const Launch& L, int cur)
 {
+    const int finish = (!skip_w(S, L) && L.step_kernel != 3) ? 1 : 0;
     if (!skip_w(S, L)) {
         // no more warps per CTA than units per SM (a CTA of 32 warps and 200 KB starts later)
         const int64_t units = int64_t(S.ntiles) * BG_UNITS;
         const int g = int(std::max<int64_t>(1, std::min<int64_t>(L.nsm, units)));
         const int warps = int(std::min<int64_t>(L.bg_block / 32, (units + g - 1) / g));
         const int block = 32 * warps, smem = L.bg_smem / (L.bg_block / 32) * warps;
-#define GBMD_BUILD(M, H, B) k_build_group<M, H, B><<<g, block, smem, L.stream>>>(A, S, cur, L.bg_rows)
+#define GBMD_BUILD(M, H, B) k_build_group<M, H, B><<<g, block, smem, L.stream>>>(A, S, cur, L.bg_rows, finish, L.in_graph)
         GBMD_BUILD_DISPATCH(GBMD_BUILD)
 #undef GBMD_BUILD
     }
     if (L.step_kernel == 3) k_tile_windows<<<tile_grid(S, L), TILE, 0, L.stream>>>(A, S, cur, 1);
-    k_rebuild_finish<<<1, 256, 0, L.stream>>>(A, S, L.in_graph);
+    if (!finish) k_rebuild_finish<<<1, 256, 0, L.stream>>>(A, S, L.in_graph);
     return cudaGetLastError();
 }
 
