@@ -474,8 +474,8 @@ int apply_tuning(md_system* s)
     const bool chosen = s->shape_set || s->L.step_kernel != 1;
     const int per_sm_tiles = (s->plan.ntiles * (TILE / 32) + s->nsm - 1) / s->nsm;
     s->L.step_single = (chosen || per_sm_tiles > 40) ? 0 : (per_sm_tiles <= 16 ? 32 : TILE);
-    const bool wide = !chosen && (s->L.step_single == 32 ||
-                                  (s->L.step_single == 0 && (s->plan.mean_nbrs >= 30.0 || s->plan.nslots <= 600000)));
+    s->L.wide_pairs = s->plan.mean_nbrs >= 30.0 || s->plan.nslots <= 600000;
+    const bool wide = !chosen && (s->L.step_single == 32 || (s->L.step_single == 0 && s->L.wide_pairs));
     const int step_ctas = wide ? 4 : per_sm;
     if (wide) s->L.nbr_batch = 8;
     s->L.ctas_req = step_ctas;
@@ -503,13 +503,54 @@ int latch_error(md_system* s)
     return fail(MD_ERR_CUDA, "unknown device error word");
 }
 
+// Whether kernels may use the caller's array of `bytes` bytes in place of a copy: memory of the current
+// device, aligned for doubles, inside one allocation.  What does not pass is copied, and the copy
+// reports what is wrong with it.
+bool direct_ptr(const void* p, size_t bytes)
+{
+    if (!p || (reinterpret_cast<uintptr_t>(p) & 7u)) return false;
+    cudaPointerAttributes a;
+    int dev = -1;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (a.type != cudaMemoryTypeDevice || a.device != dev) return false;
+    using Range = int (*)(unsigned long long*, size_t*, unsigned long long);      // cuMemGetAddressRange
+    static const Range range = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult res;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &res) != cudaSuccess ||
+            res != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return reinterpret_cast<Range>(fn);
+    }();
+    unsigned long long base = 0, at = reinterpret_cast<uintptr_t>(p);
+    size_t size = 0;
+    return range && range(&base, &size, at) == 0 && at >= base && at - base <= size && bytes <= size - (at - base);
+}
+
+bool overlap(const void* p, const void* q, size_t bytes)
+{
+    const uintptr_t a = reinterpret_cast<uintptr_t>(p), b = reinterpret_cast<uintptr_t>(q);
+    return p && q && (a < b ? b - a : a - b) < bytes;
+}
+
 int load_state(md_system* s, const double* x, const double* v)
 {
     const size_t bytes = size_t(s->plan.n_total) * 3 * sizeof(double);
-    GBMD_CUDA(cudaMemcpyAsync(s->A.xchg[0], x, bytes, cudaMemcpyDefault, s->L.stream));
-    GBMD_CUDA(cudaMemcpyAsync(s->A.xchg[1], v, bytes, cudaMemcpyDefault, s->L.stream));
+    if (!direct_ptr(x, bytes)) {
+        GBMD_CUDA(cudaMemcpyAsync(s->A.xchg[0], x, bytes, cudaMemcpyDefault, s->L.stream));
+        x = s->A.xchg[0];
+    }
+    if (!direct_ptr(v, bytes)) {
+        GBMD_CUDA(cudaMemcpyAsync(s->A.xchg[1], v, bytes, cudaMemcpyDefault, s->L.stream));
+        v = s->A.xchg[1];
+    }
     s->cur = 0;
-    GBMD_CUDA(launch_set_state(s->A, s->S, s->L, s->cur));
+    GBMD_CUDA(launch_set_state(s->A, s->S, s->L, s->cur, x, v));
     GBMD_CUDA(launch_force_rebuild(s->A, s->S, s->L, 1));
     GBMD_CUDA(launch_rebuild(s->A, s->S, s->L, s->cur, true));
     s->host_step = 0;
@@ -948,14 +989,24 @@ int md_get_state(md_system* s, double* x, double* v, double* f)
     if (!s) return fail(MD_ERR_INVALID_ARG, "system is NULL");
     if (!x && !v && !f) return MD_OK;
     {
-        Phase t(s, MD_PHASE_OTHER, (v || f) ? 2 : 1);
-        if (v || f) GBMD_CUDA(launch_forces(s->A, s->S, s->L, s->cur));
-        GBMD_CUDA(launch_get_state(s->A, s->S, s->L, s->cur, v != nullptr, f != nullptr));
+        // straight into the caller's arrays where they are this device's memory and lie apart, else
+        // through the exchange buffers
+        const size_t bytes = size_t(s->plan.n_total) * 3 * sizeof(double);
+        const bool apart = !overlap(x, v, bytes) && !overlap(x, f, bytes) && !overlap(v, f, bytes);
+        StateOut O{x, v, f};
+        double** const out[3] = {&O.x, &O.v, &O.f};
+        bool staged[3] = {false, false, false};
+        for (int q = 0; q < 3; ++q)
+            if (*out[q] && !(apart && direct_ptr(*out[q], bytes))) {
+                *out[q] = s->A.xchg[q];
+                staged[q] = true;
+            }
+        Phase t(s, MD_PHASE_OTHER, 1);
+        GBMD_CUDA(launch_get_state(s->A, s->S, s->L, s->cur, O));
+        if (staged[0]) GBMD_CUDA(cudaMemcpyAsync(x, s->A.xchg[0], bytes, cudaMemcpyDefault, s->L.stream));
+        if (staged[1]) GBMD_CUDA(cudaMemcpyAsync(v, s->A.xchg[1], bytes, cudaMemcpyDefault, s->L.stream));
+        if (staged[2]) GBMD_CUDA(cudaMemcpyAsync(f, s->A.xchg[2], bytes, cudaMemcpyDefault, s->L.stream));
     }
-    const size_t bytes = size_t(s->plan.n_total) * 3 * sizeof(double);
-    if (x) GBMD_CUDA(cudaMemcpyAsync(x, s->A.xchg[0], bytes, cudaMemcpyDefault, s->L.stream));
-    if (v) GBMD_CUDA(cudaMemcpyAsync(v, s->A.xchg[1], bytes, cudaMemcpyDefault, s->L.stream));
-    if (f) GBMD_CUDA(cudaMemcpyAsync(f, s->A.xchg[2], bytes, cudaMemcpyDefault, s->L.stream));
     return latch_error(s);
 }
 
@@ -1268,21 +1319,14 @@ int adj_plan(const md_system* s, int32_t nsteps, int32_t ckpt_every, AdjPlan* P)
 // positions and integer-step velocities (id order) into device buffers x, v
 int adj_save(md_system* s, const Scal& S, int cur, double* x, double* v)
 {
-    GBMD_CUDA(launch_forces(s->A, S, s->L, cur));
-    GBMD_CUDA(launch_get_state(s->A, S, s->L, cur, true, false));
-    const size_t bytes = size_t(s->plan.n_total) * 3 * sizeof(double);
-    GBMD_CUDA(cudaMemcpyAsync(x, s->A.xchg[0], bytes, cudaMemcpyDeviceToDevice, s->L.stream));
-    GBMD_CUDA(cudaMemcpyAsync(v, s->A.xchg[1], bytes, cudaMemcpyDeviceToDevice, s->L.stream));
+    GBMD_CUDA(launch_get_state(s->A, S, s->L, cur, StateOut{x, v, nullptr}));
     return MD_OK;
 }
 
 // restart from a checkpoint: exact binning, reorder by cell, neighbour build
 int adj_load(md_system* s, const Scal& S, const double* x, const double* v)
 {
-    const size_t bytes = size_t(s->plan.n_total) * 3 * sizeof(double);
-    GBMD_CUDA(cudaMemcpyAsync(s->A.xchg[0], x, bytes, cudaMemcpyDeviceToDevice, s->L.stream));
-    GBMD_CUDA(cudaMemcpyAsync(s->A.xchg[1], v, bytes, cudaMemcpyDeviceToDevice, s->L.stream));
-    GBMD_CUDA(launch_set_state(s->A, S, s->L, 0));
+    GBMD_CUDA(launch_set_state(s->A, S, s->L, 0, x, v));
     GBMD_CUDA(launch_force_rebuild(s->A, S, s->L, 1));
     GBMD_CUDA(launch_rebuild(s->A, S, s->L, 0, true));
     return MD_OK;

@@ -424,6 +424,7 @@ struct Launch {
     int build_block;
     int nbr_batch;            // W entries loaded together per thread in the pair loop (2, 4, 8)
     int ctas_req;             // requested resident CTAs/SM (register bound of the step kernel)
+    int wide_pairs;           // force passes outside the step: 1 = 16 warps per SM with 8 entries, 0 = 32 with 2
     int step_single;          // step kernel 1: threads per CTA when every warp-tile has a warp of its own (0: claims)
     int bg_rows;              // k_build_group: rows of each lane's list in shared memory,
     int bg_block;             // threads per CTA (one CTA per SM), dynamic shared memory,
@@ -475,6 +476,8 @@ cudaError_t launch_adj_final(const AdjView& V, const Launch& L, int ntiles);
 cudaError_t launch_dyn_sample(const Arrays& A, const Scal& S, const Launch& L, const DynView& D, const DynStep& P,
                               int cur);
 
+// the state in id order to device memory ([n][3] each, NULL where not wanted)
+struct StateOut { double *x, *v, *f; };
 // step path (kernels_step.cu)
 // launches per step without the props: the half-list pairs and the chain terms run before the step
 inline int step_kernels(const Scal& S, const Launch& L)
@@ -490,9 +493,8 @@ void stage_shape(int ctas_per_sm, int smem_per_sm, int* cap, int* smem_bytes);
 cudaError_t launch_forces(const Arrays& A, const Scal& S, const Launch& L, int cur);
 cudaError_t launch_props(const Arrays& A, const Scal& S, const Launch& L, int cur, bool from_forces,
                          bool to_series);
-cudaError_t launch_get_state(const Arrays& A, const Scal& S, const Launch& L, int cur, bool want_v,
-                             bool want_f);
-cudaError_t launch_set_state(const Arrays& A, const Scal& S, const Launch& L, int cur);
+cudaError_t launch_get_state(const Arrays& A, const Scal& S, const Launch& L, int cur, const StateOut& O);
+cudaError_t launch_set_state(const Arrays& A, const Scal& S, const Launch& L, int cur, const double* x, const double* v);
 cudaError_t launch_get_cells(const Arrays& A, const Scal& S, const Launch& L, int32_t* out_by_id);
 cudaError_t launch_get_neighbours(const Arrays& A, const Scal& S, const Launch& L, int32_t* counts_by_id,
                                   int32_t* nbr_by_id, int32_t cap_out, int64_t id_lo, int64_t id_hi);

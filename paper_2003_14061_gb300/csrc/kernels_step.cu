@@ -1467,26 +1467,85 @@ __global__ void __launch_bounds__(TILE, 2) k_step_bulk(Arrays A, Scal S, int cur
 // ------------------------------------------------------------------------------------------
 // forces only (F1): f, u_i, per-atom virial
 // ------------------------------------------------------------------------------------------
-template <int MODE, bool CELLS = false>
-__global__ void __launch_bounds__(TILE) k_forces(Arrays A, Scal S, int cur)
+// One atom's state in id order (md_get_state): position wrapped into the box, velocity closed to the
+// integer step with the force fq, force.  Pointers may be NULL.
+template <int MODE>
+__device__ __forceinline__ void write_state(const Arrays& A, const Scal& S, const Rep& R, int64_t slot, int cur, int vhalf,
+                                            const double (&fq)[3], const StateOut& O)
 {
-    for (int t = blockIdx.x; t < S.ntiles; t += gridDim.x) {
-        const int r = A.tile_rep[t];
-        const Rep& R = A.rep[r];
-        const int64_t slot = int64_t(t) * TILE + threadIdx.x;
-        if (slot - R.slot0 >= R.n) continue;
+    const int64_t id = A.id[slot];
+    if (O.x) {
+        uint32_t pw;
+        double loc[3];
         if (MODE == MD_FP64) {
-            const double4_32a pi = A.pos64[cur][slot];
-            const AccD a = force_f64<4>(A, S, R, A.pos64[cur], slot, pi);
-            A.f[slot] = make_double4_32a(a.fx, a.fy, a.fz, a.u);
-            A.wvir[slot] = a.w;
+            pw = cell_bits(A.pos64[cur][slot].w);
+            loc[0] = A.xl[0][slot]; loc[1] = A.xl[1][slot]; loc[2] = A.xl[2][slot];
         } else {
-            const float4 pi = A.pos32[cur][slot];
-            AccF a = CELLS ? force_f32_cells(A, S, R, A.pos32[cur], slot, pi)
-                           : force_f32<4>(A, S, R, A.pos32[cur], slot, pi);
-            if (S.chain_len) add_buffer(A, slot, a);
-            A.f[slot] = make_double4_32a(a.fx, a.fy, a.fz, a.u);
-            A.wvir[slot] = a.w;
+            const float4 p = A.pos32[cur][slot];
+            pw = __float_as_uint(p.w);
+            if (MODE == MD_FP32) { loc[0] = p.x; loc[1] = p.y; loc[2] = p.z; }
+            else { loc[0] = A.xl[0][slot]; loc[1] = A.xl[1][slot]; loc[2] = A.xl[2][slot]; }
+        }
+        int c[3];
+        unpack_cell(pw, c[0], c[1], c[2]);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            double x = __dadd_rn(__dmul_rn(double(c[a]), R.w[a]), loc[a]);
+            if (x < 0.0) x += R.L[a];
+            if (x >= R.L[a]) x -= R.L[a];
+            O.x[id * 3 + a] = x;
+        }
+    }
+    if (O.v) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            double v = (MODE == MD_FP32) ? double(A.v32[a][slot]) : A.v[a][slot];
+            if (vhalf) {
+                if (MODE == MD_FP32) v = double(fmaf(float(S.c), float(fq[a]), float(v)));
+                else v = fma(S.c, fq[a], v);
+            }
+            O.v[id * 3 + a] = v;
+        }
+    }
+    if (O.f)
+        for (int a = 0; a < 3; ++a) O.f[id * 3 + a] = fq[a];
+}
+
+// F1 at the current positions.  OUT: straight into the state of md_get_state, where the forces are
+// needed for nothing else (as two kernels the forces went through memory in between); else into f
+// and wvir.  Every CTA takes a contiguous run of warp-tiles, its warps side by side, so that they
+// gather from one neighbourhood; few warp-tiles are spread over all SMs.
+template <int MODE, bool CELLS, bool OUT, int WARPS, int NB>
+__global__ void __launch_bounds__(32 * WARPS, 1) k_forces(Arrays A, Scal S, int cur, StateOut O)
+{
+    const int lane = threadIdx.x & 31, wpc = blockDim.x >> 5;
+    const int nwt = S.ntiles * (TILE / 32), per = (nwt + int(gridDim.x) - 1) / int(gridDim.x);
+    const int w_end = min(nwt, (int(blockIdx.x) + 1) * per);
+    for (int w = int(blockIdx.x) * per + int(threadIdx.x >> 5); w < w_end; w += wpc) {
+        const int r = A.tile_rep[w / (TILE / 32)];
+        const Rep& R = A.rep[r];
+        const int64_t slot = int64_t(w) * 32 + lane;
+        if (slot - R.slot0 >= R.n) continue;
+        const int vhalf = OUT ? A.rs[r].vhalf : 0;
+        double fq[3] = {0.0, 0.0, 0.0}, u = 0.0, wv = 0.0;
+        if (!OUT || O.f || (O.v && vhalf)) {
+            if constexpr (MODE == MD_FP64) {
+                const double4_32a pi = A.pos64[cur][slot];
+                const AccD a = force_f64<NB>(A, S, R, A.pos64[cur], slot, pi);
+                fq[0] = a.fx; fq[1] = a.fy; fq[2] = a.fz; u = a.u; wv = a.w;
+            } else {
+                const float4 pi = A.pos32[cur][slot];
+                AccF a = CELLS ? force_f32_cells(A, S, R, A.pos32[cur], slot, pi)
+                               : force_f32<NB>(A, S, R, A.pos32[cur], slot, pi);
+                if (S.chain_len) add_buffer(A, slot, a);
+                fq[0] = a.fx; fq[1] = a.fy; fq[2] = a.fz; u = a.u; wv = a.w;
+            }
+        }
+        if (OUT) {
+            write_state<MODE>(A, S, R, slot, cur, vhalf, fq, O);
+        } else {
+            A.f[slot] = make_double4_32a(fq[0], fq[1], fq[2], u);
+            A.wvir[slot] = wv;
         }
     }
 }
@@ -1597,7 +1656,8 @@ __global__ void __launch_bounds__(PROPS_THREADS) k_props_reduce(Arrays A, Scal S
 // state exchange in id order
 // ------------------------------------------------------------------------------------------
 template <int MODE>
-__global__ void __launch_bounds__(TILE) k_set_state(Arrays A, Scal S, int cur)
+__global__ void __launch_bounds__(TILE) k_set_state(Arrays A, Scal S, int cur, const double* __restrict__ x,
+                                                    const double* __restrict__ v0)
 {
     for (int t = blockIdx.x; t < S.ntiles; t += gridDim.x) {
         const int r = A.tile_rep[t];
@@ -1617,8 +1677,8 @@ __global__ void __launch_bounds__(TILE) k_set_state(Arrays A, Scal S, int cur)
         A.id[slot] = int32_t(id);
         A.slot_of_id[id] = int32_t(slot);
         for (int a = 0; a < 3; ++a) {
-            A.xl[a][slot] = A.xchg[0][id * 3 + a];     // global position, origin cell (0,0,0)
-            double v = A.xchg[1][id * 3 + a];
+            A.xl[a][slot] = x[id * 3 + a];     // global position, origin cell (0,0,0)
+            double v = v0[id * 3 + a];
             if (!isfinite(v)) {                        // reported by the call; the atom is held still
                 atomicOr(&A.g->err, ERR_NONFINITE);
                 v = 0.0;
@@ -1631,47 +1691,19 @@ __global__ void __launch_bounds__(TILE) k_set_state(Arrays A, Scal S, int cur)
     }
 }
 
+// the state from forces in A.f (half list)
 template <int MODE>
-__global__ void __launch_bounds__(TILE) k_get_state(Arrays A, Scal S, int cur, int want_v, int want_f)
+__global__ void __launch_bounds__(TILE) k_get_state(Arrays A, Scal S, int cur, StateOut O)
 {
     for (int t = blockIdx.x; t < S.ntiles; t += gridDim.x) {
         const int r = A.tile_rep[t];
         const Rep& R = A.rep[r];
         const int64_t slot = int64_t(t) * TILE + threadIdx.x;
         if (slot - R.slot0 >= R.n) continue;
-        const int64_t id = A.id[slot];
-        uint32_t pw;
-        double loc[3];
-        if (MODE == MD_FP64) {
-            const double4_32a p = A.pos64[cur][slot];
-            pw = cell_bits(p.w);
-            loc[0] = A.xl[0][slot]; loc[1] = A.xl[1][slot]; loc[2] = A.xl[2][slot];
-        } else {
-            const float4 p = A.pos32[cur][slot];
-            pw = __float_as_uint(p.w);
-            if (MODE == MD_FP32) { loc[0] = p.x; loc[1] = p.y; loc[2] = p.z; }
-            else { loc[0] = A.xl[0][slot]; loc[1] = A.xl[1][slot]; loc[2] = A.xl[2][slot]; }
-        }
-        int c[3];
-        unpack_cell(pw, c[0], c[1], c[2]);
         const int vhalf = A.rs[r].vhalf;
-        const double4_32a f = (want_f || (want_v && vhalf)) ? A.f[slot] : make_double4_32a(0, 0, 0, 0);
+        const double4_32a f = (O.f || (O.v && vhalf)) ? A.f[slot] : make_double4_32a(0, 0, 0, 0);
         const double fq[3] = {f.x, f.y, f.z};
-        for (int a = 0; a < 3; ++a) {
-            double x = __dadd_rn(__dmul_rn(double(c[a]), R.w[a]), loc[a]);
-            if (x < 0.0) x += R.L[a];
-            if (x >= R.L[a]) x -= R.L[a];
-            A.xchg[0][id * 3 + a] = x;
-            if (want_v) {
-                double v = (MODE == MD_FP32) ? double(A.v32[a][slot]) : A.v[a][slot];
-                if (vhalf) {
-                    if (MODE == MD_FP32) v = double(fmaf(float(S.c), float(fq[a]), float(v)));
-                    else v = fma(S.c, fq[a], v);
-                }
-                A.xchg[1][id * 3 + a] = v;
-            }
-            if (want_f) A.xchg[2][id * 3 + a] = fq[a];
-        }
+        write_state<MODE>(A, S, R, slot, cur, vhalf, fq, O);
     }
 }
 
@@ -1925,24 +1957,41 @@ cudaError_t launch_step(const Arrays& A, const Scal& S, const Launch& L, int cur
     return cudaGetLastError();
 }
 
+// k_forces in the wide shape (16 warps per SM, 8 entries together) for long lists and smaller systems,
+// else with 32 warps and 2 entries (the step kernel's two shapes)
+template <int MODE, bool CELLS, bool OUT>
+static void run_forces(const Arrays& A, const Scal& S, const Launch& L, int cur, const StateOut& O)
+{
+    const int nwt = S.ntiles * (TILE / 32), g = std::max(1, std::min(L.nsm, nwt)), need = (nwt + g - 1) / g;
+    if (L.wide_pairs || CELLS || MODE == MD_FP64) {
+        constexpr int NB = (MODE == MD_FP64) ? 4 : 8;
+        k_forces<MODE, CELLS, OUT, 16, NB><<<g, 32 * std::min(16, need), 0, L.stream>>>(A, S, cur, O);
+    } else if constexpr (!CELLS && MODE != MD_FP64) {
+        k_forces<MODE, false, OUT, 32, 2><<<g, 32 * std::min(32, need), 0, L.stream>>>(A, S, cur, O);
+    }
+}
+
+template <bool OUT>
+static void run_forces_mode(const Arrays& A, const Scal& S, const Launch& L, int cur, const StateOut& O)
+{
+    // with the list-free step kernel there is no current W: the forces come from the cells too
+    const bool cells = L.step_kernel == 4;
+    if (S.mode == MD_FP64) run_forces<MD_FP64, false, OUT>(A, S, L, cur, O);
+    else if (S.mode == MD_MIXED) cells ? run_forces<MD_MIXED, true, OUT>(A, S, L, cur, O) : run_forces<MD_MIXED, false, OUT>(A, S, L, cur, O);
+    else cells ? run_forces<MD_FP32, true, OUT>(A, S, L, cur, O) : run_forces<MD_FP32, false, OUT>(A, S, L, cur, O);
+}
+
 cudaError_t launch_forces(const Arrays& A, const Scal& S, const Launch& L, int cur)
 {
     const int g = tile_grid(S, L);
-    // with the list-free step kernel there is no current W: the forces come from the cells too;
-    // with the half list, from its pairs
-    const bool cells = L.step_kernel == 4;
-    if (S.mode != MD_FP64 && L.step_kernel == 5) {
+    if (S.mode != MD_FP64 && L.step_kernel == 5) {      // the half list's pairs
         k_half_pairs<2><<<g, TILE, 0, L.stream>>>(A, S, cur);
         if (S.chain_len) k_chain_terms<<<g, TILE, 0, L.stream>>>(A, S, cur);
         k_half_to_f<<<g, TILE, 0, L.stream>>>(A, S);
         return cudaGetLastError();
     }
     if (S.chain_len && S.mode != MD_FP64) k_chain_terms<<<g, TILE, 0, L.stream>>>(A, S, cur);
-    if (S.mode == MD_FP64) k_forces<MD_FP64><<<g, TILE, 0, L.stream>>>(A, S, cur);
-    else if (S.mode == MD_MIXED && cells) k_forces<MD_MIXED, true><<<g, TILE, 0, L.stream>>>(A, S, cur);
-    else if (S.mode == MD_MIXED) k_forces<MD_MIXED><<<g, TILE, 0, L.stream>>>(A, S, cur);
-    else if (cells) k_forces<MD_FP32, true><<<g, TILE, 0, L.stream>>>(A, S, cur);
-    else k_forces<MD_FP32><<<g, TILE, 0, L.stream>>>(A, S, cur);
+    run_forces_mode<false>(A, S, L, cur, StateOut{});
     return cudaGetLastError();
 }
 
@@ -1960,22 +2009,37 @@ cudaError_t launch_props(const Arrays& A, const Scal& S, const Launch& L, int cu
     return cudaGetLastError();
 }
 
-cudaError_t launch_get_state(const Arrays& A, const Scal& S, const Launch& L, int cur, bool want_v,
-                             bool want_f)
+cudaError_t launch_get_state(const Arrays& A, const Scal& S, const Launch& L, int cur, const StateOut& O)
 {
     const int g = tile_grid(S, L);
-    if (S.mode == MD_FP64) k_get_state<MD_FP64><<<g, TILE, 0, L.stream>>>(A, S, cur, want_v, want_f);
-    else if (S.mode == MD_MIXED) k_get_state<MD_MIXED><<<g, TILE, 0, L.stream>>>(A, S, cur, want_v, want_f);
-    else k_get_state<MD_FP32><<<g, TILE, 0, L.stream>>>(A, S, cur, want_v, want_f);
+    const bool forces = O.v || O.f;
+    if (S.mode != MD_FP64 && L.step_kernel == 5) {
+        if (forces) {
+            const cudaError_t e = launch_forces(A, S, L, cur);
+            if (e != cudaSuccess) return e;
+        }
+        if (S.mode == MD_MIXED) k_get_state<MD_MIXED><<<g, TILE, 0, L.stream>>>(A, S, cur, O);
+        else k_get_state<MD_FP32><<<g, TILE, 0, L.stream>>>(A, S, cur, O);
+        return cudaGetLastError();
+    }
+    // the chain terms wait in their buffers for a force pass: only where every replica makes one
+    if (S.chain_len && S.mode != MD_FP64 && forces) {
+        const cudaError_t e = launch_forces(A, S, L, cur);
+        if (e != cudaSuccess) return e;
+        if (S.mode == MD_MIXED) k_get_state<MD_MIXED><<<g, TILE, 0, L.stream>>>(A, S, cur, O);
+        else k_get_state<MD_FP32><<<g, TILE, 0, L.stream>>>(A, S, cur, O);
+        return cudaGetLastError();
+    }
+    run_forces_mode<true>(A, S, L, cur, O);
     return cudaGetLastError();
 }
 
-cudaError_t launch_set_state(const Arrays& A, const Scal& S, const Launch& L, int cur)
+cudaError_t launch_set_state(const Arrays& A, const Scal& S, const Launch& L, int cur, const double* x, const double* v)
 {
     const int g = tile_grid(S, L);
-    if (S.mode == MD_FP64) k_set_state<MD_FP64><<<g, TILE, 0, L.stream>>>(A, S, cur);
-    else if (S.mode == MD_MIXED) k_set_state<MD_MIXED><<<g, TILE, 0, L.stream>>>(A, S, cur);
-    else k_set_state<MD_FP32><<<g, TILE, 0, L.stream>>>(A, S, cur);
+    if (S.mode == MD_FP64) k_set_state<MD_FP64><<<g, TILE, 0, L.stream>>>(A, S, cur, x, v);
+    else if (S.mode == MD_MIXED) k_set_state<MD_MIXED><<<g, TILE, 0, L.stream>>>(A, S, cur, x, v);
+    else k_set_state<MD_FP32><<<g, TILE, 0, L.stream>>>(A, S, cur, x, v);
     return cudaGetLastError();
 }
 
