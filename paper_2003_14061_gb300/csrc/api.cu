@@ -877,7 +877,7 @@ int md_integrate(md_system* s, int32_t nsteps)
             GBMD_CUDA(launch_bin_order(s->A, s->S, s->L, s->cur, false));
         }
         {
-            Phase t(s, MD_PHASE_REORDER, REORDER_KERNELS);
+            Phase t(s, MD_PHASE_REORDER, reorder_kernels(s->S));
             GBMD_CUDA(launch_reorder(s->A, s->S, s->L, s->cur));
         }
         {
@@ -904,7 +904,7 @@ int md_get_timing(md_system* s, double* ms, int64_t* calls, int64_t* launches)
         // rebuild sequences inside graphs ran only when their IF node opened: count them here
         long long gr = 0;
         GBMD_CUDA(cudaMemcpy(&gr, &s->A.g->graph_rebuilds, sizeof(gr), cudaMemcpyDeviceToHost));
-        s->launches[MD_PHASE_BUILD] += (bin_kernels(s->S, s->L) + REORDER_KERNELS + build_kernels(s->S, s->L)) *
+        s->launches[MD_PHASE_BUILD] += (bin_kernels(s->S, s->L) + reorder_kernels(s->S) + build_kernels(s->S, s->L)) *
                                        (gr - s->graph_rebuilds_seen);
         s->graph_rebuilds_seen = gr;
     }

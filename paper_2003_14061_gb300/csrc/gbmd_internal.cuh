@@ -458,7 +458,7 @@ cudaError_t launch_bin_order(const Arrays& A, const Scal& S, const Launch& L, in
 cudaError_t launch_reorder(const Arrays& A, const Scal& S, const Launch& L, int cur);
 cudaError_t launch_build_only(const Arrays& A, const Scal& S, const Launch& L, int cur);
 int bin_kernels(const Scal& S, const Launch& L);     // kernels of launch_bin_order
-constexpr int REORDER_KERNELS = 1;                   // kernels of launch_reorder
+int reorder_kernels(const Scal& S);                  // kernels of launch_reorder
 int build_kernels(const Scal& S, const Launch& L);   // kernels of launch_build_only
 // rows of k_build_group's lists, its CTA size, shared memory and grid, into L
 void build_group_shape(const Scal& S, Launch& L, double mean_nbrs, int smem_per_cta);

@@ -102,6 +102,11 @@ __global__ void __launch_bounds__(1024) k_rebuild_list(Arrays A, Scal S)
     if (blockIdx.x == 0 && threadIdx.x == 0) A.g->n_rb_tiles = carry;
 }
 
+// The it-th tile of the rebuild and its replica.  A single system's list is all its tiles: no need to
+// wait for two loads, one after the other, before the replica's geometry.
+__device__ __forceinline__ int rebuild_tile(const Arrays& A, const Scal& S, int it) { return S.nrep == 1 ? it : A.rb_tiles[it]; }
+__device__ __forceinline__ int tile_replica(const Arrays& A, const Scal& S, int t) { return S.nrep == 1 ? 0 : A.tile_rep[t]; }
+
 // ------------------------------------------------------------------------------------------
 // N1 + N2
 // ------------------------------------------------------------------------------------------
@@ -114,8 +119,8 @@ __global__ void __launch_bounds__(TILE) k_bin(Arrays A, Scal S, int cur, int fro
     const int t_begin = blockIdx.x * per, t_end = min(nrb, t_begin + per);
     int run_r = -1, run_occ = 0;
     for (int it = t_begin; it < t_end; ++it) {
-        const int t = A.rb_tiles[it];
-        const int r = A.tile_rep[t];
+        const int t = rebuild_tile(A, S, it);
+        const int r = tile_replica(A, S, t);
         if (r != run_r) {
             if (run_r >= 0) flush_stats(nullptr, &A.rs[run_r].max_occ, 0, run_occ);
             run_r = r;
@@ -398,8 +403,8 @@ __global__ void __launch_bounds__(TILE) k_scatter(Arrays A, Scal S, int keep)
     const int nrb = A.g->n_rb_tiles;
     const int32_t* __restrict__ cs = A.cstart;
     for (int it = blockIdx.x; it < nrb; it += gridDim.x) {
-        const int t = A.rb_tiles[it];
-        const int r = A.tile_rep[t];
+        const int t = rebuild_tile(A, S, it);
+        const int r = tile_replica(A, S, t);
         const Rep& R = A.rep[r];
         const int64_t slot = int64_t(t) * TILE + threadIdx.x;
         if (slot - R.slot0 < R.n) A.tmp_i[0][cs[A.cell[slot]] + A.layer[slot]] = int32_t(slot);
@@ -428,15 +433,15 @@ __global__ void __launch_bounds__(TILE) k_scatter(Arrays A, Scal S, int keep)
 // place was a serial chain of dependent loads (cells of 18 atoms: 428 us for 16.4M atoms, 22 us
 // for 4000); the rank takes one pass over the cell's slots, which the lanes of a cell share.
 template <int MODE>
-__global__ void __launch_bounds__(TILE) k_order(Arrays A, Scal S, int cur)
+__global__ void __launch_bounds__(TILE) k_order(Arrays A, Scal S, int cur, int move)
 {
     if (!A.g->any_rebuild) return;
     const int nrb = A.g->n_rb_tiles;
     const int32_t* __restrict__ unsorted = A.tmp_i[0];
     const int32_t* __restrict__ cs = A.cstart;
     for (int it = blockIdx.x; it < nrb; it += gridDim.x) {
-        const int t = A.rb_tiles[it];
-        const int r = A.tile_rep[t];
+        const int t = rebuild_tile(A, S, it);
+        const int r = tile_replica(A, S, t);
         const Rep& R = A.rep[r];
         const int64_t slot = int64_t(t) * TILE + threadIdx.x;
         if (slot - R.slot0 >= R.n) continue;
@@ -469,7 +474,7 @@ __global__ void __launch_bounds__(TILE) k_order(Arrays A, Scal S, int cur)
         const int P = cand_place(R, prow, rs) + (k - rs);
         const bool reorder = A.rs[r].reorder != 0;
         const int64_t out_slot = reorder ? R.slot0 + (k - cs[R.cell0]) : slot;
-        if (reorder) {                                // the atom's state to its new place in the scratch
+        if (move && reorder) {                        // the atom's state to its new place in the scratch
             if (MODE == MD_FP64) A.tmp_p64[out_slot] = A.pos64[cur][slot];
             else A.tmp_p32[out_slot] = A.pos32[cur][slot];
 #pragma unroll
@@ -493,16 +498,48 @@ __global__ void __launch_bounds__(TILE) k_order(Arrays A, Scal S, int cur)
 
 // ------------------------------------------------------------------------------------------
 // reorder (Sec. 4.1 item 1): new slot slot0 + j takes the j-th atom in cell order, from the scratch
-// that k_order has filled
+// that k_order or k_reorder_gather has filled
 // ------------------------------------------------------------------------------------------
+// Larger systems gather the scratch in a launch of its own: k_order's scattered writes take longer there
+// (4M atoms: 253 us against 52 + 110), and the launch they save is nothing.
+template <int MODE>
+__global__ void __launch_bounds__(TILE) k_reorder_gather(Arrays A, Scal S, int cur)
+{
+    if (!A.g->any_reorder) return;
+    const int nrb = A.g->n_rb_tiles;
+    for (int it = blockIdx.x; it < nrb; it += gridDim.x) {
+        const int t = rebuild_tile(A, S, it);
+        const int r = tile_replica(A, S, t);
+        if (!A.rs[r].reorder) continue;
+        const Rep& R = A.rep[r];
+        const int64_t slot = int64_t(t) * TILE + threadIdx.x;
+        const int64_t j = slot - R.slot0;
+        if (j >= R.n) continue;
+        const int32_t src = A.perm[A.cstart[R.cell0] + j];
+        if (MODE == MD_FP64) A.tmp_p64[slot] = A.pos64[cur][src];
+        else A.tmp_p32[slot] = A.pos32[cur][src];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            if (MODE == MD_FP32) {
+                A.tmp_v[a][slot] = double(A.v32[a][src]);
+            } else {
+                A.tmp_d[a][slot] = A.xl[a][src];
+                A.tmp_v[a][slot] = A.v[a][src];
+            }
+        }
+        A.tmp_i[1][slot] = A.cell[src];
+        A.tmp_id[slot] = A.id[src];
+    }
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(TILE) k_reorder_copy(Arrays A, Scal S, int cur)
 {
     if (!A.g->any_reorder) return;
     const int nrb = A.g->n_rb_tiles;
     for (int it = blockIdx.x; it < nrb; it += gridDim.x) {
-        const int t = A.rb_tiles[it];
-        const int r = A.tile_rep[t];
+        const int t = rebuild_tile(A, S, it);
+        const int r = tile_replica(A, S, t);
         if (!A.rs[r].reorder) continue;
         const Rep& R = A.rep[r];
         const int64_t slot = int64_t(t) * TILE + threadIdx.x;
@@ -767,8 +804,8 @@ __global__ void __launch_bounds__(32 * WARPS, 1) k_build_group(Arrays A, Scal S,
     };
     for (int uid = u_begin + wl; uid < u_end; uid += wpc) {
         const int it = uid / BG_UNITS, u = uid - it * BG_UNITS;
-        const int t = A.rb_tiles[it];
-        const int r = A.tile_rep[t];
+        const int t = rebuild_tile(A, S, it);
+        const int r = tile_replica(A, S, t);
         const Rep& R = A.rep[r];
         const int j0 = (t - R.tile0) * TILE + u * BG_ATOMS;
         const int na = min(min(BG_ATOMS, TILE - u * BG_ATOMS), R.n - j0);
@@ -937,8 +974,8 @@ __global__ void __launch_bounds__(TILE) k_tile_windows(Arrays A, Scal S, int cur
     if (!enabled || !A.g->any_rebuild || !A.tile_win) return;
     const int nrb = A.g->n_rb_tiles;
     for (int it = blockIdx.x; it < nrb; it += gridDim.x) {
-        const int t = A.rb_tiles[it];
-        const Rep& R = A.rep[A.tile_rep[t]];
+        const int t = rebuild_tile(A, S, it);
+        const Rep& R = A.rep[tile_replica(A, S, t)];
         if (threadIdx.x < 9) {
             sh_lo[threadIdx.x] = INT32_MAX;
             sh_hi[threadIdx.x] = -1;
@@ -1063,8 +1100,11 @@ void prime_rebuild_grids(const Scal& S, const Launch& L)
     (void)resident_grid<k_order<MD_MIXED>>(S, L);
     (void)resident_grid<k_order<MD_FP32>>(S, L);
     (void)resident_grid<k_reorder_copy<MD_FP64>>(S, L);
+    (void)resident_grid<k_reorder_gather<MD_FP64>>(S, L);
     (void)resident_grid<k_reorder_copy<MD_MIXED>>(S, L);
+    (void)resident_grid<k_reorder_gather<MD_MIXED>>(S, L);
     (void)resident_grid<k_reorder_copy<MD_FP32>>(S, L);
+    (void)resident_grid<k_reorder_gather<MD_FP32>>(S, L);
 }
 
 cudaError_t launch_all_tiles(const Arrays& A, const Scal& S, const Launch& L)
@@ -1079,24 +1119,32 @@ cudaError_t launch_force_rebuild(const Arrays& A, const Scal& S, const Launch& L
     return cudaGetLastError();
 }
 
+static bool moves_in_order(const Scal& S) { return S.ntiles <= 2048; }
+
 cudaError_t launch_bin_order(const Arrays& A, const Scal& S, const Launch& L, int cur, bool from_set)
 {
     // a single system's list is all its tiles, written at creation
     if (S.nrep > 1) k_rebuild_list<<<std::min((S.nrep + 31) / 32, L.nsm), 1024, 0, L.stream>>>(A, S);
-    const int fs = from_set ? 1 : 0;
+    const int fs = from_set ? 1 : 0, move = moves_in_order(S) ? 1 : 0;
     if (S.mode == MD_FP64) k_bin<MD_FP64><<<resident_grid<k_bin<MD_FP64>>(S, L), TILE, 0, L.stream>>>(A, S, cur, fs);
     else if (S.mode == MD_MIXED) k_bin<MD_MIXED><<<resident_grid<k_bin<MD_MIXED>>(S, L), TILE, 0, L.stream>>>(A, S, cur, fs);
     else k_bin<MD_FP32><<<resident_grid<k_bin<MD_FP32>>(S, L), TILE, 0, L.stream>>>(A, S, cur, fs);
     launch_scan(A, S, L.stream);
     k_scatter<<<resident_grid<k_scatter>(S, L), TILE, 0, L.stream>>>(A, S, L.step_kernel == 4 ? 1 : 0);
-    if (S.mode == MD_FP64) k_order<MD_FP64><<<resident_grid<k_order<MD_FP64>>(S, L), TILE, 0, L.stream>>>(A, S, cur);
-    else if (S.mode == MD_MIXED) k_order<MD_MIXED><<<resident_grid<k_order<MD_MIXED>>(S, L), TILE, 0, L.stream>>>(A, S, cur);
-    else k_order<MD_FP32><<<resident_grid<k_order<MD_FP32>>(S, L), TILE, 0, L.stream>>>(A, S, cur);
+    if (S.mode == MD_FP64) k_order<MD_FP64><<<resident_grid<k_order<MD_FP64>>(S, L), TILE, 0, L.stream>>>(A, S, cur, move);
+    else if (S.mode == MD_MIXED) k_order<MD_MIXED><<<resident_grid<k_order<MD_MIXED>>(S, L), TILE, 0, L.stream>>>(A, S, cur, move);
+    else k_order<MD_FP32><<<resident_grid<k_order<MD_FP32>>(S, L), TILE, 0, L.stream>>>(A, S, cur, move);
     return cudaGetLastError();
 }
 
 cudaError_t launch_reorder(const Arrays& A, const Scal& S, const Launch& L, int cur)
 {
+#define GBMD_GATHER(M) k_reorder_gather<M><<<resident_grid<k_reorder_gather<M>>(S, L), TILE, 0, L.stream>>>(A, S, cur)
+    if (moves_in_order(S)) {
+    } else if (S.mode == MD_FP64) GBMD_GATHER(MD_FP64);
+    else if (S.mode == MD_MIXED) GBMD_GATHER(MD_MIXED);
+    else GBMD_GATHER(MD_FP32);
+#undef GBMD_GATHER
 #define GBMD_REORDER(M) k_reorder_copy<M><<<resident_grid<k_reorder_copy<M>>(S, L), TILE, 0, L.stream>>>(A, S, cur)
     if (S.mode == MD_FP64) GBMD_REORDER(MD_FP64);
     else if (S.mode == MD_MIXED) GBMD_REORDER(MD_MIXED);
@@ -1115,6 +1163,8 @@ cudaError_t launch_bin_only(const Arrays& A, const Scal& S, const Launch& L, int
 // the list-free step kernel reads no neighbour matrix; it is built only where the exact
 // displacement rule needs the positions at the rebuild (written by the build)
 static bool skip_w(const Scal& S, const Launch& L) { return L.step_kernel == 4 && S.rule != MD_REBUILD_DISP; }
+
+int reorder_kernels(const Scal& S) { return moves_in_order(S) ? 1 : 2; }
 
 int bin_kernels(const Scal& S, const Launch&) { return (S.nrep > 1 ? 1 : 0) + (solo_scan(S) ? 4 : 6); }
 
