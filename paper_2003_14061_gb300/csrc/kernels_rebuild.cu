@@ -144,18 +144,25 @@ __global__ void __launch_bounds__(TILE) k_bin(Arrays A, Scal S, int cur, int fro
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 double xa = x[a];
-                if (!isfinite(xa)) {                  // reported; the atom goes to cell 0
-                    atomicOr(&A.g->err, ERR_NONFINITE);
-                    xa = 0.0;
-                }
-                if (xa < 0.0) xa = __dadd_rn(xa, R.L[a]);
-                if (xa >= R.L[a]) xa = __dsub_rn(xa, R.L[a]);
-                if (!(xa >= 0.0 && xa < R.L[a])) {    // more than one period away: whole periods
-                    xa = __dsub_rn(xa, __dmul_rn(R.L[a], floor(xa / R.L[a])));
+                // inside [0, L) on the bit patterns (for x >= 0 they order as the values do): the FP64
+                // pipe, which bounds this pass, is left the arithmetic
+                if (static_cast<unsigned long long>(__double_as_longlong(xa)) >=
+                    static_cast<unsigned long long>(__double_as_longlong(R.L[a]))) {
+                    if (!isfinite(xa)) {              // reported; the atom goes to cell 0
+                        atomicOr(&A.g->err, ERR_NONFINITE);
+                        xa = 0.0;
+                    }
                     if (xa < 0.0) xa = __dadd_rn(xa, R.L[a]);
                     if (xa >= R.L[a]) xa = __dsub_rn(xa, R.L[a]);
+                    if (!(xa >= 0.0 && xa < R.L[a])) {    // more than one period away: whole periods
+                        xa = __dsub_rn(xa, __dmul_rn(R.L[a], floor(xa / R.L[a])));
+                        if (xa < 0.0) xa = __dadd_rn(xa, R.L[a]);
+                        if (xa >= R.L[a]) xa = __dsub_rn(xa, R.L[a]);
+                    }
                 }
-                int ca = int(floor(__dmul_rn(xa, R.s[a])));
+                // xa >= 0, so rounding towards zero is the floor (xa in a hair's breadth of 0 or L after
+                // the wraps is clamped)
+                int ca = __double2int_rz(__dmul_rn(xa, R.s[a]));
                 ca = min(max(ca, 0), R.nc[a] - 1);
                 c[a] = ca;
                 loc[a] = __dsub_rn(xa, __dmul_rn(double(ca), R.w[a]));
