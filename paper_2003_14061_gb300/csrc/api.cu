@@ -234,7 +234,7 @@ size_t carve(const Plan& P, char* base, Arrays* A)
     a.props = c.take<md_props>(size_t(P.nrep));
     a.series = c.take<double>(size_t(P.nrep) * P.series_cap * SERIES_COLS);
     a.g = c.take<Global>(1);
-    a.sm_claim = c.take<int32_t>(size_t(SM_RANGES) + 1);
+    a.sm_claim = c.take<int32_t>(size_t(SM_RANGES + 1) * SM_CLAIM_STRIDE);
     for (int q = 0; q < 3; ++q) a.xchg[q] = c.take<double>(size_t(P.n_total) * 3);
     if (A) *A = a;
     return (c.off + 255) & ~size_t(255);

@@ -28,6 +28,10 @@ namespace gbmd {
 constexpr int TILE = 128;                 // slots per tile
 constexpr int NPROP = 8;                  // U, K, W, px, py, pz, (spare), vmax^2
 constexpr int SM_RANGES = 256;            // slot ranges of the step kernel's per-SM schedule
+// Their counters lie a 128-byte line apart: on the 5 lines that 152 of them fill side by side the claims
+// of all SMs queued in L2, by 8-16 % of a step and differently for every placement of the workspace
+// (1M WCA atoms 66-73 us a step, with a line each 61; 4M 199-207, 196; a sector each 65 and 199)
+constexpr int SM_CLAIM_STRIDE = 32;
 constexpr int SERIES_COLS = 9;            // step, U, K, W, P, px, py, pz, vmax
 constexpr int IDX_SHIFT = 6;              // W entry: slot << 6 | (o_z+1) << 4 | (o_y+1) << 2 | (o_x+1)
 constexpr int64_t MAX_SLOTS = int64_t(1) << 26;
@@ -154,7 +158,7 @@ struct Arrays {
     md_props* props;          // per replica, output of the props reduction
     double* series;           // [nrep][series_cap][SERIES_COLS]
     Global* g;
-    int32_t* sm_claim;        // [SM_RANGES] warp-tiles claimed per range in this step, then warps done
+    int32_t* sm_claim;        // [SM_RANGES][SM_CLAIM_STRIDE] warp-tiles claimed per range in this step, then warps done
     // id-ordered exchange buffers (3 doubles per atom)
     double* xchg[3];
 };

@@ -1098,13 +1098,13 @@ __global__ void __launch_bounds__(TILE, MINB) k_step_sm(Arrays A, Scal S, int cu
             for (int i = 0; i * 32 < nr && sel < 0; ++i) {
                 const int q = i * 32 + lane;
                 const int rr = (home + 1 + q) % nr;
-                const bool avail = q < nr && ld_relaxed_gpu(claimc + rr) < range_len(rr);
+                const bool avail = q < nr && ld_relaxed_gpu(claimc + rr * SM_CLAIM_STRIDE) < range_len(rr);
                 const unsigned b = __ballot_sync(0xffffffffu, avail);
                 if (b) sel = (home + 1 + i * 32 + __ffs(b) - 1) % nr;
             }
             if (sel < 0) return -1;
             int k = 0;
-            if (lane == 0) k = atomicAdd(claimc + sel, 1);
+            if (lane == 0) k = atomicAdd(claimc + sel * SM_CLAIM_STRIDE, 1);
             k = __shfl_sync(0xffffffffu, k, 0);
             if (k < range_len(sel)) return sel * per + k;
         }
@@ -1114,7 +1114,7 @@ __global__ void __launch_bounds__(TILE, MINB) k_step_sm(Arrays A, Scal S, int cu
     auto claim_now = [&]() -> int {
         if (home_open) {
             int k = 0;
-            if (lane == 0) k = atomicAdd(claimc + home, 1);
+            if (lane == 0) k = atomicAdd(claimc + home * SM_CLAIM_STRIDE, 1);
             k = __shfl_sync(0xffffffffu, k, 0);
             if (k < range_len(home)) return home * per + k;
             home_open = false;
@@ -1142,7 +1142,7 @@ __global__ void __launch_bounds__(TILE, MINB) k_step_sm(Arrays A, Scal S, int cu
     while (w0 >= 0) {
         int pend = 0;
         const bool pending = home_open && w1 >= 0;
-        if (pending && lane == 0) pend = atomicAdd(claimc + home, 1);
+        if (pending && lane == 0) pend = atomicAdd(claimc + home * SM_CLAIM_STRIDE, 1);
         int c1 = 0;
         if (w1 >= 0) {
             // one prefetch per 128-byte line: 4 lines of positions (8 in FP64), 2 of each FP64 stream
@@ -1294,11 +1294,15 @@ __global__ void __launch_bounds__(TILE, MINB) k_step_sm(Arrays A, Scal S, int cu
     }
     if (run_r >= 0) flush_replica_warp(A, S, run_r, run_max, run_cnt, cond, use_cond, pacc, pvm);
     // the last warp of the launch resets the counters; the next launch is ordered after this one
-    if (!single && lane == 0) {
-        __threadfence();
-        if (atomicAdd(claimc + SM_RANGES, 1) == nwarps - 1) {
-            for (int q = 0; q < nr; ++q) claimc[q] = 0;
-            claimc[SM_RANGES] = 0;
+    if (!single) {
+        int done = 0;
+        if (lane == 0) {
+            __threadfence();
+            done = atomicAdd(claimc + SM_RANGES * SM_CLAIM_STRIDE, 1) == nwarps - 1;
+        }
+        if (__shfl_sync(0xffffffffu, done, 0)) {
+            for (int q = lane; q < nr; q += 32) claimc[q * SM_CLAIM_STRIDE] = 0;
+            if (lane == 0) claimc[SM_RANGES * SM_CLAIM_STRIDE] = 0;
             __threadfence();
         }
     }
