@@ -1292,6 +1292,34 @@ __global__ void __launch_bounds__(TILE, MINB) k_step_sm(Arrays A, Scal S, int cu
         w1 = w2;
         c0 = c1;                                 // read one warp-tile ahead
     }
+    if (S.nrep == 1 && wpc > 1) {
+        // one replica: the CTA's warps are merged first, so that a quarter of the atomics meets on the
+        // replica's words at the end of the launch (integer sums and maxima, the same bits)
+        __shared__ float s_max[TILE / 32];
+        __shared__ int s_cnt[TILE / 32];
+        const float m = warp_max(run_max);
+        if (lane == 0) {
+            s_max[threadIdx.x >> 5] = m;
+            s_cnt[threadIdx.x >> 5] = run_cnt;
+        }
+        __syncthreads();
+        if (threadIdx.x >= 32) run_r = -1;
+        else {
+            run_cnt = 0;
+            for (int q = 0; q < wpc; ++q) {
+                run_max = fmaxf(run_max, s_max[q]);
+                run_cnt += s_cnt[q];
+            }
+            if (FIX) {
+                if (lane < 8)
+                    for (int q = 1; q < wpc; ++q) s_pacc[0][lane] += s_pacc[q][lane];
+                if (lane == 0)
+                    for (int q = 1; q < wpc; ++q) s_pvm[0] = fmaxf(s_pvm[0], s_pvm[q]);
+                __syncwarp();
+            }
+            run_r = run_cnt > 0 ? 0 : -1;
+        }
+    }
     if (run_r >= 0) flush_replica_warp(A, S, run_r, run_max, run_cnt, cond, use_cond, pacc, pvm);
     // the last warp of the launch resets the counters; the next launch is ordered after this one
     if (!single) {
