@@ -79,7 +79,9 @@ __device__ __forceinline__ void add_buffer(const Arrays& A, int64_t slot, AccF& 
 }
 
 // One thread per atom over its column of W, NB entries at a time; wr(m) returns the m-th entry
-// and pr(e) the FP32 cell-local position of the neighbour an entry names.
+// and pr(e) the FP32 cell-local position of the neighbour an entry names.  What pads a column past mm
+// takes the atom's own position: it is masked by a factor of zero, which does not keep out a
+// position that is not finite, as any other atom's, of another replica even, may be.
 // The entries of batch b+1 are read together with the position gathers of batch b, so each
 // thread keeps 2 NB loads in flight and a batch waits for one memory latency, not two.  The
 // arithmetic runs on packed FP32x2 operations (one instruction for two lanes, each lane rounded as
@@ -87,7 +89,7 @@ __device__ __forceinline__ void add_buffer(const Arrays& A, int64_t slot, AccF& 
 // lanes' sums are added at the end, so the summation order is the same for every NB and every
 // source of the entries.
 template <int NB, class WRead, class PRead>
-__device__ __forceinline__ AccF pair_loop_f32(const Scal& S, const Rep& R, float4 pi, int mm, WRead wr, PRead pr)
+__device__ __forceinline__ AccF pair_loop_f32(const Scal& S, const Rep& R, float4 pi, int64_t slot, int mm, WRead wr, PRead pr)
 {
     static_assert(NB % 2 == 0, "W entries are processed in pairs");
     const float2 wx = make_float2(R.wf[0], R.wf[0]);
@@ -99,19 +101,21 @@ __device__ __forceinline__ AccF pair_loop_f32(const Scal& S, const Rep& R, float
     const float2 npx = make_float2(-pi.x, -pi.x), npy = make_float2(-pi.y, -pi.y), npz = make_float2(-pi.z, -pi.z);
     const float2 sig2 = make_float2(S.sig2f, S.sig2f), eps48 = make_float2(S.eps48f, S.eps48f);
     float2 fx = make_float2(0.f, 0.f), fy = fx, fz = fx, u = fx, w = fx;
+    // past mm: the atom's own slot, o = 0; two entries per batch select pi below (a word less to keep:
+    // at the bound of 64 registers 4M WCA atoms with props take 223 us a step, with it 247)
+    const uint32_t self = (NB >= 4) ? (uint32_t(slot) << IDX_SHIFT) | 0x15u : 0u;
     uint32_t e[NB];
 #pragma unroll
-    for (int k = 0; k < NB; ++k) e[k] = (k < mm) ? wr(k) : 0u;
+    for (int k = 0; k < NB; ++k) e[k] = (k < mm) ? wr(k) : self;
     for (int m0 = 0; m0 < mm; m0 += NB) {
         float4 pj[NB];
 #pragma unroll
-        // entries past mm are 0 (slot 0, a valid address) and masked below; with 4 or 8 entries
-        // per batch the unconditional gathers measured faster (LJ, 8 per batch: 2.61 against
-        // 2.73 ms), with 2 slower (0.227 against 0.206 ms), so the select stays there
+        // with 4 or 8 entries per batch the unconditional gathers measured faster (LJ, 8 per batch:
+        // 2.61 against 2.73 ms), with 2 slower (0.227 against 0.206 ms), so the select stays there
         for (int k = 0; k < NB; ++k) pj[k] = (NB >= 4 || m0 + k < mm) ? pr(e[k]) : pi;
         uint32_t en[NB];
 #pragma unroll
-        for (int k = 0; k < NB; ++k) en[k] = (m0 + NB + k < mm) ? wr(m0 + NB + k) : 0u;
+        for (int k = 0; k < NB; ++k) en[k] = (m0 + NB + k < mm) ? wr(m0 + NB + k) : self;
 #pragma unroll
         for (int k = 0; k < NB; k += 2) {
             const uint32_t e0 = e[k], e1 = e[k + 1];
@@ -154,7 +158,7 @@ __device__ __forceinline__ AccF force_f32_rows(const Arrays& A, const Scal& S, c
 {
     const uint32_t* __restrict__ Wc = A.W + slot;
     const int64_t ns = S.nslots;
-    return pair_loop_f32<NB>(S, R, pi, mm, [=](int m) { return __ldcs(Wc + int64_t(m) * ns); },
+    return pair_loop_f32<NB>(S, R, pi, slot, mm, [=](int m) { return __ldcs(Wc + int64_t(m) * ns); },
                              [=](uint32_t e) { return __ldg(pos + (e >> IDX_SHIFT)); });
 }
 
@@ -538,7 +542,8 @@ __device__ __forceinline__ void prefetch_l2(const void* p)
 }
 
 // FP64 pairs, NB entries at a time: their W rows, positions and pair terms are independent of each
-// other, the sums are added entry by entry in the column's order
+// other, the sums are added entry by entry in the column's order.  What is out of range, or pads the
+// column (slot 0), is left out of the sums, not added as zero: its position need not be finite.
 template <int NB>
 __device__ __forceinline__ AccD force_f64(const Arrays& A, const Scal& S, const Rep& R,
                                           const double4_32a* __restrict__ pos, int64_t slot, double4_32a pi)
@@ -563,12 +568,15 @@ __device__ __forceinline__ AccD force_f64(const Arrays& A, const Scal& S, const 
             const double ri2 = 1.0 / r2;
             const double sr2 = S.sig2d * ri2;
             const double sr6 = sr2 * sr2 * sr2;
-            const double fs = in ? S.eps48d * sr6 * (sr6 - 0.5) * ri2 : 0.0;
-            a.fx -= fs * dx;
-            a.fy -= fs * dy;
-            a.fz -= fs * dz;
-            a.u += in ? S.eps4d * sr6 * (sr6 - 1.0) - S.ucd : 0.0;
-            a.w += fs * r2;
+            const double fs = S.eps48d * sr6 * (sr6 - 0.5) * ri2;
+            const double ut = S.eps4d * sr6 * (sr6 - 1.0) - S.ucd;
+            if (in) {
+                a.fx -= fs * dx;
+                a.fy -= fs * dy;
+                a.fz -= fs * dz;
+                a.u += ut;
+                a.w += fs * r2;
+            }
         }
     }
     return a;
@@ -966,7 +974,7 @@ __global__ void __launch_bounds__(TILE, MINB) k_step(Arrays A, Scal S, int cur, 
                     const uint32_t* __restrict__ Wc = A.W + slot;
                     const int64_t ns = S.nslots;
                     a = pair_loop_f32<NB>(
-                        S, R, pi, mm, [=](int m) { return __ldcs(Wc + int64_t(m) * ns); },
+                        S, R, pi, slot, mm, [=](int m) { return __ldcs(Wc + int64_t(m) * ns); },
                         [=](uint32_t e) {
                             const int j = int(e >> IDX_SHIFT);
                             const int4 w = sh_win[(e >> 2) & 15u];
@@ -1451,7 +1459,7 @@ __global__ void __launch_bounds__(TILE, 2) k_step_bulk(Arrays A, Scal S, int cur
             const uint32_t* __restrict__ gw = A.W + slot;
             const int64_t ns = S.nslots;
             AccF a = pair_loop_f32<NB>(
-                S, R, pi, mm, [=](int m) { return (m < rows) ? sw[m * TILE] : __ldcs(gw + int64_t(m) * ns); },
+                S, R, pi, slot, mm, [=](int m) { return (m < rows) ? sw[m * TILE] : __ldcs(gw + int64_t(m) * ns); },
                 [=](uint32_t e) { return __ldg(pos + (e >> IDX_SHIFT)); });
             if (S.chain_len) add_buffer(A, slot, a);
             double v[3], x[3];
