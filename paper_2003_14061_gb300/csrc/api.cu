@@ -460,7 +460,7 @@ int apply_tuning(md_system* s)
     s->S.half_list = (s->L.step_kernel == 5) ? 1 : 0;      // W keeps each pair once
     bulk_shape(s->S, per_sm, s->smem_per_sm, s->smem_per_cta, &s->L.bulk_rows, &s->L.bulk_smem);
     stage_shape(per_sm, s->smem_per_sm, &s->L.stage_cap, &s->L.stage_smem);
-    build_group_shape(s->S, s->L, s->plan.mean_nbrs, s->smem_per_cta);
+    GBMD_CUDA(build_group_shape(s->S, s->L, s->plan.mean_nbrs, s->smem_per_cta));
     // Step-kernel shape.  One that md_set_tuning never named is chosen by size: 4 CTAs per SM with 8
     // W entries together (120 registers) up to 600k atoms and at 30 neighbours or more, else 8 CTAs
     // and 2 entries, whose warps hide the HBM latency that the larger fluids wait for.  Step kernel,
@@ -764,9 +764,10 @@ int md_create_batch(const md_params* p, int32_t nrep, const int64_t* n_rep, cons
     s->tune.step_kernel = 1;
     s->tune.reorder_every = s->p.reorder_every == 0 ? -1 : s->p.reorder_every;
     s->tune.build_stage = 2;            // 2 = off (0 keeps the current value in md_set_tuning)
-    apply_tuning(s);
 
     auto bail = [&](int code) { delete s; return code; };
+    rc = apply_tuning(s);
+    if (rc) return bail(rc);
     if (cudaMemsetAsync(d_workspace, 0, need, s->L.stream) != cudaSuccess) return bail(fail(MD_ERR_CUDA, "memset"));
     if (cudaMemcpyAsync(s->A.rep, s->plan.reps.data(), sizeof(Rep) * s->plan.nrep, cudaMemcpyHostToDevice,
                         s->L.stream) != cudaSuccess ||

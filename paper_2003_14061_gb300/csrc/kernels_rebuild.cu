@@ -1185,20 +1185,16 @@ int build_kernels(const Scal& S, const Launch& L)
 // 60 % of the capacity for denser regions than the mean.  A longer list sends its unit through
 // build_column.  One CTA per SM with as many warps as their lists allow,
 // up to 32; with room for fewer than 24 the kernel compiled for 20, which has more registers.
+// The opt-in limit is raised at each call: it belongs to the kernel in the context that is current, so
+// one raised for a system on another device says nothing about this one.
 template <int MODE, bool HALF, int WARPS>
-static void group_limit()
+static cudaError_t group_limit(int smem_per_cta)
 {
-    // the opt-in limit, once per kernel
-    static const bool raised = [] {
-        int optin = 0, dev = 0;
-        cudaFuncAttributes fa;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        return cudaFuncGetAttributes(&fa, k_build_group<MODE, HALF, WARPS>) == cudaSuccess &&
-               cudaFuncSetAttribute(k_build_group<MODE, HALF, WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    optin - int(fa.sharedSizeBytes)) == cudaSuccess;
-    }();
-    (void)raised;
+    cudaFuncAttributes fa;
+    const cudaError_t e = cudaFuncGetAttributes(&fa, k_build_group<MODE, HALF, WARPS>);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_build_group<MODE, HALF, WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                smem_per_cta - int(fa.sharedSizeBytes));
 }
 
 // F(MODE, HALF, WARPS) for the system's precision, list and list length
@@ -1208,7 +1204,7 @@ static void group_limit()
     else if (S.mode == MD_MIXED) { if (S.half_list) GBMD_BUILD_WARPS(MD_MIXED, true, F) else GBMD_BUILD_WARPS(MD_MIXED, false, F) } \
     else { if (S.half_list) GBMD_BUILD_WARPS(MD_FP32, true, F) else GBMD_BUILD_WARPS(MD_FP32, false, F) }
 
-void build_group_shape(const Scal& S, Launch& L, double mean_nbrs, int smem_per_cta)
+cudaError_t build_group_shape(const Scal& S, Launch& L, double mean_nbrs, int smem_per_cta)
 {
     const int room = smem_per_cta - 2048;
     const double want = std::max(0.69 * 1.35 * mean_nbrs + 12.0, 0.6 * S.cap);
@@ -1219,9 +1215,11 @@ void build_group_shape(const Scal& S, Launch& L, double mean_nbrs, int smem_per_
     L.bg_block = 32 * std::min(L.bg_warps, fit);
     L.bg_rows = rows;
     L.bg_smem = (BG_TABLE + (rows + BG_STEP) * int(BG_ROW)) * (L.bg_block / 32);
-#define GBMD_LIMIT(M, H, B) group_limit<M, H, B>()
+    cudaError_t e = cudaSuccess;
+#define GBMD_LIMIT(M, H, B) e = group_limit<M, H, B>(smem_per_cta)
     GBMD_BUILD_DISPATCH(GBMD_LIMIT)
 #undef GBMD_LIMIT
+    return e;
 }
 
 cudaError_t launch_build_only(const Arrays& A, const Scal& S, const Launch& L, int cur)
