@@ -1244,8 +1244,6 @@ __global__ void __launch_bounds__(TILE, MINB) k_step_sm(Arrays A, Scal S, int cu
             } else if (SRC == 2) {
                 const float4 fb = __ldcs(A.fbuf + slot);
                 a = AccF{fb.x, fb.y, fb.z, fb.w, __ldcs(A.wbuf + slot)};
-                A.fbuf[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
-                A.wbuf[slot] = 0.f;
             } else {
                 a = force_f32_rows<NB>(A, S, R, pos, slot, pi, min(c0, S.cap));
             }
@@ -1272,6 +1270,13 @@ __global__ void __launch_bounds__(TILE, MINB) k_step_sm(Arrays A, Scal S, int cu
                 }
             }
             A.pos32[nxt][slot] = make_float4(pn[0], pn[1], pn[2], pi.w);
+            if (SRC == 2) {
+                // cleared last, when the loads have returned: a store to a line that is still on its
+                // way into L1 holds up every access behind it (2M atoms: this kernel 177 us with
+                // the clears right behind the loads, as the compiler had kept them, 62 with them here)
+                A.fbuf[slot] = make_float4(0.f, 0.f, 0.f, 0.f);
+                A.wbuf[slot] = 0.f;
+            }
             if (S.rule == MD_REBUILD_DISP) {
                 const float4 xr = A.xref[slot];
                 const float d0 = pn[0] - xr.x, d1 = pn[1] - xr.y, d2 = pn[2] - xr.z;
