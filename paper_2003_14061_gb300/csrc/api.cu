@@ -400,6 +400,7 @@ void fill_scal(md_system* s)
     S.series_cap = P.series_cap;
     S.shift = p.shift_energy;
     S.props_split = props_split(P);
+    S.dilute = dilute_cells(P.reps) ? 1 : 0;
     S.dt = p.dt;
     S.mass = p.mass;
     S.c = p.dt / (2.0 * p.mass);

@@ -21,6 +21,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "gbmd.h"
 
 namespace gbmd {
@@ -176,6 +178,7 @@ struct Scal {
     int32_t series_cap;
     int32_t shift;
     int32_t props_split;      // CTAs per replica of the props reduction (1..PROPS_SPLIT_MAX)
+    int32_t dilute;           // some replica has its cells done apart from its tiles (dilute_cells)
     int32_t half_list;        // 1: W keeps each pair once, at the lower slot (step kernel 5)
     int32_t chain_len;        // polymer chains (md_set_chains): atoms per chain, 0 = none
     float ch_kb, ch_r0sq, ch_ka, ch_kd;   // FENE stiffness, R0^2, bend and dihedral constants
@@ -453,6 +456,7 @@ int set_last_error(int code, const char* msg);
 cudaError_t launch_debug_error(const Arrays& A, const Launch& L, int bits, int nbr_seen);
 
 // rebuild path (kernels_rebuild.cu)
+bool dilute_cells(const std::vector<Rep>& reps);
 cudaError_t launch_all_tiles(const Arrays& A, const Scal& S, const Launch& L);           // creation, one system
 cudaError_t launch_force_rebuild(const Arrays& A, const Scal& S, const Launch& L, int reorder);
 void prime_rebuild_grids(const Scal& S, const Launch& L);

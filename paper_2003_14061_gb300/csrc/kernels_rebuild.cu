@@ -404,6 +404,35 @@ static void launch_scan(const Arrays& A, const Scal& S, cudaStream_t st)
 // ------------------------------------------------------------------------------------------
 // N4 and the deterministic order within cells
 // ------------------------------------------------------------------------------------------
+// What a rebuild keeps of cell c of a replica: its run of candidates, its counter cleared for the next
+// binning, and (keep) its slot range for the list-free step kernel.
+__device__ __forceinline__ void cell_done(const Arrays& A, const Rep& R, const int32_t* __restrict__ cs, int c, int k0, int P0,
+                                          int keep)
+{
+    const int ncx = R.nc[0], prow = c / ncx, cx = c - prow * ncx;
+    const int32_t* row = cs + R.cell0 + prow * ncx;
+    const int rs = row[0];
+    const int base = cand_place(R, prow, rs) - P0;
+    A.crun[R.cell0 + c] = make_int2((base + ((row[max(cx - 1, 0)] - rs) & ~3)) >> 2,
+                                    (base + ((row[min(cx + 1, ncx - 1) + 1] - rs + 3) & ~3)) >> 2);
+    A.ccount[R.cell0 + c] = 0;
+    if (keep) A.ckeep[R.cell0 + c] = make_int2(row[cx] - k0, row[cx + 1] - k0);
+}
+
+// A tile does its share of its replica's cells.  In a dilute gas that is far more cells than slots
+// (one tile of 128 atoms in 10^6 cells: 2.63 ms a binning and build); replicas beyond CELLS_PER_TILE have theirs
+// done in chunks by all CTAs instead (S.dilute; 61 us, 20000 atoms in 8 10^6 cells 281 -> 137).
+constexpr int CELLS_PER_TILE = 256, CELL_CHUNK = 4 * TILE;
+
+__host__ __device__ __forceinline__ bool dilute_rep(const Rep& R) { return R.ncells > int64_t(CELLS_PER_TILE) * R.ntiles; }
+
+bool dilute_cells(const std::vector<Rep>& reps)
+{
+    for (const Rep& R : reps)
+        if (dilute_rep(R)) return true;
+    return false;
+}
+
 __global__ void __launch_bounds__(TILE) k_scatter(Arrays A, Scal S, int keep)
 {
     if (!A.g->any_rebuild) return;
@@ -415,20 +444,24 @@ __global__ void __launch_bounds__(TILE) k_scatter(Arrays A, Scal S, int keep)
         const Rep& R = A.rep[r];
         const int64_t slot = int64_t(t) * TILE + threadIdx.x;
         if (slot - R.slot0 < R.n) A.tmp_i[0][cs[A.cell[slot]] + A.layer[slot]] = int32_t(slot);
-        // this tile's share of the replica's cells: their runs of candidates, their counters cleared
-        // (keep: also their slot ranges, for the list-free step kernel)
-        const int tt = t - R.tile0, ncx = R.nc[0];
+        if (S.dilute && dilute_rep(R)) continue;
+        const int tt = t - R.tile0;
         const int c_end = int(int64_t(R.ncells) * (tt + 1) / R.ntiles);
         const int k0 = cs[R.cell0], P0 = cand_place(R, 0, k0);
-        for (int c = int(int64_t(R.ncells) * tt / R.ntiles) + int(threadIdx.x); c < c_end; c += TILE) {
-            const int prow = c / ncx, cx = c - prow * ncx;
-            const int32_t* row = cs + R.cell0 + prow * ncx;
-            const int rs = row[0];
-            const int base = cand_place(R, prow, rs) - P0;
-            A.crun[R.cell0 + c] = make_int2((base + ((row[max(cx - 1, 0)] - rs) & ~3)) >> 2,
-                                            (base + ((row[min(cx + 1, ncx - 1) + 1] - rs + 3) & ~3)) >> 2);
-            A.ccount[R.cell0 + c] = 0;               // ready for the next binning
-            if (keep) A.ckeep[R.cell0 + c] = make_int2(row[cx] - k0, row[cx + 1] - k0);
+        for (int c = int(int64_t(R.ncells) * tt / R.ntiles) + int(threadIdx.x); c < c_end; c += TILE)
+            cell_done(A, R, cs, c, k0, P0, keep);
+    }
+    if (!S.dilute) return;
+    for (int64_t c0 = int64_t(blockIdx.x) * CELL_CHUNK; c0 < S.ncells; c0 += int64_t(gridDim.x) * CELL_CHUNK) {
+        const int64_t c1 = min(c0 + CELL_CHUNK, int64_t(S.ncells));
+        const int r1 = (S.nrep == 1) ? 0 : A.cell_rep[c1 - 1];
+        for (int r = (S.nrep == 1) ? 0 : A.cell_rep[c0]; r <= r1; ++r) {
+            const Rep& R = A.rep[r];
+            if (!A.rs[r].rebuild || !dilute_rep(R)) continue;
+            const int k0 = cs[R.cell0], P0 = cand_place(R, 0, k0);
+            const int end = int(min(c1 - R.cell0, int64_t(R.ncells)));
+            for (int c = int(max(c0 - R.cell0, int64_t(0))) + int(threadIdx.x); c < end; c += TILE)
+                cell_done(A, R, cs, c, k0, P0, keep);
         }
     }
 }
@@ -1079,13 +1112,12 @@ static int tile_grid(const Scal& S, const Launch& L)
     return std::max(1, std::min(L.grid, S.ntiles));
 }
 
-// Grid of a per-tile rebuild kernel that holds nothing across tiles (binning, scatter, reorder,
-// the neighbour build): every CTA the device can keep resident.  Binning, scatter and reorder wait
-// on memory and atomics, so each resident warp adds requests in flight; the build gains warps to
-// issue from (9 CTAs per SM instead of the step kernel's 8: 3 % less build time on the 4M-atom
-// fluid).  The occupancy of each kernel is looked up once.
+// Grid of a rebuild kernel over tiles or other items that holds nothing across them (binning,
+// scatter, order, reorder): every CTA the device can keep resident.  They wait on memory and
+// atomics, so each resident warp adds requests in flight.  The occupancy of each kernel is looked
+// up once.
 template <auto Kernel>
-static int resident_grid(const Scal& S, const Launch& L)
+static int resident_grid(const Scal& S, const Launch& L, int items = 0)
 {
     static const int per_sm = [] {
         int b = 0;
@@ -1093,7 +1125,7 @@ static int resident_grid(const Scal& S, const Launch& L)
         return b;
     }();
     const int g = (per_sm > 0) ? L.nsm * per_sm : L.grid;
-    return std::max(1, std::min(g, S.ntiles));
+    return std::max(1, std::min(g, items > 0 ? items : S.ntiles));
 }
 
 // looks the occupancies up outside any stream capture
@@ -1137,7 +1169,8 @@ cudaError_t launch_bin_order(const Arrays& A, const Scal& S, const Launch& L, in
     else if (S.mode == MD_MIXED) k_bin<MD_MIXED><<<resident_grid<k_bin<MD_MIXED>>(S, L), TILE, 0, L.stream>>>(A, S, cur, fs);
     else k_bin<MD_FP32><<<resident_grid<k_bin<MD_FP32>>(S, L), TILE, 0, L.stream>>>(A, S, cur, fs);
     launch_scan(A, S, L.stream);
-    k_scatter<<<resident_grid<k_scatter>(S, L), TILE, 0, L.stream>>>(A, S, L.step_kernel == 4 ? 1 : 0);
+    const int items = S.dilute ? std::max(S.ntiles, int((int64_t(S.ncells) + CELL_CHUNK - 1) / CELL_CHUNK)) : S.ntiles;
+    k_scatter<<<resident_grid<k_scatter>(S, L, items), TILE, 0, L.stream>>>(A, S, L.step_kernel == 4 ? 1 : 0);
     if (S.mode == MD_FP64) k_order<MD_FP64><<<resident_grid<k_order<MD_FP64>>(S, L), TILE, 0, L.stream>>>(A, S, cur, move);
     else if (S.mode == MD_MIXED) k_order<MD_MIXED><<<resident_grid<k_order<MD_MIXED>>(S, L), TILE, 0, L.stream>>>(A, S, cur, move);
     else k_order<MD_FP32><<<resident_grid<k_order<MD_FP32>>(S, L), TILE, 0, L.stream>>>(A, S, cur, move);

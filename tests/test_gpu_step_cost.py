@@ -1,6 +1,7 @@
 """Costs of a step relative to one another, as ratios of times on the same system: a choice that the
 interface offers must not fall far behind what it is there for.  Each bound lies about midway between
 the ratio that the kernels have and the one of the fault that it guards against."""
+import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -38,3 +39,28 @@ def test_half_list_step_against_the_full_list():
     s.integrate(20)
     half = _step_us(s)
     assert half < 1.9 * full, (half, full)
+
+
+def _rebuild_us(s):
+    best = 1e30
+    for _ in range(5):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        s.build_neighbours()
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b) * 1e3)
+    return best
+
+
+def _gas(n, cells):
+    m = int(np.ceil(n ** (1.0 / 3.0)))
+    side = 1.53 * cells
+    g = np.stack(np.meshgrid(*[np.arange(m)] * 3, indexing="ij"), -1).reshape(-1, 3)[:n]
+    x = (g + np.random.default_rng(4).uniform(0.2, 0.8, (n, 3))) * (side / m)
+    return MDSystem(x, np.zeros_like(x), np.array([side] * 3), skin=0.4, nbr_capacity=40)
+
+
+def test_rebuild_of_few_atoms_in_many_cells():
+    # measured 1.4; 62 while the one tile of the atoms did all 10^6 cells
+    assert _rebuild_us(_gas(128, 100)) < 8.0 * _rebuild_us(_gas(128, 10))
