@@ -41,6 +41,7 @@ struct Plan {
     int32_t series_cap = 0;
     int64_t nrows = 0;            // rows of cells of all replicas
     double mean_nbrs = 0.0;       // neighbours within r_c + skin at the largest mean density
+    double dense_nbrs = 0.0;      // the same in a liquid of density 1.2 sigma^-3, denser than any at its triple point
     int64_t n_total = 0;
     int mode = MD_MIXED;
     int rule = MD_REBUILD_VMAX;
@@ -152,6 +153,7 @@ int make_plan(const md_params* p, int32_t nrep, const int64_t* n_rep, const doub
     P->n_total = ids;
     P->nrows = rows;
     P->mean_nbrs = 4.0 / 3.0 * M_PI * rl * rl * rl * rho_max;
+    P->dense_nbrs = 4.0 / 3.0 * M_PI * std::pow(rl / p->sigma, 3.0) * 1.2;
     P->tile_rep.resize(P->ntiles);
     for (int32_t r = 0; r < nrep; ++r)
         for (int32_t k = 0; k < P->reps[r].ntiles; ++k) P->tile_rep[P->reps[r].tile0 + k] = r;
@@ -461,7 +463,7 @@ int apply_tuning(md_system* s)
     s->S.half_list = (s->L.step_kernel == 5) ? 1 : 0;      // W keeps each pair once
     bulk_shape(s->S, per_sm, s->smem_per_sm, s->smem_per_cta, &s->L.bulk_rows, &s->L.bulk_smem);
     stage_shape(per_sm, s->smem_per_sm, &s->L.stage_cap, &s->L.stage_smem);
-    GBMD_CUDA(build_group_shape(s->S, s->L, s->plan.mean_nbrs, s->smem_per_cta));
+    GBMD_CUDA(build_group_shape(s->S, s->L, s->plan.mean_nbrs, s->plan.dense_nbrs, s->smem_per_cta));
     // Step-kernel shape.  One that md_set_tuning never named is chosen by size: 4 CTAs per SM with 8
     // W entries together (120 registers) up to 600k atoms and at 30 neighbours or more, else 8 CTAs
     // and 2 entries, whose warps hide the HBM latency that the larger fluids wait for.  Step kernel,

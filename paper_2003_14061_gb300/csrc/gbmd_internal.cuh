@@ -469,7 +469,7 @@ int bin_kernels(const Scal& S, const Launch& L);     // kernels of launch_bin_or
 int reorder_kernels(const Scal& S);                  // kernels of launch_reorder
 int build_kernels(const Scal& S, const Launch& L);   // kernels of launch_build_only
 // rows of k_build_group's lists, its CTA size, shared memory and grid, into L
-cudaError_t build_group_shape(const Scal& S, Launch& L, double mean_nbrs, int smem_per_cta);
+cudaError_t build_group_shape(const Scal& S, Launch& L, double mean_nbrs, double dense_nbrs, int smem_per_cta);
 
 // adjoint (kernels_adjoint.cu)
 cudaError_t launch_adj_reverse(const Arrays& A, const Scal& S, const Launch& L, const AdjView& V, int q, double kappa,

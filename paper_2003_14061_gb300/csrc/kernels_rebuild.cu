@@ -1214,10 +1214,13 @@ int build_kernels(const Scal& S, const Launch& L)
 }
 
 // The lists of k_build_group hold one z plane's neighbours of an atom.  A slab of thickness w >= r_l
-// around it holds up to 69 % of them; half as many again and 12 leave room for fluctuations, and
-// 60 % of the capacity for denser regions than the mean.  A longer list sends its unit through
-// build_column.  One CTA per SM with as many warps as their lists allow,
-// up to 32; with room for fewer than 24 the kernel compiled for 20, which has more registers.
+// around it holds up to 69 % of them; a third as many again and 12 leave room for fluctuations, at
+// the largest mean density or, as far as 60 % of the capacity allows, in the densest liquid
+// (mean_nbrs, dense_nbrs), so that a droplet's lists fit.  A capacity beyond that must not cost warps:
+// 256k WCA atoms with room for 1000 neighbours each had 601 rows and 5 warps per SM, 260 us a binning
+// and build against 106 with 29.  A longer list sends its unit through build_column.  One CTA per SM
+// with as many warps as their lists allow, up to 32; with room for fewer than 24 the kernel compiled
+// for 20, which has more registers.
 // The opt-in limit is raised at each call: it belongs to the kernel in the context that is current, so
 // one raised for a system on another device says nothing about this one.
 template <int MODE, bool HALF, int WARPS>
@@ -1237,10 +1240,11 @@ static cudaError_t group_limit(int smem_per_cta)
     else if (S.mode == MD_MIXED) { if (S.half_list) GBMD_BUILD_WARPS(MD_MIXED, true, F) else GBMD_BUILD_WARPS(MD_MIXED, false, F) } \
     else { if (S.half_list) GBMD_BUILD_WARPS(MD_FP32, true, F) else GBMD_BUILD_WARPS(MD_FP32, false, F) }
 
-cudaError_t build_group_shape(const Scal& S, Launch& L, double mean_nbrs, int smem_per_cta)
+cudaError_t build_group_shape(const Scal& S, Launch& L, double mean_nbrs, double dense_nbrs, int smem_per_cta)
 {
     const int room = smem_per_cta - 2048;
-    const double want = std::max(0.69 * 1.35 * mean_nbrs + 12.0, 0.6 * S.cap);
+    auto for_mean = [](double nbrs) { return 0.69 * 1.35 * nbrs + 12.0; };
+    const double want = std::max(for_mean(mean_nbrs), std::min(0.6 * S.cap, for_mean(dense_nbrs)));
     int rows = std::min(S.cap, int(std::min(want, 1.0e6)) + 1);
     rows = std::min(rows, (room - BG_TABLE) / int(BG_ROW) - BG_STEP);
     const int fit = room / (BG_TABLE + (rows + BG_STEP) * int(BG_ROW));
