@@ -240,7 +240,11 @@ typedef struct {
                                 12 or 16 CTAs per SM (the largest not above this) and its grid is
                                 capped at residency.  The rebuild kernels (binning, scatter,
                                 reorder, neighbour build) always run at their full residency */
-    int32_t nbr_batch;       /* W entries each thread loads together in the pair loop: 2, 4 or 8 */
+    int32_t nbr_batch;       /* W entries each thread loads together in the pair loop: 2, 4 or 8.
+                                With step_kernel 1, ctas_per_sm 8 and nbr_batch 2 together, the
+                                values at creation, leave both to the library: by the number of
+                                atoms and their neighbours it runs a warp per 32 atoms, 4 CTAs
+                                with 8 entries or 8 with 2 (the same results) */
     int32_t build_batch;     /* neighbour build: 1, 2, 4 or 32 are accepted and select the same
                                 kernel (units of 10 atoms per warp, a lane per atom and z plane of
                                 cells); the columns of W are in the order rows of cells, cells,

@@ -270,7 +270,6 @@ struct md_system {
     int64_t host_step = 0;
     bool binned_fresh = false;
     md_tuning tune;
-    bool shape_set = false;       // md_set_tuning has named ctas_per_sm or nbr_batch
     void* ws = nullptr;
     size_t ws_bytes = 0;
     // per-phase timers (CUDA events on the system's stream) and kernel-launch counts
@@ -447,6 +446,8 @@ void fill_scal(md_system* s)
     S.ucf = float(uc);
 }
 
+constexpr int AUTO_CTAS = 8, AUTO_BATCH = 2;
+
 int apply_tuning(md_system* s)
 {
     const int per_sm = std::max(1, s->tune.ctas_per_sm);
@@ -464,17 +465,18 @@ int apply_tuning(md_system* s)
     bulk_shape(s->S, per_sm, s->smem_per_sm, s->smem_per_cta, &s->L.bulk_rows, &s->L.bulk_smem);
     stage_shape(per_sm, s->smem_per_sm, &s->L.stage_cap, &s->L.stage_smem);
     GBMD_CUDA(build_group_shape(s->S, s->L, s->plan.mean_nbrs, s->plan.dense_nbrs, s->smem_per_cta));
-    // Step-kernel shape.  One that md_set_tuning never named is chosen by size: 4 CTAs per SM with 8
-    // W entries together (120 registers) up to 600k atoms and at 30 neighbours or more, else 8 CTAs
-    // and 2 entries, whose warps hide the HBM latency that the larger fluids wait for.  Step kernel,
-    // 4/8 against 8/2: LJ 256k atoms 59 / 71 us, 1M 176 / 198, 6.9M 1127 / 1158; WCA 108k 25 / 31,
-    // 1M 72 / 74 (density 1.0: 70 / 67), 4M 244 / 206.
+    // Step-kernel shape.  The values at creation (AUTO_CTAS and AUTO_BATCH together) stand for one chosen
+    // by size, so that tuning read, changed elsewhere and written back keeps it, and a caller or tuner
+    // that has named others gets back to it: 4 CTAs per SM with 8 W entries together (120 registers) up
+    // to 600k atoms and at 30 neighbours or more, else 8 CTAs and 2 entries, whose warps hide the HBM
+    // latency that the larger fluids wait for.  Step kernel, 4/8 against 8/2: LJ 256k atoms 59 / 71 us,
+    // 1M 176 / 198, 6.9M 1127 / 1158; WCA 108k 25 / 31, 1M 72 / 74 (density 1.0: 70 / 67), 4M 244 / 206.
     // Up to 40 warp-tiles per SM every warp-tile gets a warp of its own and none claims or steals
     // tiles: up to 16 per SM one warp per CTA in the wide shape, which spreads them over all SMs
     // (4000 LJ atoms 71 -> 11 us), else CTAs of 4 in the 8/2 shape, of which an SM holds 32 (100k WCA
     // atoms 16 us against 22 with claims, 108k LJ 32 against 39, 187k WCA in 64 replicas 27 against
     // 35; at 389k atoms, 80 per SM, the claims' locality wins, 36 against 41).
-    const bool chosen = s->shape_set || s->L.step_kernel != 1;
+    const bool chosen = s->tune.ctas_per_sm != AUTO_CTAS || s->tune.nbr_batch != AUTO_BATCH || s->L.step_kernel != 1;
     const int per_sm_tiles = (s->plan.ntiles * (TILE / 32) + s->nsm - 1) / s->nsm;
     s->L.step_single = (chosen || per_sm_tiles > 40) ? 0 : (per_sm_tiles <= 16 ? 32 : TILE);
     s->L.wide_pairs = s->plan.mean_nbrs >= 30.0 || s->plan.nslots <= 600000;
@@ -760,8 +762,8 @@ int md_create_batch(const md_params* p, int32_t nrep, const int64_t* n_rep, cons
     }
     s->smem_per_sm = int(prop.sharedMemPerMultiprocessor);
     s->smem_per_cta = int(prop.sharedMemPerBlockOptin);
-    s->tune.ctas_per_sm = 8;            // the measured best for the 4M-atom fluid (the tuner searches 4-16)
-    s->tune.nbr_batch = 2;
+    s->tune.ctas_per_sm = AUTO_CTAS;    // (as named, the measured best for the 4M-atom fluid)
+    s->tune.nbr_batch = AUTO_BATCH;
     s->tune.build_batch = 2;
     s->tune.use_graph = 1;
     s->tune.step_kernel = 1;
@@ -1213,7 +1215,6 @@ int md_set_tuning(md_system* s, const md_tuning* t)
     if (t->build_stage < 0 || t->build_stage > 2) return fail(MD_ERR_INVALID_ARG, "build_stage must be 0, 1 or 2");
     if (t->reorder_every < -1) return fail(MD_ERR_INVALID_ARG, "reorder_every must be >= -1");
     const int old_kernel = s->L.step_kernel;
-    if (t->ctas_per_sm || t->nbr_batch) s->shape_set = true;
     if (t->ctas_per_sm) s->tune.ctas_per_sm = t->ctas_per_sm;
     if (t->nbr_batch) s->tune.nbr_batch = t->nbr_batch;
     if (t->build_batch) s->tune.build_batch = t->build_batch;

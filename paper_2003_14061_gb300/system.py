@@ -242,7 +242,8 @@ class MDSystem:
 
     def set_tuning(self, ctas_per_sm: int = 0, nbr_batch: int = 0, build_batch: int = 0, use_graph: int = 0,
                    step_kernel: int = 0, build_stage: int = 0, reorder_every: int = 0):
-        """Launch shapes (0 keeps the current value); use_graph: 1 = CUDA graphs, 2 = direct;
+        """Launch shapes (0 keeps the current value; ctas_per_sm 8 with nbr_batch 2, a new system's, is the
+        shape the library chooses by size); use_graph: 1 = CUDA graphs, 2 = direct;
         step_kernel: 1 = per-thread loads with L2 prefetch, 2 = bulk-copy shared-memory ring,
         3 = staged cell-row windows in shared memory, 4 = list-free (27 cells every step),
         5 = half neighbour list with atomic reactions; build_batch and build_stage select the same

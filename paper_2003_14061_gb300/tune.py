@@ -13,8 +13,10 @@ Search: coordinate descent over (step kernel, ctas_per_sm, nbr_batch) for the st
 per-thread kernel at register-bound residencies, the list-free and half-list kernels, and on
 request the shared-memory ring and the staged-neighbour kernel (2 and 3, slower on every measured
 workload) at the residencies their shared memory allows -- then the accepted build_batch and
-build_stage values (one kernel serves them all), then the reorder policy (every 100 steps or at every rebuild: the paper's
-reorder, Sec. 4.1 item 1, is a trade between the reorder's cost and the locality it restores).
+build_stage values (one kernel serves them all), then the reorder policy (every 100 steps or at
+every rebuild: the paper's reorder, Sec. 4.1 item 1, is a trade between the reorder's cost and the
+locality it restores).  8 CTAs per SM with batches of 2, the values of a new system, stand for the
+shape that the library chooses by size, so that shape is among the candidates and can win.
 
 Measurement: each candidate runs with direct launches and the library's per-phase CUDA events,
 and is scored as (step-phase ms per step) + (rebuild-phase ms per rebuild) x (rebuilds per step
@@ -41,7 +43,7 @@ NBR_BATCH = (2, 4, 8)
 REBUILD_PHASES = ("bin", "build")
 REORDER = (100, -1)            # reorder every 100 steps, or at every rebuild
 BUILD_BATCH = (1, 2, 4, 32)
-BUILD_STAGE = (2, 1)           # the build writes W entry by entry, or rows from shared memory
+BUILD_STAGE = (2, 1)           # accepted values; the build is the same for each
 
 
 def signature(system) -> str:
