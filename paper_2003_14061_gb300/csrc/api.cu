@@ -475,10 +475,12 @@ int apply_tuning(md_system* s)
     // tiles: up to 16 per SM one warp per CTA in the wide shape, which spreads them over all SMs
     // (4000 LJ atoms 71 -> 11 us), else CTAs of 4 in the 8/2 shape, of which an SM holds 32 (100k WCA
     // atoms 16 us against 22 with claims, 108k LJ 32 against 39, 187k WCA in 64 replicas 27 against
-    // 35; at 389k atoms, 80 per SM, the claims' locality wins, 36 against 41).
+    // 35; at 389k atoms, 80 per SM, the claims' locality wins, 36 against 41).  FP64 steps, bound by the
+    // FP64 pipe of each SM, keep to one warp per CTA: 108k atoms are 22.2 warp-tiles per SM, in CTAs of 4
+    // up to 24 on some (110.7 us, 108.5 so).
     const bool chosen = s->tune.ctas_per_sm != AUTO_CTAS || s->tune.nbr_batch != AUTO_BATCH || s->L.step_kernel != 1;
     const int per_sm_tiles = (s->plan.ntiles * (TILE / 32) + s->nsm - 1) / s->nsm;
-    s->L.step_single = (chosen || per_sm_tiles > 40) ? 0 : (per_sm_tiles <= 16 ? 32 : TILE);
+    s->L.step_single = (chosen || per_sm_tiles > 40) ? 0 : (per_sm_tiles <= 16 || s->S.mode == MD_FP64 ? 32 : TILE);
     s->L.wide_pairs = s->plan.mean_nbrs >= 30.0 || s->plan.nslots <= 600000;
     const bool wide = !chosen && (s->L.step_single == 32 || (s->L.step_single == 0 && s->L.wide_pairs));
     const int step_ctas = wide ? 4 : per_sm;

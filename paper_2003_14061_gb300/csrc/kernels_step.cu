@@ -541,44 +541,60 @@ __device__ __forceinline__ void prefetch_l2(const void* p)
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
-// FP64 pairs, NB entries at a time: their W rows, positions and pair terms are independent of each
-// other, the sums are added entry by entry in the column's order.  What is out of range, or pads the
-// column (slot 0), is left out of the sums, not added as zero: its position need not be finite.
+// FP64 pairs m0 .. m0 + NB - 1 of a column: their W rows and positions are loaded together, the sums
+// are added entry by entry in the column's order.  What is out of range, or past the column (slot 0),
+// is skipped, not added as zero: its position need not be finite.
+template <int NB>
+__device__ __forceinline__ void pairs_f64(AccD& a, const Scal& S, const Rep& R, const double4_32a* __restrict__ pos,
+                                          const uint32_t* __restrict__ Wc, double4_32a pi, int m0, int mm)
+{
+    uint32_t e[NB];
+    double4_32a pj[NB];
+#pragma unroll
+    for (int k = 0; k < NB; ++k) e[k] = (m0 + k < mm) ? Wc[int64_t(m0 + k) * S.nslots] : 0u;
+#pragma unroll
+    for (int k = 0; k < NB; ++k) pj[k] = pos[e[k] >> IDX_SHIFT];
+#pragma unroll
+    for (int k = 0; k < NB; ++k) {
+        const double dx = fma(double(int(e[k] & 3u) - 1), R.w[0], pj[k].x - pi.x);
+        const double dy = fma(double(int((e[k] >> 2) & 3u) - 1), R.w[1], pj[k].y - pi.y);
+        const double dz = fma(double(int((e[k] >> 4) & 3u) - 1), R.w[2], pj[k].z - pi.z);
+        const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+        const bool in = m0 + k < mm && r2 < S.rc2d;
+        if (in) {
+            const double ri2 = 1.0 / r2;
+            const double sr2 = S.sig2d * ri2;
+            const double sr6 = sr2 * sr2 * sr2;
+            const double fs = S.eps48d * sr6 * (sr6 - 0.5) * ri2;
+            a.fx -= fs * dx;
+            a.fy -= fs * dy;
+            a.fz -= fs * dz;
+            a.u += S.eps4d * sr6 * (sr6 - 1.0) - S.ucd;
+            a.w += fs * r2;
+        }
+    }
+}
+
+// The column in batches of NB, the rows that are left over in batches of 2 and 1, and the terms behind
+// a branch: the FP64 pipe bounds the pass beyond a few warps per SM and is given neither a padded
+// batch (a longest column of 17 entries is 17 rows, not 20) nor terms out of range.  4M WCA atoms, step
+// and force pass: padded and masked 3455 and 3890 us, so 2976 and 3302; LJ 256k 1110 and 1294, so
+// 1087 and 1263; one row at a time in CTAs of 4 warps, 4M: 3264 and 3475, 2048 atoms 29.5 against 25.5.
 template <int NB>
 __device__ __forceinline__ AccD force_f64(const Arrays& A, const Scal& S, const Rep& R,
                                           const double4_32a* __restrict__ pos, int64_t slot, double4_32a pi)
 {
     AccD a{0.0, 0.0, 0.0, 0.0, 0.0};
     const int mm = min(A.nbr_count[slot], S.cap);
+    const int mx = __reduce_max_sync(__activemask(), mm);
     const uint32_t* __restrict__ Wc = A.W + slot;
-    for (int m0 = 0; m0 < mm; m0 += NB) {
-        uint32_t e[NB];
-        double4_32a pj[NB];
-#pragma unroll
-        for (int k = 0; k < NB; ++k) e[k] = (m0 + k < mm) ? Wc[int64_t(m0 + k) * S.nslots] : 0u;
-#pragma unroll
-        for (int k = 0; k < NB; ++k) pj[k] = pos[e[k] >> IDX_SHIFT];
-#pragma unroll
-        for (int k = 0; k < NB; ++k) {
-            const double dx = fma(double(int(e[k] & 3u) - 1), R.w[0], pj[k].x - pi.x);
-            const double dy = fma(double(int((e[k] >> 2) & 3u) - 1), R.w[1], pj[k].y - pi.y);
-            const double dz = fma(double(int((e[k] >> 4) & 3u) - 1), R.w[2], pj[k].z - pi.z);
-            const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-            const bool in = m0 + k < mm && r2 < S.rc2d;
-            const double ri2 = 1.0 / r2;
-            const double sr2 = S.sig2d * ri2;
-            const double sr6 = sr2 * sr2 * sr2;
-            const double fs = S.eps48d * sr6 * (sr6 - 0.5) * ri2;
-            const double ut = S.eps4d * sr6 * (sr6 - 1.0) - S.ucd;
-            if (in) {
-                a.fx -= fs * dx;
-                a.fy -= fs * dy;
-                a.fz -= fs * dz;
-                a.u += ut;
-                a.w += fs * r2;
-            }
-        }
+    int m0 = 0;
+    for (; m0 + NB <= mx; m0 += NB) pairs_f64<NB>(a, S, R, pos, Wc, pi, m0, mm);
+    if (NB > 2 && m0 + 2 <= mx) {
+        pairs_f64<2>(a, S, R, pos, Wc, pi, m0, mm);
+        m0 += 2;
     }
+    if (m0 < mx) pairs_f64<1>(a, S, R, pos, Wc, pi, m0, mm);
     return a;
 }
 

@@ -64,3 +64,26 @@ def _gas(n, cells):
 def test_rebuild_of_few_atoms_in_many_cells():
     # measured 1.4; 62 while the one tile of the atoms did all 10^6 cells
     assert _rebuild_us(_gas(128, 100)) < 8.0 * _rebuild_us(_gas(128, 10))
+
+
+def test_fp64_forces_of_short_columns_cost_their_rows():
+    # the FP64 pipe bounds the force pass row by row: columns of 3 entries (tetrahedra) must cost more
+    # than columns of 1 (pairs), which they would not if both were padded to batches of 4
+    tetra = 1.1 / np.sqrt(8.0) * np.array([[1, 1, 1], [1, -1, -1], [-1, 1, -1], [-1, -1, 1]])
+    us = []
+    for size, m in ((2, 63), (4, 50)):
+        g = (np.stack(np.meshgrid(*[np.arange(m)] * 3, indexing="ij"), -1).reshape(-1, 1, 3) + 0.5) * 4.0
+        x = (g + tetra[:size]).reshape(-1, 3)
+        s = MDSystem(x, np.zeros_like(x), np.array([4.0 * m] * 3), skin=0.2, precision="fp64")
+        assert s.props()[0]["max_nbrs"] == size - 1
+        best = 1e30
+        for _ in range(6):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            s.compute_forces()
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b) * 1e3)
+        us.append(best)
+        s.close()
+    assert us[1] > 1.4 * us[0], us
