@@ -481,8 +481,8 @@ int apply_tuning(md_system* s)
     const bool chosen = s->tune.ctas_per_sm != AUTO_CTAS || s->tune.nbr_batch != AUTO_BATCH || s->L.step_kernel != 1;
     const int per_sm_tiles = (s->plan.ntiles * (TILE / 32) + s->nsm - 1) / s->nsm;
     s->L.step_single = (chosen || per_sm_tiles > 40) ? 0 : (per_sm_tiles <= 16 || s->S.mode == MD_FP64 ? 32 : TILE);
-    s->L.wide_pairs = s->plan.mean_nbrs >= 30.0 || s->plan.nslots <= 600000;
-    const bool wide = !chosen && (s->L.step_single == 32 || (s->L.step_single == 0 && s->L.wide_pairs));
+    const bool wide = !chosen && (s->L.step_single == 32 ||
+                                  (s->L.step_single == 0 && (s->plan.mean_nbrs >= 30.0 || s->plan.nslots <= 600000)));
     const int step_ctas = wide ? 4 : per_sm;
     if (wide) s->L.nbr_batch = 8;
     s->L.ctas_req = step_ctas;

@@ -431,7 +431,6 @@ struct Launch {
     int build_block;
     int nbr_batch;            // W entries loaded together per thread in the pair loop (2, 4, 8)
     int ctas_req;             // requested resident CTAs/SM (register bound of the step kernel)
-    int wide_pairs;           // force passes outside the step: 1 = 16 warps per SM with 8 entries, 0 = 32 with 2
     int step_single;          // step kernel 1: threads per CTA when every warp-tile has a warp of its own (0: claims)
     int bg_rows;              // k_build_group: rows of each lane's list in shared memory,
     int bg_block;             // threads per CTA (one CTA per SM), dynamic shared memory,

@@ -2018,17 +2018,19 @@ cudaError_t launch_step(const Arrays& A, const Scal& S, const Launch& L, int cur
     return cudaGetLastError();
 }
 
-// k_forces in the wide shape (16 warps per SM, 8 entries together) for long lists and smaller systems,
-// else with 32 warps and 2 entries (the step kernel's two shapes)
+// k_forces on one CTA per SM: up to 16 warp-tiles each with 8 entries together, beyond with 32 warps and
+// 4 entries (64 registers).  Force pass, 32 warps / 4 entries against 16 / 8: LJ 4000 atoms 21 / 16 us
+// (one warp per SM), 32k 23 / 20, 108k 31 / 36, 864k 155 / 185, 16.4M 2750 / 3180; WCA 32k 13 / 13, 108k
+// 15 / 17, 864k 46 / 55, 4M 176 / 213 (32 / 2: 172); 4096 replicas of 108 atoms 30 / 37.
 template <int MODE, bool CELLS, bool OUT>
 static void run_forces(const Arrays& A, const Scal& S, const Launch& L, int cur, const StateOut& O)
 {
     const int nwt = S.ntiles * (TILE / 32), g = std::max(1, std::min(L.nsm, nwt)), need = (nwt + g - 1) / g;
-    if (L.wide_pairs || CELLS || MODE == MD_FP64) {
+    if (CELLS || MODE == MD_FP64 || need <= 16) {
         constexpr int NB = (MODE == MD_FP64) ? 4 : 8;
         k_forces<MODE, CELLS, OUT, 16, NB><<<g, 32 * std::min(16, need), 0, L.stream>>>(A, S, cur, O);
     } else if constexpr (!CELLS && MODE != MD_FP64) {
-        k_forces<MODE, false, OUT, 32, 2><<<g, 32 * std::min(32, need), 0, L.stream>>>(A, S, cur, O);
+        k_forces<MODE, false, OUT, 32, 4><<<g, 32 * std::min(32, need), 0, L.stream>>>(A, S, cur, O);
     }
 }
 

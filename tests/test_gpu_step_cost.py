@@ -31,6 +31,18 @@ def _step_us(s, steps=60):
     return best
 
 
+def _call_us(f):
+    best = 1e30
+    for _ in range(6):
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        a.record()
+        f()
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b) * 1e3)
+    return best
+
+
 def test_half_list_step_against_the_full_list():
     # measured 1.4 (2M atoms); 2.5 while the force buffers were cleared on top of their loads
     s = _system(80, skin=0.4)
@@ -39,18 +51,6 @@ def test_half_list_step_against_the_full_list():
     s.integrate(20)
     half = _step_us(s)
     assert half < 1.9 * full, (half, full)
-
-
-def _rebuild_us(s):
-    best = 1e30
-    for _ in range(5):
-        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
-        a.record()
-        s.build_neighbours()
-        b.record()
-        torch.cuda.synchronize()
-        best = min(best, a.elapsed_time(b) * 1e3)
-    return best
 
 
 def _gas(n, cells):
@@ -63,7 +63,7 @@ def _gas(n, cells):
 
 def test_rebuild_of_few_atoms_in_many_cells():
     # measured 1.4; 62 while the one tile of the atoms did all 10^6 cells
-    assert _rebuild_us(_gas(128, 100)) < 8.0 * _rebuild_us(_gas(128, 10))
+    assert _call_us(_gas(128, 100).build_neighbours) < 8.0 * _call_us(_gas(128, 10).build_neighbours)
 
 
 def test_fp64_forces_of_short_columns_cost_their_rows():
@@ -76,14 +76,13 @@ def test_fp64_forces_of_short_columns_cost_their_rows():
         x = (g + tetra[:size]).reshape(-1, 3)
         s = MDSystem(x, np.zeros_like(x), np.array([4.0 * m] * 3), skin=0.2, precision="fp64")
         assert s.props()[0]["max_nbrs"] == size - 1
-        best = 1e30
-        for _ in range(6):
-            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
-            a.record()
-            s.compute_forces()
-            b.record()
-            torch.cuda.synchronize()
-            best = min(best, a.elapsed_time(b) * 1e3)
-        us.append(best)
+        us.append(_call_us(s.compute_forces))
         s.close()
     assert us[1] > 1.4 * us[0], us
+
+
+def test_force_pass_against_the_step():
+    # the force pass gathers what the step gathers and moves less besides; it took 1.2 of a step of the
+    # LJ liquid with too few warps per SM
+    s = _system(60, 0.8442, rc=2.5, skin=0.3)
+    assert _call_us(s.compute_forces) < 1.1 * _step_us(s)
