@@ -832,7 +832,7 @@ int md_build_neighbours(md_system* s)
 int md_compute_forces(md_system* s)
 {
     if (!s) return fail(MD_ERR_INVALID_ARG, "system is NULL");
-    Phase t(s, MD_PHASE_OTHER, 1);
+    Phase t(s, MD_PHASE_OTHER, force_kernels(s->S, s->L));
     GBMD_CUDA(launch_forces(s->A, s->S, s->L, s->cur));
     return MD_OK;
 }
@@ -939,7 +939,7 @@ int md_reduce_props(md_system* s, md_props* out)
 {
     if (!s || !out) return fail(MD_ERR_INVALID_ARG, "system or out is NULL");
     {
-        Phase t(s, MD_PHASE_PROPS, 3);
+        Phase t(s, MD_PHASE_PROPS, force_kernels(s->S, s->L) + 2);
         GBMD_CUDA(launch_props(s->A, s->S, s->L, s->cur, true, false));
     }
     GBMD_CUDA(cudaMemcpyAsync(out, s->A.props, sizeof(md_props) * s->plan.nrep, cudaMemcpyDeviceToHost,
@@ -1009,7 +1009,7 @@ int md_get_state(md_system* s, double* x, double* v, double* f)
                 *out[q] = s->A.xchg[q];
                 staged[q] = true;
             }
-        Phase t(s, MD_PHASE_OTHER, 1);
+        Phase t(s, MD_PHASE_OTHER, state_kernels(s->S, s->L, v || f));
         GBMD_CUDA(launch_get_state(s->A, s->S, s->L, s->cur, O));
         if (staged[0]) GBMD_CUDA(cudaMemcpyAsync(x, s->A.xchg[0], bytes, cudaMemcpyDefault, s->L.stream));
         if (staged[1]) GBMD_CUDA(cudaMemcpyAsync(v, s->A.xchg[1], bytes, cudaMemcpyDefault, s->L.stream));
@@ -1166,7 +1166,7 @@ int md_dyn_sample(md_system* s)
         if (P.lag[b] >= 0) s->dyn_counts[size_t(P.lag[b])] += 1;
     }
     {
-        Phase t(s, MD_PHASE_OTHER, 3);
+        Phase t(s, MD_PHASE_OTHER, force_kernels(s->S, s->L) + 2);
         GBMD_CUDA(launch_forces(s->A, s->S, s->L, s->cur));
         GBMD_CUDA(launch_dyn_sample(s->A, s->S, s->L, s->dyn, P, s->cur));
     }

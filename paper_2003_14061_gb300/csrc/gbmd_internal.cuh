@@ -491,6 +491,13 @@ inline int step_kernels(const Scal& S, const Launch& L)
 {
     return (L.step_kernel == 5 ? 2 : 1) + ((S.chain_len && S.mode != MD_FP64) ? 1 : 0);
 }
+// launches of launch_forces: the pairs (half list: and their sums into f) and the chain terms before them
+inline int force_kernels(const Scal& S, const Launch& L) { return step_kernels(S, L); }
+// launches of launch_get_state: one, or the forces into f and a kernel that reads them
+inline int state_kernels(const Scal& S, const Launch& L, bool forces)
+{
+    return 1 + ((forces && (L.step_kernel == 5 || (S.chain_len && S.mode != MD_FP64))) ? force_kernels(S, L) : 0);
+}
 cudaError_t launch_step(const Arrays& A, const Scal& S, const Launch& L, int cur, bool props);
 int step_ctas_per_sm(const Scal& S, const Launch& L);     // resident CTAs/SM of the chosen k_step
 // rows of W and dynamic shared memory of the ring kernel for ctas_per_sm resident CTAs/SM
