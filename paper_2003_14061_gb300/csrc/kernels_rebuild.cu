@@ -681,12 +681,20 @@ constexpr int BG_STEP = 4;                                       // candidates p
 constexpr int BG_TABLE = 12 * 32 * 4;                            // bytes of a warp's table of run starts
 constexpr uint32_t BG_ROW = 32 * 2;                              // bytes of one row of the lists
 
-// append v to the list at shared address w where d < 0
+// append v to the list at shared address w where d < 0.  The appends tell the compiler of no memory, so
+// that loads of candidates can pass them; the lists are read through a pointer it takes to be
+// unrelated, behind lists_fence() (volatile, as the appends are, and so in order with them), and a
+// second one lies between those reads and the next unit's appends.
 __device__ __forceinline__ void list_append(uint32_t& w, float d, uint32_t v)
 {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %1, 0f00000000;\n\t@p st.shared.u16 [%0], %2;\n\t"
                  "@p add.u32 %0, %0, 64;\n\t}"
                  : "+r"(w) : "f"(d), "h"(uint16_t(v)));
+}
+__device__ __forceinline__ void lists_fence()
+{
+    __syncwarp();
+    asm volatile("" ::: "memory");
 }
 // the same where also e != self (NE) or e > self (unsigned)
 template <bool GT>
@@ -930,7 +938,7 @@ __global__ void __launch_bounds__(32 * WARPS, 1) k_build_group(Arrays A, Scal S,
         }
         // join the planes: entry m of atom a comes from plane 0, 1 or 2
         const int cnt = int((L.w - (L.wlim - uint32_t(rows) * BG_ROW) + L.lost) / BG_ROW);
-        __syncwarp();
+        lists_fence();
         const int c0 = __shfl_sync(0xffffffffu, cnt, a), c1 = __shfl_sync(0xffffffffu, cnt, a + BG_ATOMS);
         const int c2 = __shfl_sync(0xffffffffu, cnt, a + 2 * BG_ATOMS);
         int m = c0 + c1 + c2;
@@ -962,7 +970,7 @@ __global__ void __launch_bounds__(32 * WARPS, 1) k_build_group(Arrays A, Scal S,
                 }
             }
         }
-        __syncwarp();
+        lists_fence();
         if (act && pl == 0) {
             A.nbr_count[slot] = m;
             if (S.rule == MD_REBUILD_DISP) {
