@@ -454,8 +454,6 @@ int apply_tuning(md_system* s)
     s->L.grid = std::max(1, s->nsm * per_sm);
     s->L.nsm = std::max(1, s->nsm);
     prime_rebuild_grids(s->S, s->L);
-    s->L.step_block = TILE;
-    s->L.build_block = TILE;
     s->L.nbr_batch = s->tune.nbr_batch;
     s->L.step_kernel = (s->S.mode == MD_FP64) ? 1 : s->tune.step_kernel;
     // the list-free kernel reads each row of cells as a run of slots: atoms reorder at every rebuild
@@ -783,7 +781,9 @@ int md_create_batch(const md_params* p, int32_t nrep, const int64_t* n_rep, cons
         cudaMemcpyAsync(s->A.cell_rep, s->plan.cell_rep.data(), sizeof(int32_t) * s->plan.ncells,
                         cudaMemcpyHostToDevice, s->L.stream) != cudaSuccess)
         return bail(fail(MD_ERR_CUDA, "upload of the replica table"));
-    if (s->plan.nrep == 1 && launch_all_tiles(s->A, s->S, s->L) != cudaSuccess) return bail(fail(MD_ERR_CUDA, "tile list"));
+    if (s->plan.nrep == 1 && cudaMemcpyAsync(&s->A.g->n_rb_tiles, &s->plan.ntiles, sizeof(int32_t), cudaMemcpyHostToDevice,
+                                             s->L.stream) != cudaSuccess)
+        return bail(fail(MD_ERR_CUDA, "number of tiles"));
     rc = load_state(s, x0, v0);
     if (rc) return bail(rc);
     rc = latch_error(s);

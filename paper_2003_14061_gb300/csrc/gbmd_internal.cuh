@@ -102,7 +102,7 @@ struct Global {               // device-wide words
     int32_t any_reorder;      // some rebuilding replica reorders
     int32_t err;              // ErrBits, latched
     int32_t max_nbr_seen;     // largest m_i that overflowed
-    int32_t n_rb_tiles;       // entries of rb_tiles for the rebuild in progress
+    int32_t n_rb_tiles;       // tiles of the rebuild in progress (a batch: entries of rb_tiles)
     int32_t build_done;       // CTAs of the build that have finished
     long long graph_rebuilds; // rebuild sequences that ran inside captured graphs
 };
@@ -427,8 +427,6 @@ struct Launch {
     int grid;                 // persistent CTAs for tile loops
     int nsm;                  // SMs of the device
     int grid_step;            // persistent CTAs of the step kernel (capped at its occupancy)
-    int step_block;
-    int build_block;
     int nbr_batch;            // W entries loaded together per thread in the pair loop (2, 4, 8)
     int ctas_req;             // requested resident CTAs/SM (register bound of the step kernel)
     int step_single;          // step kernel 1: threads per CTA when every warp-tile has a warp of its own (0: claims)
@@ -456,7 +454,6 @@ cudaError_t launch_debug_error(const Arrays& A, const Launch& L, int bits, int n
 
 // rebuild path (kernels_rebuild.cu)
 bool dilute_cells(const std::vector<Rep>& reps);
-cudaError_t launch_all_tiles(const Arrays& A, const Scal& S, const Launch& L);           // creation, one system
 cudaError_t launch_force_rebuild(const Arrays& A, const Scal& S, const Launch& L, int reorder);
 void prime_rebuild_grids(const Scal& S, const Launch& L);
 cudaError_t launch_rebuild(const Arrays& A, const Scal& S, const Launch& L, int cur, bool from_set);

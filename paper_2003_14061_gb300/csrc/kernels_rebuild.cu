@@ -25,27 +25,20 @@
 namespace gbmd {
 
 // ------------------------------------------------------------------------------------------
-// Per-replica statistics (N3: max occupancy; neighbour counts) are accumulated per thread over a
-// CTA's contiguous run of tiles and folded in once per replica: one block reduction and one
-// atomic, instead of an atomic per warp on the same address.  All threads of the CTA call this.
+// The largest occupancy (N3) is kept per thread over a CTA's contiguous run of tiles and folded in once
+// per replica: one block reduction and one atomic, instead of an atomic per warp on the same address.
+// All threads of the CTA call this.
 // ------------------------------------------------------------------------------------------
-__device__ void flush_stats(int64_t* sum_dst, int* max_dst, long long sum, int mx)
+__device__ void flush_max(int* dst, int mx)
 {
-    __shared__ long long sh_sum[TILE / 32];
     __shared__ int sh_max[TILE / 32];
-    sum = warp_sum_ll(sum);
     mx = warp_max_i(mx);
-    if ((threadIdx.x & 31) == 0) {
-        sh_sum[threadIdx.x >> 5] = sum;
-        sh_max[threadIdx.x >> 5] = mx;
-    }
+    if ((threadIdx.x & 31) == 0) sh_max[threadIdx.x >> 5] = mx;
     __syncthreads();
     if (threadIdx.x == 0) {
-        long long tot = 0;
         int m = 0;
-        for (int w = 0; w < TILE / 32; ++w) { tot += sh_sum[w]; m = max(m, sh_max[w]); }
-        if (sum_dst && tot) atomicAdd(reinterpret_cast<unsigned long long*>(sum_dst), static_cast<unsigned long long>(tot));
-        if (max_dst && m > 0) atomicMax(max_dst, m);
+        for (int w = 0; w < TILE / 32; ++w) m = max(m, sh_max[w]);
+        if (m > 0) atomicMax(dst, m);
     }
     __syncthreads();
 }
@@ -122,7 +115,7 @@ __global__ void __launch_bounds__(TILE) k_bin(Arrays A, Scal S, int cur, int fro
         const int t = rebuild_tile(A, S, it);
         const int r = tile_replica(A, S, t);
         if (r != run_r) {
-            if (run_r >= 0) flush_stats(nullptr, &A.rs[run_r].max_occ, 0, run_occ);
+            if (run_r >= 0) flush_max(&A.rs[run_r].max_occ, run_occ);
             run_r = r;
             run_occ = 0;
         }
@@ -258,7 +251,7 @@ __global__ void __launch_bounds__(TILE) k_bin(Arrays A, Scal S, int cur, int fro
         }
         run_occ = max(run_occ, occ);
     }
-    if (run_r >= 0) flush_stats(nullptr, &A.rs[run_r].max_occ, 0, run_occ);
+    if (run_r >= 0) flush_max(&A.rs[run_r].max_occ, run_occ);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -825,7 +818,7 @@ __global__ void __launch_bounds__(32 * WARPS, 1) k_build_group(Arrays A, Scal S,
     extern __shared__ uint32_t s_list[];              // [warps][rows + BG_STEP][32]
     if (!A.g->any_rebuild) return;
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-    // per warp: the table of run starts [BG_RUNS + 3][32], then the lists [rows + BG_STEP][32]
+    // per warp: the table of run starts [12][32], then the lists [rows + BG_STEP][32]
     unsigned char* const mem = reinterpret_cast<unsigned char*>(s_list) + wl * (BG_TABLE + (rows + BG_STEP) * int(BG_ROW));
     int* const my_runs = reinterpret_cast<int*>(mem);
     const uint16_t* const my_lists = reinterpret_cast<const uint16_t*>(mem + BG_TABLE);
@@ -1091,13 +1084,6 @@ __global__ void k_rebuild_finish(Arrays A, Scal S, int in_graph)
     rebuild_finish(A, S, in_graph);
 }
 
-// The tile list of a single system: all its tiles, written once at creation.
-__global__ void k_all_tiles(Arrays A, Scal S)
-{
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < S.ntiles; t += gridDim.x * blockDim.x) A.rb_tiles[t] = t;
-    if (blockIdx.x == 0 && threadIdx.x == 0) A.g->n_rb_tiles = S.ntiles;
-}
-
 // Mark every replica for a rebuild (creation, md_set_state, md_bin_cells).
 __global__ void k_force_rebuild(Arrays A, Scal S, int reorder)
 {
@@ -1154,12 +1140,6 @@ void prime_rebuild_grids(const Scal& S, const Launch& L)
     (void)resident_grid<k_reorder_gather<MD_FP32>>(S, L);
 }
 
-cudaError_t launch_all_tiles(const Arrays& A, const Scal& S, const Launch& L)
-{
-    k_all_tiles<<<std::max(1, std::min(L.nsm, (S.ntiles + 255) / 256)), 256, 0, L.stream>>>(A, S);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_force_rebuild(const Arrays& A, const Scal& S, const Launch& L, int reorder)
 {
     k_force_rebuild<<<1, 256, 0, L.stream>>>(A, S, reorder);
@@ -1170,7 +1150,7 @@ static bool moves_in_order(const Scal& S) { return S.ntiles <= 2048; }
 
 cudaError_t launch_bin_order(const Arrays& A, const Scal& S, const Launch& L, int cur, bool from_set)
 {
-    // a single system's list is all its tiles, written at creation
+    // a single system rebuilds all its tiles, always (rebuild_tile; n_rb_tiles is set at creation)
     if (S.nrep > 1) k_rebuild_list<<<std::min((S.nrep + 31) / 32, L.nsm), 1024, 0, L.stream>>>(A, S);
     const int fs = from_set ? 1 : 0, move = moves_in_order(S) ? 1 : 0;
     if (S.mode == MD_FP64) k_bin<MD_FP64><<<resident_grid<k_bin<MD_FP64>>(S, L), TILE, 0, L.stream>>>(A, S, cur, fs);
