@@ -467,15 +467,18 @@ int apply_tuning(md_system* s)
     // by size, so that tuning read, changed elsewhere and written back keeps it, and a caller or tuner
     // that has named others gets back to it: 4 CTAs per SM with 8 W entries together (120 registers) up
     // to 600k atoms and at 30 neighbours or more, else 8 CTAs and 2 entries, whose warps hide the HBM
-    // latency that the larger fluids wait for.  Step kernel, 4/8 against 8/2: LJ 256k atoms 59 / 71 us,
-    // 1M 176 / 198, 6.9M 1127 / 1158; WCA 108k 25 / 31, 1M 72 / 74 (density 1.0: 70 / 67), 4M 244 / 206.
+    // latency that the larger fluids wait for.  Step kernel, 4/8 against 8/2, us: LJ 256k atoms 59 / 64,
+    // 389k 81 / 96, 864k 154 / 171; WCA 389k 36.5 / 34.7, 500k 42.7 / 42.9, 595k 46.9 / 44.1, 864k 61 / 53,
+    // 4M 244 / 206.
     // Up to 40 warp-tiles per SM every warp-tile gets a warp of its own and none claims or steals
     // tiles: up to 16 per SM one warp per CTA in the wide shape, which spreads them over all SMs
-    // (4000 LJ atoms 71 -> 11 us), else CTAs of 4 in the 8/2 shape, of which an SM holds 32 (100k WCA
-    // atoms 16 us against 22 with claims, 108k LJ 32 against 39, 187k WCA in 64 replicas 27 against
-    // 35; at 389k atoms, 80 per SM, the claims' locality wins, 36 against 41).  FP64 steps, bound by the
-    // FP64 pipe of each SM, keep to one warp per CTA: 108k atoms are 22.2 warp-tiles per SM, in CTAs of 4
-    // up to 24 on some (110.7 us, 108.5 so).
+    // (4000 LJ atoms 71 -> 11 us), else CTAs of 4 in the 8/2 shape, of which an SM holds 32.  One-warp
+    // CTAs / CTAs of 4 / claims in the better shape: 14.5 per SM, WCA 14.3 / 14.6 / 14.3, LJ 22.6 / 27.0 /
+    // 23.1; 18 per SM 18.9 / 16.2 / 16.0, LJ 29.7 / 28.8 / 28.9; 38 per SM 27.6 / 22.7 / 24.8, LJ 50.4 /
+    // 54.6 / 50.9; 42 per SM 28.2 / 23.3 / 26.2, LJ 53.4 / 56.4 / 52.0; 80 per SM 45 / 34.3 / 34.7, LJ 89 /
+    // 93 / 81.  The LJ liquid gains nothing from it beyond 16 per SM, WCA up to 80.  FP64 steps, bound
+    // by the FP64 pipe of each SM, keep to one warp per CTA: 108k atoms are 22.2 warp-tiles per SM, in
+    // CTAs of 4 up to 24 on some (110.7 us, 108.5 so).
     const bool chosen = s->tune.ctas_per_sm != AUTO_CTAS || s->tune.nbr_batch != AUTO_BATCH || s->L.step_kernel != 1;
     const int per_sm_tiles = (s->plan.ntiles * (TILE / 32) + s->nsm - 1) / s->nsm;
     s->L.step_single = (chosen || per_sm_tiles > 40) ? 0 : (per_sm_tiles <= 16 || s->S.mode == MD_FP64 ? 32 : TILE);

@@ -534,7 +534,10 @@ __global__ void __launch_bounds__(TILE) k_order(Arrays A, Scal S, int cur, int m
 // that k_order or k_reorder_gather has filled
 // ------------------------------------------------------------------------------------------
 // Larger systems gather the scratch in a launch of its own: k_order's scattered writes take longer there
-// (4M atoms: 253 us against 52 + 110), and the launch they save is nothing.
+// (4M atoms: 253 us against 52 + 110), and the launch they save is nothing.  New positions to W built,
+// WCA, written by k_order / gathered: 2048 atoms 77 / 83 us, 108k 109 / 110, 256k 151 / 158, 500k 237 /
+// 237, 1M 416 / 397, 4M 1471 / 1344 (LJ 256k 285 / 285, 1M 888 / 866); moves_in_order draws the line at
+// 2048 tiles (262k atoms), within the sizes where the two are level.
 template <int MODE>
 __global__ void __launch_bounds__(TILE) k_reorder_gather(Arrays A, Scal S, int cur)
 {
