@@ -44,7 +44,7 @@ def _call_us(f):
 
 
 def test_half_list_step_against_the_full_list():
-    # measured 1.4 (2M atoms); 2.5 while the force buffers were cleared on top of their loads
+    # measured 1.5 (2M atoms); 2.5 while the force buffers were cleared on top of their loads
     s = _system(80, skin=0.4)
     full = _step_us(s)
     s.set_tuning(step_kernel=5)
